@@ -95,7 +95,10 @@ typedef struct {
   uint64_t order_seed;        /* seed of those restarts                                      */
   int    max_host_absorb_log2;/* size cap of host-side absorption of order<=2 tensors (0: 12)*/
   int    small_max_bits;      /* contractions with <= this many contracted and new legs use the
-                                 streaming small-operand kernel (0: 4; -1: none, all GEMM steps) */
+                                 streaming small-operand kernel (0: 4; -1: none, all GEMM steps).  With 4,
+                                 other steps that are small or narrow run as one direct FP32 kernel
+                                 where that is modelled faster than permute, B preparation and GEMM
+                                 (not the bf16 steps of BF16X3 plans, not SIMT_FP32 plans) */
   int    auto_slice;          /* 0: off.  Otherwise, when no order fits the cap, slice up to this
                                  many more wires (at most 24), chosen on the best over-cap order:
                                  each is the bond carried by the most over-cap intermediates
@@ -377,7 +380,7 @@ int  tn_profile_slices(tn_plan_t* plan, tn_range slice_range, tn_head_t* head, v
                        double* step_ms, int64_t n_entries);
 /* Kind (tn step kind: 0 small-operand, 1 permute, 2 B prep (tensor core),
  * 3 tensor-core GEMM, 4 B prep (SIMT), 5 SIMT GEMM, 6 operand max (FP16x3
- * scaling), -1 accumulation) and the
+ * scaling), -1 accumulation; a direct contraction on the CUDA cores counts as 0) and the
  * algorithmic complex multiply-adds and HBM bytes of launch i of one pass
  * (a slice runs 2^n_internal_sliced passes). */
 int  tn_plan_step_info(const tn_plan_t* plan, int64_t i, int* kind, double* macs, double* bytes);
@@ -414,9 +417,11 @@ int  tn_head_norm_noalloc(const void* head_c128, int64_t n_groups, int n_open, d
  * M, N and K are powers of two (K >= 2 on the tensor-core engines; 16-bit
  * engines take K = 2 in tf32, as the planner does).  mapA / mapB are host
  * arrays of PC pattern indices, or NULL for the identity (P = PC) or pattern 0
- * (P = 1).  The operands pass through the same split permute, B preparation
- * and GEMM kernels as a plan's steps (engine TN_GEMM_*; pair as
- * tn_plan_opts.gemm_pair).  It allocates its
+ * (P = 1).  The operands pass through the same kernels as a plan's steps
+ * (engine TN_GEMM_*): split permute, B preparation and GEMM, or, with pair = 0
+ * and a tensor-core engine, the direct FP32 kernel where it is modelled faster
+ * (small or narrow shapes; not in bf16).  pair = -1: one-CTA GEMM tiles,
+ * pair > 0: the GEMM kernels with CTA pairs where they apply.  It allocates its
  * scratch (split planes, prepared B, tables) with cudaMalloc, frees it before
  * returning, and synchronises `stream`.  TN_ERR_TIMEOUT if a bounded device
  * wait gave up. */

@@ -140,6 +140,7 @@ static int plan_upload(tn_plan_t* p) {
   CUDA_TRY(cudaGetDevice(&p->device));
   CUDA_TRY(tn::prepare_gemm_tc());
   CUDA_TRY(tn::prepare_permute());
+  CUDA_TRY(tn::prepare_direct());
   std::vector<float2> leaves(P.leaf_arena.size());
   for (size_t i = 0; i < leaves.size(); ++i)
     leaves[i] = make_float2((float)P.leaf_arena[i].real(), (float)P.leaf_arena[i].imag());
@@ -432,6 +433,25 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
   cudaError_t e = cudaSuccess;
   switch (x.kind) {
     case tn::ST_SMALL: {
+      if (x.direct) {
+        const tn::Ref &rx = x.dp.swap ? x.b : x.a, &ry = x.dp.swap ? x.a : x.b;
+        tn::DirectParams dp{};
+        tn::direct_fill(x.dp, x.PC, dp);
+        dp.X = ref_ptr(p, rx, s);
+        dp.Y = ref_ptr(p, ry, s);
+        dp.C = buf_ptr(p, x.c);
+        dp.x_pstride = 1LL << (x.dp.swap ? x.rB : x.rA);
+        dp.y_pstride = 1LL << (x.dp.swap ? x.rA : x.rB);
+        dp.c_pstride = 1LL << x.rC;
+        dp.mapX = p->d_meta + (x.dp.swap ? x.mapB_off : x.mapA_off);
+        dp.mapY = p->d_meta + (x.dp.swap ? x.mapA_off : x.mapB_off);
+        dp.mapX_mode = x.dp.swap ? x.mapB_mode : x.mapA_mode;
+        dp.mapY_mode = x.dp.swap ? x.mapA_mode : x.mapB_mode;
+        dp.vec = 1;                      // buffers start on 256 bytes, rows pair up from even ones
+        dp.amax = scale_ptr(p, x.max_slot);
+        e = tn::launch_direct(dp, x.dp.config, st);
+        break;
+      }
       tn::SmallParams sp;
       sp.A = ref_ptr(p, x.a, s);
       sp.B = ref_ptr(p, x.b, s);
@@ -1295,6 +1315,66 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
     }
   }
   cudaStream_t st = (cudaStream_t)stream;
+  // The direct kernel where it is modelled faster than the three launches
+  // below (as the planner chooses; C is row-major, so its rows are N and X is
+  // B).  pair != 0 asks for the GEMM kernels themselves.
+  if (!simt && pair == 0 && !(engine == TN_GEMM_TC_BF16X3 && nk >= 2) && nmk <= 31 && nk + nn <= 31) {
+    int nm = nmk - nk;
+    std::vector<int> xr, xk, yk, yc;
+    for (int j = 0; j < nn; ++j) xr.push_back(j);
+    for (int q = 0; q < nk; ++q) { xk.push_back(nn + q); yk.push_back(q); }
+    for (int j = 0; j < nm; ++j) yc.push_back(nk + j);
+    tn::DirectPlan best;
+    for (int fold = 0; fold < 2; ++fold) {
+      if (fold && (PC == 1 || mode[1] != 1)) continue;
+      tn::DirectShape ds;
+      ds.nr = nn;
+      ds.nk = nk;
+      ds.nc = nm;
+      ds.xr = xr.data();
+      ds.xk = xk.data();
+      ds.yk = yk.data();
+      ds.yc = yc.data();
+      ds.PC = PC;
+      ds.x_shared = mode[1] == 1;
+      ds.x_elems = (double)PB * (double)(K * N);
+      ds.y_elems = (double)PA * (double)(M * K);
+      const tn::DirectPlan d = tn::plan_direct(ds, fold != 0);
+      if (d.seconds < best.seconds) best = d;
+    }
+    if (best.seconds < tn::tc_seconds(nm, nn, nk, PC, mode[0] == 1, (double)PA * (double)(M * K),
+                                      (double)PB * (double)(K * N), (double)PC * (double)(M * N), h16 != 0)) {
+      CUDA_TRY(tn::prepare_direct());
+      uint32_t* d_maps = nullptr;
+      const size_t n_map = maps[0].size() + maps[1].size();
+      if (n_map && cudaMalloc(&d_maps, n_map * sizeof(uint32_t)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(TN_ERR_OOM, "tn_gemm_c64 scratch allocation failed");
+      }
+      maps[0].insert(maps[0].end(), maps[1].begin(), maps[1].end());
+      cudaError_t e = cudaSuccess;
+      if (n_map) e = cudaMemcpyAsync(d_maps, maps[0].data(), n_map * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
+      tn::DirectParams dp{};
+      tn::direct_fill(best, PC, dp);
+      dp.X = (const float2*)B;
+      dp.Y = (const float2*)A;
+      dp.C = (float2*)C;
+      dp.x_pstride = K * N;
+      dp.y_pstride = M * K;
+      dp.c_pstride = M * N;
+      dp.mapX = d_maps + (n_map - maps[1].size());
+      dp.mapY = d_maps;
+      dp.mapX_mode = mode[1];
+      dp.mapY_mode = mode[0];
+      dp.vec = (uintptr_t)C % 16 == 0;
+      dp.amax = nullptr;
+      if (e == cudaSuccess) e = tn::launch_direct(dp, best.config, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      cudaFree(d_maps);
+      if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("tn_gemm_c64: ") + cudaGetErrorString(e));
+      return TN_OK;
+    }
+  }
   CUDA_TRY(tn::prepare_gemm_tc());   // kernel attributes (shared-memory size), as at plan upload
   CUDA_TRY(tn::prepare_permute());
   // scratch: split A planes, prepared B, tables, scale slots

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "direct.h"
+
 namespace tn {
 
 // Operand scaling of the FP16x3 engine.  An ABSMAX step writes m = max over a
@@ -93,6 +95,13 @@ struct GemmTile {
 };
 GemmTile gemm_tc_tile(const GemmParams& p);
 
+// C[p][c][r] = sum_k X[mapX(p)][r, k] Y[mapY(p)][k, c], operands where they lie
+struct DirectParams : DirectParamsBase {
+  const float2* X; const float2* Y; float2* C;
+  const uint32_t* mapX; const uint32_t* mapY;
+  unsigned int* amax;        // non-null: atomicMax of the output's max |re|, |im| (fp32 bits)
+};
+
 struct AccumParams {
   const float2* F; double2* H;
   int64_t f_pstride;
@@ -114,6 +123,8 @@ cudaError_t launch_accum(const AccumParams& p, cudaStream_t s);
 // `status` receives a nonzero code if a bounded wait gave up.
 cudaError_t launch_gemm_tc(const GemmParams& p, unsigned int* status, cudaStream_t s);
 cudaError_t prepare_gemm_tc();   // kernel attributes; call before launching or capturing
+cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s);
+cudaError_t prepare_direct();    // the direct step's opt-in shared-memory sizes; likewise
 cudaError_t prepare_permute();   // the permute's opt-in shared-memory size; likewise
 
 // amplitude lookup: out[i] = H[g][mu] (c128 or c64); status <- min missing

@@ -792,7 +792,7 @@ static int64_t vt_elems(const VTensor& v) { return v.P * (1LL << v.legs.size());
 
 // Pattern maps of C's pattern axis onto an operand's.
 static void set_map(Plan& plan, const VTensor& X, const VTensor& C, int& mode, int64_t& off) {
-  if (X.tq == 0) { mode = 1; off = 0; return; }
+  if (X.tq == 0 || X.P == 1) { mode = 1; off = 0; return; }   // one pattern: every p reads it
   if (X.tq == C.tq) { mode = 0; off = 0; return; }
   const auto& pc = plan.book.get(C.tq);
   const auto& px = plan.book.get(X.tq);
@@ -919,6 +919,30 @@ static void add_permute(Plan& plan, const VTensor& X, const std::vector<int>& ta
   plan.steps.push_back(s);
 }
 
+// Modelled time of a contraction as split permute, B preparation and
+// tensor-core GEMM, to set against the direct form's (plan_direct).  Measured
+// on GB300: about 4 us per launch; the passes stream at 5 TB/s and a
+// GEMM writes C at 2.4 TB/s; it runs
+// its tiles of 128 rows x BN real columns in whole waves of 152, each SM at
+// its share of 280 (3xTF32) or 560 (16-bit) TFLOP/s for BN >= 256, where an
+// MMA narrower than 128 columns takes as long as one of 128.
+double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, double a, double b, double c, bool h16) {
+  int64_t cols = 2LL << nn, groups = PC;
+  if (a_shared && cols >= 16)
+    while (cols < 256 && groups > 1) {
+      cols *= 2;
+      groups = (groups + 1) / 2;
+    }
+  const double bn = (double)std::min<int64_t>(256, std::max<int64_t>(cols, 16));
+  const double tiles = (double)groups * std::ceil((double)cols / bn) * std::ceil(std::ldexp(1.0, nm) / 128.0);
+  const double peak = h16 ? 560e12 : 280e12;
+  const double tile_flops = 8.0 * 128.0 * std::max(bn, 128.0) / 2.0 * std::ldexp(1.0, nk);
+  const double mma = std::ceil(tiles / 152.0) * tile_flops * 152.0 / peak;
+  const double plane = h16 ? 8.0 : 16.0;
+  const double gemm = std::max(mma, plane * a / 5.0e12 + 8.0 * c / 2.4e12);
+  return gemm + (8.0 + plane) * a / 5.0e12 + (8.0 + 2.0 * plane) * b / 5.0e12 + 12e-6;
+}
+
 static int layout_steps(Plan& plan, std::string& err) {
   plan.steps.clear();
   plan.bufs.clear();
@@ -975,7 +999,46 @@ static int layout_steps(Plan& plan, std::string& err) {
     C.legs.clear();
     std::vector<int> cl;
     const bool use_small = nk <= plan.small_max_bits && nn <= plan.small_max_bits;
-    if (use_small) {
+    set_map(plan, big, C, mapA_mode, mapA_off);
+    set_map(plan, sml, C, mapB_mode, mapB_off);
+    // The direct form (see direct.cu): either operand may have the rows, and
+    // patterns fold into the columns where they share that operand; the
+    // cheapest of those forms is taken where its modelled time is below the
+    // three-launch GEMM's.  Limited to plans whose streaming steps have their
+    // full range, and to operands whose offsets fit 32 bits.  A BF16x3 plan
+    // keeps the GEMM for every step that runs in bf16: FP32 in some of them
+    // moves its amplitudes by as much as that engine's own error (2e-5).
+    DirectPlan dp;
+    const bool h16_step = nk >= 2 && (plan.gemm_engine == TN_GEMM_TC_BF16X3 || plan.gemm_engine == TN_GEMM_TC_FP16X3);
+    if (!use_small && !(h16_step && plan.gemm_engine == TN_GEMM_TC_BF16X3) && plan.small_max_bits >= 4 && plan.gemm_engine != TN_GEMM_SIMT_FP32 && nm <= 31 &&
+        big.legs.size() <= 31) {
+      std::vector<int> mp, kp, ks, np;
+      for (int l : M) mp.push_back(find_pos(big.legs, l));
+      for (int l : K) { kp.push_back(find_pos(big.legs, l)); ks.push_back(find_pos(sml.legs, l)); }
+      for (int l : N) np.push_back(find_pos(sml.legs, l));
+      for (int form = 0; form < 4; ++form) {
+        const bool swap = (form & 1) != 0, fold = (form & 2) != 0;
+        if (fold && (C.P == 1 || (swap ? mapB_mode : mapA_mode) != 1)) continue;
+        DirectShape ds;
+        ds.nr = swap ? nn : nm;
+        ds.nk = nk;
+        ds.nc = swap ? nm : nn;
+        ds.xr = swap ? np.data() : mp.data();
+        ds.xk = swap ? ks.data() : kp.data();
+        ds.yk = swap ? kp.data() : ks.data();
+        ds.yc = swap ? mp.data() : np.data();
+        ds.PC = C.P;
+        ds.x_shared = (swap ? mapB_mode : mapA_mode) == 1;
+        ds.x_elems = (double)vt_elems(swap ? sml : big);
+        ds.y_elems = (double)vt_elems(swap ? big : sml);
+        DirectPlan d = plan_direct(ds, fold);
+        d.swap = swap;
+        if (d.seconds < dp.seconds) dp = d;
+      }
+    }
+    const bool direct = dp.seconds < tc_seconds(nm, nn, nk, C.P, mapA_mode == 1, (double)vt_elems(big),
+                                                (double)vt_elems(sml), (double)C.P * std::exp2(nm + nn), h16_step);
+    if (use_small || (direct && !dp.swap)) {
       for (int l : M) cl.push_back(l);
       for (int l : N) cl.push_back(l);
     } else {
@@ -989,8 +1052,6 @@ static int layout_steps(Plan& plan, std::string& err) {
       return TN_ERR_OOM;
     }
     plan.max_log2 = std::max(plan.max_log2, lc);
-    set_map(plan, big, C, mapA_mode, mapA_off);
-    set_map(plan, sml, C, mapB_mode, mapB_off);
     const int64_t eC = vt_elems(C);
     const double macs = (double)C.P * std::exp2((double)(nm + nn + nk));
     plan.tc_macs += macs;
@@ -1010,7 +1071,7 @@ static int layout_steps(Plan& plan, std::string& err) {
       bn[n] = o;
     }
 
-    if (use_small) {
+    if (use_small || direct) {
       Step s;
       s.kind = ST_SMALL;
       s.contraction = ci;
@@ -1023,9 +1084,14 @@ static int layout_steps(Plan& plan, std::string& err) {
       s.nk = nk; s.nm = nm; s.nn = nn;
       s.mapA_mode = mapA_mode; s.mapA_off = mapA_off;
       s.mapB_mode = mapB_mode; s.mapB_off = mapB_off;
-      for (int q = 0; q < nk; ++q) s.kposA[q] = find_pos(big.legs, K[q]);
-      for (size_t k = 0; k < bk.size(); ++k) s.boffK[k] = bk[k];
-      for (size_t n = 0; n < bn.size(); ++n) s.boffN[n] = bn[n];
+      if (direct) {
+        s.direct = true;
+        s.dp = dp;
+      } else {
+        for (int q = 0; q < nk; ++q) s.kposA[q] = find_pos(big.legs, K[q]);
+        for (size_t k = 0; k < bk.size(); ++k) s.boffK[k] = bk[k];
+        for (size_t n = 0; n < bn.size(); ++n) s.boffN[n] = bn[n];
+      }
       s.macs = macs;
       s.bytes = 8.0 * (double)(vt_elems(big) + vt_elems(sml) + eC);
       const int st = (int)plan.steps.size();
@@ -1607,7 +1673,30 @@ std::string describe_plan(const Plan& plan, bool with_data) {
     for (int v = 0; v < 16; ++v) o << (v ? "," : "") << st.boffN[v];
     o << "],\"mapA\":[" << st.mapA_mode << "," << st.mapA_off << "],\"mapB\":[" << st.mapB_mode << ","
       << st.mapB_off << "],\"bk_off\":" << st.bk_off << ",\"bn_off\":" << st.bn_off << ",\"bprep_embed0\":" << st.bprep_embed0 << ",\"variant\":" << st.variant
-      << ",\"tile_cap\":" << st.tile_cap << ",\"pair\":" << st.pair << ",\"alts\":[";
+      << ",\"direct\":" << (st.direct ? 1 : 0);
+    if (st.direct) {
+      const DirectPlan& d = st.dp;
+      auto list = [&o](const char* name, const uint8_t* v, int n) {
+        o << ",\"" << name << "\":[";
+        for (int i = 0; i < n; ++i) o << (i ? "," : "") << (int)v[i];
+        o << "]";
+      };
+      const DirectConfig& g = kDirectConfigs[d.config];
+      const int trb = std::min(d.nr, g.tr), tkb = std::min(d.nk, g.tk), tcb = std::min(d.nc, g.tc);
+      o << ",\"dp\":{\"tile\":[" << g.tr << "," << g.tc << "," << g.tk << "],\"swap\":" << (int)d.swap << ",\"fold\":"
+        << (int)d.fold << ",\"cluster\":" << d.cluster << ",\"nr\":" << d.nr << ",\"nk\":" << d.nk << ",\"nc\":" << d.nc
+        << ",\"cols\":" << d.cols << ",\"col_tiles\":" << d.col_tiles;
+      list("rrest", d.rrest, d.n_rrest);
+      list("crest", d.crest, d.n_crest);
+      list("kxrest", d.kxrest, d.nk - tkb);
+      list("kyrest", d.kyrest, d.nk - tkb);
+      list("xpos", d.xpos, trb + tkb);
+      list("xleg", d.xleg, trb + tkb);
+      list("ypos", d.ypos, tcb + tkb);
+      list("yleg", d.yleg, tcb + tkb);
+      o << "}";
+    }
+    o << ",\"tile_cap\":" << st.tile_cap << ",\"pair\":" << st.pair << ",\"alts\":[";
     for (size_t a = 0; a < st.alts.size(); ++a) {
       const PermSched& ps = st.alts[a];
       o << (a ? "," : "") << "{\"t_bits\":" << ps.t_bits << ",\"vec4\":" << ps.vec4 << ",\"tab_off\":" << ps.tab_off << ",\"n_rest\":" << ps.n_rest

@@ -14,6 +14,8 @@
 #include <unordered_map>
 #include <vector>
 
+#include "direct.h"
+
 namespace tn {
 
 using cd = std::complex<double>;
@@ -48,7 +50,8 @@ struct PatternBook {
 };
 
 enum StepKind {
-  ST_SMALL = 0,      // streaming contraction with a <=16x16 operand, any A layout
+  ST_SMALL = 0,      // contraction on the operands where they lie: with a <=16x16 operand (k_small), or
+                     // a direct one (Step::direct, k_direct)
   ST_PERMUTE = 1,    // bit permutation of a tensor's legs
   ST_BPREP_TC = 2,   // B -> real-embedded K-major fp32 hi/lo operand (tensor-core GEMM)
   ST_GEMM_TC = 3,    // tcgen05 complex GEMM (4M real embedding, 3xTF32)
@@ -97,6 +100,9 @@ struct Step {
   // SMALL
   int kposA[4] = {0, 0, 0, 0};
   uint32_t boffK[16] = {0}, boffN[16] = {0};
+  // SMALL in the direct form (direct.cu): small or narrow contractions of any K
+  bool direct = false;
+  DirectPlan dp;
   // PERMUTE: tile bits t; tables in meta: in_off[2^t], out_off[2^t], slot[2^t]
   int t_bits = 0;
   int split = 0;           // PERMUTE: 1 tf32 hi/lo planes, 2 bf16, 3 scaled fp16 (tensor-core GEMM operand)
@@ -215,6 +221,9 @@ struct PlanInput {
   bool side_bprep = false;  // B-prep steps whose operand is ready run beside the previous GEMM
 };
 
+// Modelled time of a contraction as split permute, B preparation and
+// tensor-core GEMM (a, b, c: elements of the operands and the result).
+double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, double a, double b, double c, bool h16);
 int build_plan(const PlanInput& in, Plan& plan, std::string& err);
 void apply_perm_schedule(Step& s, const PermSched& ps);
 std::string describe_plan(const Plan& plan, bool with_data);
