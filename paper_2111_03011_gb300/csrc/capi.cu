@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -30,15 +31,6 @@ int fail(int code, const std::string& msg) {
     cudaError_t e_ = (x);                                                                    \
     if (e_ != cudaSuccess) return fail(TN_ERR_CUDA, std::string(#x) + ": " + cudaGetErrorString(e_)); \
   } while (0)
-
-bool is_device_ptr(const void* p) {
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
-}
 
 // NVTX range around a scope: a profiler (nsys, or ncu with --nvtx) sees each
 // pass and each step's launch by name; without a tool attached the calls do
@@ -350,9 +342,7 @@ extern "C" int tn_head_create(tn_plan_t* plan, void* dev_c128, tn_head_t** out) 
   cudaError_t e1 = cudaMemset(h->H, 0, (size_t)elems * sizeof(double2));
   if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(0);   // zeroed before any stream, blocking or not, uses it
   cudaError_t e2 = cudaMalloc(&h->d_Z, (size_t)std::max<int64_t>(L, 1) * sizeof(double));
-  cudaError_t e3 = cudaMalloc(&h->d_N, sizeof(double));
-  cudaError_t e4 = cudaMalloc(&h->d_status, sizeof(unsigned long long));
-  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess) {
+  if (e1 != cudaSuccess || e2 != cudaSuccess) {
     cudaGetLastError();
     tn_head_free(h);
     return fail(TN_ERR_CUDA, "head set-up failed");
@@ -365,8 +355,6 @@ extern "C" void tn_head_free(tn_head_t* h) {
   if (!h) return;
   if (h->owns) cudaFree(h->H);
   cudaFree(h->d_Z);
-  cudaFree(h->d_N);
-  cudaFree(h->d_status);
   cudaFree(h->d_stage);
   delete h;
 }
@@ -1098,6 +1086,113 @@ static int ensure_stage(tn_head* h, size_t bytes) {
   return TN_OK;
 }
 
+// Per-call scratch of the head operations: a report in mapped host memory and
+// the partial sums of a reduction on the device, plus a device buffer that
+// grows on demand (the sampler's prefix sums).  Each call takes one for its
+// duration, so calls on one head from several threads and streams do not share
+// any.  At most kMost of them stay between calls, and one whose
+// buffer grew past kKeepBytes gives it back.
+struct CallScratch {
+  tn::HeadReport* rep = nullptr;
+  double* part = nullptr;
+  void* buf = nullptr;
+  size_t bytes = 0;
+  int device = -1;
+};
+
+static std::mutex g_scratch_mu;
+static std::vector<CallScratch> g_scratch;
+
+static void free_scratch(CallScratch& c) {
+  cudaFreeHost(c.rep);
+  cudaFree(c.part);
+  cudaFree(c.buf);
+  c = CallScratch();
+}
+
+struct ScratchLease {
+  static constexpr size_t kMost = 32, kKeepBytes = (size_t)64 << 20;
+  CallScratch c;
+  cudaStream_t stream;
+  bool in_flight = false;
+  explicit ScratchLease(cudaStream_t st) : stream(st) {}
+  ScratchLease(const ScratchLease&) = delete;
+  ScratchLease& operator=(const ScratchLease&) = delete;
+  ~ScratchLease() {
+    if (!c.rep) return;
+    if (in_flight) cudaStreamSynchronize(stream);   // the call failed after a launch
+    if (c.bytes > kKeepBytes) {
+      cudaFree(c.buf);
+      c.buf = nullptr;
+      c.bytes = 0;
+    }
+    {
+      std::lock_guard<std::mutex> lock(g_scratch_mu);
+      if (g_scratch.size() < kMost) {
+        g_scratch.push_back(c);
+        return;
+      }
+    }
+    free_scratch(c);
+  }
+  // The report, once the stream is synchronised.
+  tn::HeadReport done() {
+    in_flight = false;
+    return *c.rep;
+  }
+  // Call before the launches; the report starts as "nothing missing, no status".
+  int take(size_t bytes) {
+    int dev = -1;
+    CUDA_TRY(cudaGetDevice(&dev));
+    {
+      std::lock_guard<std::mutex> lock(g_scratch_mu);
+      g_scratch.reserve(kMost);
+      for (size_t i = g_scratch.size(); i-- > 0;)
+        if (g_scratch[i].device == dev) {
+          c = g_scratch[i];
+          g_scratch.erase(g_scratch.begin() + (std::ptrdiff_t)i);
+          break;
+        }
+    }
+    if (!c.rep) {
+      c.device = dev;
+      void* h = nullptr;
+      if (cudaHostAlloc(&h, sizeof(tn::HeadReport), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
+          cudaMalloc(&c.part, 2 * tn::kHeadParts * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        if (h) cudaFreeHost(h);
+        return fail(TN_ERR_OOM, "scratch allocation failed");
+      }
+      c.rep = (tn::HeadReport*)h;   // one address on host and device (unified addressing)
+    }
+    if (c.bytes < bytes) {
+      cudaFree(c.buf);
+      c.buf = nullptr;
+      c.bytes = 0;
+      if (cudaMalloc(&c.buf, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(TN_ERR_OOM, "scratch allocation failed");
+      }
+      c.bytes = bytes;
+    }
+    *c.rep = tn::HeadReport{~0ULL, 0u, {0.0, 0.0}};
+    in_flight = true;
+    return TN_OK;
+  }
+};
+
+// A pointer that kernels can use as it is: device or managed memory, or pinned
+// host memory, which GB300 reads and writes over NVLink-C2C without a copy.
+static bool kernel_ptr(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged ||
+         (a.type == cudaMemoryTypeHost && a.devicePointer == p);
+}
+
 extern "C" int tn_amplitudes(tn_head_t* h, const uint64_t* bitstrings, int64_t n, void* out, int dtype, void* stream) {
   if (!h || (n > 0 && (!bitstrings || !out))) return fail(TN_ERR_INVALID, "NULL argument");
   if (n < 0) return fail(TN_ERR_INVALID, "n < 0");
@@ -1107,7 +1202,7 @@ extern "C" int tn_amplitudes(tn_head_t* h, const uint64_t* bitstrings, int64_t n
   tn_plan_t* p = h->plan;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t esz = dtype == TN_C128 ? 16 : 8;
-  const bool dev_in = is_device_ptr(bitstrings), dev_out = is_device_ptr(out);
+  const bool dev_in = kernel_ptr(bitstrings), dev_out = kernel_ptr(out);
   size_t need = 0;
   if (!dev_in) need += (size_t)n * 8;
   size_t out_off = (need + 255) / 256 * 256;
@@ -1116,26 +1211,23 @@ extern "C" int tn_amplitudes(tn_head_t* h, const uint64_t* bitstrings, int64_t n
     int rc = ensure_stage(h, need);
     if (rc) return rc;
   }
+  ScratchLease lease(st);
+  if (int rc = lease.take(0)) return rc;
   const uint64_t* d_bits = bitstrings;
   if (!dev_in) {
     CUDA_TRY(cudaMemcpyAsync(h->d_stage, bitstrings, (size_t)n * 8, cudaMemcpyHostToDevice, st));
     d_bits = (const uint64_t*)h->d_stage;
   }
   void* d_out = dev_out ? out : (void*)((char*)h->d_stage + out_off);
-  unsigned long long init = ~0ULL;
-  CUDA_TRY(cudaMemcpyAsync(h->d_status, &init, sizeof(init), cudaMemcpyHostToDevice, st));
   CUDA_TRY(tn::launch_amplitudes(h->H, (int)p->P.open_qubits.size(), p->d_keys, p->d_key_groups, p->n_keys,
-                                 p->P.tail_mask, p->d_open, d_bits, n, d_out, dtype == TN_C128 ? 1 : 0, h->d_status,
-                                 st));
-  unsigned long long status = 0;
-  CUDA_TRY(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, st));
+                                 p->P.tail_mask, p->d_open, d_bits, n, d_out, dtype == TN_C128 ? 1 : 0,
+                                 &lease.c.rep->missing, st, nullptr, 1, lease.c.rep, p->d_status));
   if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, d_out, (size_t)n * esz, cudaMemcpyDeviceToHost, st));
-  unsigned int word = 0;
-  CUDA_TRY(cudaMemcpyAsync(&word, p->d_status, sizeof(word), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
-  if (int rc = tn::report_status(h, word, st)) return rc;
-  if (status != ~0ULL)
-    return fail(TN_ERR_NOT_IN_STATE, "bitstring " + std::to_string(status) + " has a tail that is not a group");
+  const tn::HeadReport rep = lease.done();
+  if (int rc = tn::report_status(h, rep.word, st)) return rc;
+  if (rep.missing != ~0ULL)
+    return fail(TN_ERR_NOT_IN_STATE, "bitstring " + std::to_string(rep.missing) + " has a tail that is not a group");
   return TN_OK;
 }
 
@@ -1146,36 +1238,23 @@ extern "C" int tn_xeb(tn_head_t* h, const uint64_t* samples, int64_t n, double* 
   if (h->invalid) return fail(TN_ERR_INVALID, "head is invalid after a failed or timed-out contraction");
   tn_plan_t* p = h->plan;
   cudaStream_t st = (cudaStream_t)stream;
-  const bool dev_in = is_device_ptr(samples);
-  // stage: [samples (host input)] [amplitudes c128] [partials] [2 sums]
-  const size_t in_b = dev_in ? 0 : (size_t)n * 8;
-  const size_t amp_off = (in_b + 255) / 256 * 256;
-  const size_t part_off = amp_off + (size_t)n * 16;
-  const size_t sums_off = part_off + (size_t)tn::xeb_partials(n) * 8;
-  int rc = ensure_stage(h, sums_off + 16);
-  if (rc) return rc;
-  char* stg = (char*)h->d_stage;
   const uint64_t* d_bits = samples;
-  if (!dev_in) {
-    CUDA_TRY(cudaMemcpyAsync(stg, samples, in_b, cudaMemcpyHostToDevice, st));
-    d_bits = (const uint64_t*)stg;
+  if (!kernel_ptr(samples)) {
+    if (int rc = ensure_stage(h, (size_t)n * 8)) return rc;
+    CUDA_TRY(cudaMemcpyAsync(h->d_stage, samples, (size_t)n * 8, cudaMemcpyHostToDevice, st));
+    d_bits = (const uint64_t*)h->d_stage;
   }
-  unsigned long long init = ~0ULL;
-  CUDA_TRY(cudaMemcpyAsync(h->d_status, &init, sizeof(init), cudaMemcpyHostToDevice, st));
-  CUDA_TRY(tn::launch_amplitudes(h->H, (int)p->P.open_qubits.size(), p->d_keys, p->d_key_groups, p->n_keys,
-                                 p->P.tail_mask, p->d_open, d_bits, n, stg + amp_off, 1, h->d_status, st));
-  CUDA_TRY(tn::launch_xeb_sums((const double2*)(stg + amp_off), n, (double*)(stg + part_off),
-                               (double*)(stg + sums_off), st));
-  double sums[2] = {0.0, 0.0};
-  unsigned long long status = 0;
-  CUDA_TRY(cudaMemcpyAsync(sums, stg + sums_off, 16, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, st));
+  ScratchLease lease(st);
+  if (int rc = lease.take(0)) return rc;
+  CUDA_TRY(tn::launch_xeb(h->H, (int)p->P.open_qubits.size(), p->d_keys, p->d_key_groups, p->n_keys, p->P.tail_mask,
+                          p->d_open, d_bits, n, lease.c.part, lease.c.rep, st));
   CUDA_TRY(cudaStreamSynchronize(st));
-  if (status != ~0ULL)
-    return fail(TN_ERR_NOT_IN_STATE, "sample " + std::to_string(status) + " has a tail that is not a group");
+  const tn::HeadReport rep = lease.done();
+  if (rep.missing != ~0ULL)
+    return fail(TN_ERR_NOT_IN_STATE, "sample " + std::to_string(rep.missing) + " has a tail that is not a group");
   const int nq = p->P.n_qubits;
-  if (linear) *linear = std::ldexp(sums[0] / (double)n, nq) - 1.0;
-  if (log_xeb) *log_xeb = nq * std::log(2.0) + 0.57721566490153286 + sums[1] / (double)n;
+  if (linear) *linear = std::ldexp(rep.sum[0] / (double)n, nq) - 1.0;
+  if (log_xeb) *log_xeb = nq * std::log(2.0) + 0.57721566490153286 + rep.sum[1] / (double)n;
   return TN_OK;
 }
 
@@ -1185,13 +1264,15 @@ extern "C" int tn_head_norm(tn_head_t* h, double* norm, double* group_norms, voi
   tn_plan_t* p = h->plan;
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t L = (int64_t)p->P.tails_raw.size();
-  CUDA_TRY(tn::launch_group_norms(h->H, L, (int)p->P.open_qubits.size(), h->d_Z, h->d_N, st));
-  if (norm) CUDA_TRY(cudaMemcpyAsync(norm, h->d_N, sizeof(double), cudaMemcpyDeviceToHost, st));
+  ScratchLease lease(st);
+  if (int rc = lease.take(0)) return rc;
+  CUDA_TRY(tn::launch_group_norms(h->H, L, (int)p->P.open_qubits.size(), h->d_Z, nullptr, lease.c.part, st,
+                                  lease.c.rep, p->d_status));
   if (group_norms) CUDA_TRY(cudaMemcpyAsync(group_norms, h->d_Z, (size_t)L * sizeof(double), cudaMemcpyDeviceToHost, st));
-  unsigned int word = 0;
-  CUDA_TRY(cudaMemcpyAsync(&word, p->d_status, sizeof(word), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
-  return tn::report_status(h, word, st);
+  const tn::HeadReport rep = lease.done();
+  if (norm) *norm = rep.sum[0];
+  return tn::report_status(h, rep.word, st);
 }
 
 static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t seed, int method, int64_t param,
@@ -1227,13 +1308,17 @@ static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t
   double mix = 0.0;
   if (target_fidelity > 0.0 && f_head > 0.0 && target_fidelity < f_head) mix = 1.0 - target_fidelity / f_head;
   cudaStream_t st = (cudaStream_t)stream;
-  const bool dev_out = is_device_ptr(out);
+  const bool dev_out = kernel_ptr(out);
   uint64_t* d_out = out;
   if (!dev_out) {
     int rc = ensure_stage(h, (size_t)n * 8);
     if (rc) return rc;
     d_out = (uint64_t*)h->d_stage;
   }
+  ScratchLease lease(st);
+  if (int rc = lease.take(8 * tn::sample_scratch_doubles((int64_t)p->P.tails_raw.size(),
+                                                         (int)p->P.open_qubits.size(), n, method)))
+    return rc;
   tn::SampleParams sp;
   sp.H = h->H;
   sp.L = (int64_t)p->P.tails_raw.size();
@@ -1248,12 +1333,13 @@ static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t
   sp.out = d_out;
   sp.method = method;
   sp.param = param;
+  sp.carry = (double*)lease.c.buf;
+  sp.rep = lease.c.rep;
+  sp.plan_status = p->d_status;
   CUDA_TRY(tn::launch_sample(sp, st));
   if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, d_out, (size_t)n * 8, cudaMemcpyDeviceToHost, st));
-  unsigned int word = 0;
-  CUDA_TRY(cudaMemcpyAsync(&word, p->d_status, sizeof(word), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
-  return tn::report_status(h, word, st);
+  return tn::report_status(h, lease.done().word, st);
 }
 
 namespace tn {

@@ -71,8 +71,6 @@ struct tn_head {
   double f_value = 0.0;
   // scratch
   double* d_Z = nullptr;
-  double* d_N = nullptr;
-  unsigned long long* d_status = nullptr;
   void* d_stage = nullptr;
   size_t stage_bytes = 0;
 };

@@ -1,6 +1,5 @@
 // Streaming kernels of the contraction path (HBM-bound steps), the plain
-// FP32 CUDA-core complex GEMM, slice accumulation, amplitude lookup, norms and
-// the group sampler.
+// FP32 CUDA-core complex GEMM and slice accumulation.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -605,275 +604,6 @@ cudaError_t launch_accum(const AccumParams& p, cudaStream_t s) {
   const int64_t total = p.L << p.h;
   const int64_t grid = std::min<int64_t>((total + 255) / 256, (int64_t)kSMs * 8);
   k_accum<<<(unsigned)std::max<int64_t>(grid, 1), 256, 0, s>>>(p);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------- K7
-// With seg_end (n_seg cumulative ends of merged requests), a missing key i of
-// segment j records its index within the segment in status[j]; otherwise
-// status[0] receives the smallest missing index.
-__global__ void k_amplitudes(const double2* __restrict__ H, int h, const uint64_t* __restrict__ keys,
-                             const uint32_t* __restrict__ groups, int64_t n_keys, uint64_t tail_mask,
-                             const int* __restrict__ open_q, const uint64_t* __restrict__ bits, int64_t n, void* out,
-                             int dtype, unsigned long long* status, const int64_t* __restrict__ seg_end, int n_seg) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t b = bits[i];
-    const uint64_t key = b & tail_mask;
-    int64_t lo = 0, hi = n_keys;
-    while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (keys[mid] < key) lo = mid + 1; else hi = mid;
-    }
-    double2 v = make_double2(0.0, 0.0);
-    if (lo < n_keys && keys[lo] == key) {
-      const int64_t g = groups[lo];
-      int64_t mu = 0;
-      for (int j = 0; j < h; ++j) mu |= (int64_t)((b >> open_q[j]) & 1ULL) << j;
-      v = H[(g << h) + mu];
-    } else if (seg_end) {
-      int j = 0;
-      while (j < n_seg - 1 && i >= seg_end[j]) ++j;
-      atomicMin(status + j, (unsigned long long)(i - (j ? seg_end[j - 1] : 0)));
-    } else {
-      atomicMin(status, (unsigned long long)i);
-    }
-    if (dtype == 1) ((double2*)out)[i] = v;
-    else ((float2*)out)[i] = make_float2((float)v.x, (float)v.y);
-  }
-}
-
-cudaError_t launch_amplitudes(const double2* H, int h, const uint64_t* keys, const uint32_t* groups, int64_t n_keys,
-                              uint64_t tail_mask, const int* open_q, const uint64_t* bits, int64_t n, void* out,
-                              int dtype, unsigned long long* status, cudaStream_t s, const int64_t* seg_end,
-                              int n_seg) {
-  if (n <= 0) return cudaSuccess;
-  const int64_t grid = std::min<int64_t>((n + 255) / 256, (int64_t)kSMs * 8);
-  k_amplitudes<<<(unsigned)grid, 256, 0, s>>>(H, h, keys, groups, n_keys, tail_mask, open_q, bits, n, out, dtype,
-                                              status, seg_end, n_seg);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------- K5
-// One warp per group: chunks of 32 members, each chunk reduced by an inclusive
-// warp scan whose last lane is added to a running carry.  The sampler repeats
-// exactly this order, so its prefix sums end at the same Z[g].
-__device__ __forceinline__ double warp_inclusive_scan(double v) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const double u = __shfl_up_sync(0xffffffffu, v, d);
-    if (lane >= d) v += u;
-  }
-  return v;
-}
-
-__global__ void k_group_norms(const double2* __restrict__ H, int64_t L, int h, double* __restrict__ Z) {
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t l = 1LL << h;
-  for (int64_t g = warp; g < L; g += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    double carry = 0.0;
-    for (int64_t c = 0; c < l; c += 32) {
-      double w = 0.0;
-      if (c + lane < l) {
-        const double2 v = H[(g << h) + c + lane];
-        w = v.x * v.x + v.y * v.y;
-      }
-      const double s = warp_inclusive_scan(w);
-      carry += __shfl_sync(0xffffffffu, s, 31);
-    }
-    if (lane == 0) Z[g] = carry;
-  }
-}
-
-// Deterministic single-block sum of Z into N.
-__global__ void k_sum(const double* __restrict__ Z, int64_t L, double* N) {
-  __shared__ double part[32];
-  double acc = 0.0;
-  for (int64_t i = threadIdx.x; i < L; i += blockDim.x) acc += Z[i];
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    if (threadIdx.x == 0) *N = v;
-  }
-}
-
-// XEB reductions (FP64): part[b] = sum |a_i|^2 and part[nb + b] = sum log |a_i|^2
-// over block b's share of the n amplitudes (grid-stride, then a block tree).
-__global__ void __launch_bounds__(256) k_xeb_partial(const double2* __restrict__ a, int64_t n, double* part) {
-  __shared__ double s1[8], s2[8];
-  double p = 0.0, lp = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = a[i];
-    const double w = v.x * v.x + v.y * v.y;
-    p += w;
-    lp += log(w);
-  }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    p += __shfl_xor_sync(0xffffffffu, p, d);
-    lp += __shfl_xor_sync(0xffffffffu, lp, d);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    s1[threadIdx.x >> 5] = p;
-    s2[threadIdx.x >> 5] = lp;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t1 = 0.0, t2 = 0.0;
-    for (int w = 0; w < 8; ++w) {
-      t1 += s1[w];
-      t2 += s2[w];
-    }
-    part[blockIdx.x] = t1;
-    part[gridDim.x + blockIdx.x] = t2;
-  }
-}
-
-cudaError_t launch_xeb_sums(const double2* amp, int64_t n, double* part, double* sums, cudaStream_t s) {
-  const int64_t nb = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)kSMs * 4));
-  k_xeb_partial<<<(unsigned)nb, 256, 0, s>>>(amp, n, part);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_sum<<<1, 1024, 0, s>>>(part, nb, sums);
-  k_sum<<<1, 1024, 0, s>>>(part + nb, nb, sums + 1);
-  return cudaGetLastError();
-}
-
-int64_t xeb_partials(int64_t n) { return 2 * std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)kSMs * 4)); }
-
-cudaError_t launch_group_norms(const double2* H, int64_t L, int h, double* Z, double* N, cudaStream_t s) {
-  const int64_t warps = L;
-  const int64_t grid = std::min<int64_t>((warps * 32 + 255) / 256, (int64_t)kSMs * 8);
-  k_group_norms<<<(unsigned)std::max<int64_t>(grid, 1), 256, 0, s>>>(H, L, h, Z);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (N) {
-    k_sum<<<1, 1024, 0, s>>>(Z, L, N);
-    e = cudaGetLastError();
-  }
-  return e;
-}
-
-// ---------------------------------------------------------------------- K6
-// Philox-4x32-10 (Salmon et al., SC'11): multipliers 0xD2511F53, 0xCD9E8D57,
-// Weyl key increments 0x9E3779B9, 0xBB67AE85, ten rounds.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-    const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-    c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
-    if (r != 9) { k.x += 0x9E3779B9u; k.y += 0xBB67AE85u; }
-  }
-  return c;
-}
-
-__device__ __forceinline__ double u53(uint32_t lo, uint32_t hi) {
-  const uint64_t x = ((uint64_t)hi << 32) | lo;
-  return (double)(x >> 11) * 0x1.0p-53;
-}
-
-// |h|^2 with each operation rounded to nearest (no fused multiply-add), so
-// that weights and the comparisons built on them are reproducible bit by bit.
-__device__ __forceinline__ double weight_rn(double2 v) { return __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)); }
-
-// One warp per sample, group i mod L.
-//   method 0: exact draw by inverse CDF over the chunked warp-scan prefix sums
-//             of |H[g][mu]|^2 (same order as k_group_norms);
-//   method 1: Metropolis chain with uniform proposals (the paper's in-group
-//             MCMC, Method and Supplement): start at member 0; for t < T,
-//             propose mu' = bits of Philox(i, 2, t), accept when
-//             u * w(mu) < w(mu');
-//   method 2: frugal rejection sampling (Supplement, bitstring choice): for
-//             t < 64 M rounds, draw mu = bits of Philox(i, 3, t) and accept
-//             when (u * M) * Z < w(mu) * l; after the last round keep mu.
-__global__ void k_sample(SampleParams p) {
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t l = 1LL << p.h;
-  const uint2 key = make_uint2((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
-  const uint64_t full = p.n_qubits >= 64 ? ~0ULL : ((1ULL << p.n_qubits) - 1);
-  for (int64_t i = warp; i < p.n; i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t g = i % p.L;
-    const uint32_t ilo = (uint32_t)i, ihi = (uint32_t)((uint64_t)i >> 32);
-    const uint4 r = philox4x32_10(make_uint4(ilo, ihi, 0u, 0u), key);
-    const double u_mix = u53(r.x, r.y), u_pick = u53(r.z, r.w);
-    if (p.mix > 0.0 && u_mix < p.mix) {
-      const uint4 q = philox4x32_10(make_uint4(ilo, ihi, 1u, 0u), key);
-      if (lane == 0) p.out[i] = ((((uint64_t)q.y) << 32) | q.x) & full;
-      continue;
-    }
-    const double2* __restrict__ Hg = p.H + (g << p.h);
-    int64_t mu = l - 1;
-    if (p.method == 1) {
-      // lane 0 runs the chain (it is sequential); the other lanes idle
-      if (lane == 0) {
-        int64_t cur = 0;
-        double wc = weight_rn(Hg[0]);
-        for (int64_t t = 0; t < p.param; ++t) {
-          const uint4 q = philox4x32_10(make_uint4(ilo, ihi, 2u, (uint32_t)t), key);
-          const int64_t prop = (int64_t)(q.x & (uint32_t)(l - 1));
-          const double wp = weight_rn(Hg[prop]);
-          const double u = u53(q.z, q.w);
-          if (__dmul_rn(u, wc) < wp) { cur = prop; wc = wp; }
-        }
-        mu = cur;
-      }
-    } else {
-      // chunked warp-scan total (exact draw and frugal bound)
-      double Z = 0.0;
-      for (int64_t c = 0; c < l; c += 32) {
-        const double w = (c + lane < l) ? weight_rn(Hg[c + lane]) : 0.0;
-        const double s = warp_inclusive_scan(w);
-        Z += __shfl_sync(0xffffffffu, s, 31);
-      }
-      if (p.method == 2) {
-        if (lane == 0) {
-          const double M = (double)p.param;
-          const double bound = __dmul_rn(M, Z);
-          int64_t cand = 0;
-          for (int64_t t = 0; t < 64 * p.param; ++t) {
-            const uint4 q = philox4x32_10(make_uint4(ilo, ihi, 3u, (uint32_t)t), key);
-            cand = (int64_t)(q.x & (uint32_t)(l - 1));
-            const double u = u53(q.z, q.w);
-            if (__dmul_rn(u, bound) < __dmul_rn(weight_rn(Hg[cand]), (double)l)) break;
-          }
-          mu = cand;
-        }
-      } else if (Z > 0.0) {
-        const double t = u_pick * Z;
-        double carry = 0.0;
-        for (int64_t c = 0; c < l; c += 32) {
-          const double w = (c + lane < l) ? weight_rn(Hg[c + lane]) : 0.0;
-          const double s = warp_inclusive_scan(w);
-          const bool hit = (c + lane < l) && (carry + s > t);
-          const unsigned ball = __ballot_sync(0xffffffffu, hit);
-          if (ball) { mu = c + __ffs(ball) - 1; break; }
-          carry += __shfl_sync(0xffffffffu, s, 31);
-        }
-      } else {
-        mu = (int64_t)(u_pick * (double)l);
-        if (mu >= l) mu = l - 1;
-      }
-    }
-    if (lane == 0) {
-      uint64_t s = p.tails[g] & ~p.open_mask;
-      for (int j = 0; j < p.h; ++j) s |= (uint64_t)((mu >> j) & 1) << p.open_q[j];
-      p.out[i] = s;
-    }
-  }
-}
-
-cudaError_t launch_sample(const SampleParams& p, cudaStream_t s) {
-  if (p.n <= 0) return cudaSuccess;
-  const int64_t grid = std::min<int64_t>((p.n * 32 + 255) / 256, (int64_t)kSMs * 16);
-  k_sample<<<(unsigned)grid, 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <cstddef>
 #include <cstdint>
 
 #include "direct.h"
@@ -127,21 +128,32 @@ cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s);
 cudaError_t prepare_direct();    // the direct step's opt-in shared-memory sizes; likewise
 cudaError_t prepare_permute();   // the permute's opt-in shared-memory size; likewise
 
+// What a head operation reports to the host, in mapped host memory.  The host
+// sets `missing` to ~0 and `word` to 0 before the launch.
+struct HeadReport {
+  unsigned long long missing;   // smallest index whose bitstring is not in the state
+  unsigned int word;            // the plan's status word
+  double sum[2];                // norm; or the XEB sums
+};
+// Scratch of the norm and XEB reductions: 2 * kHeadParts doubles.
+constexpr int kHeadParts = 1216;
+
 // amplitude lookup: out[i] = H[g][mu] (c128 or c64); status <- min missing
 // index, or with seg_end (cumulative ends of n_seg merged requests, device)
 // status[j] <- min missing index within request j
 cudaError_t launch_amplitudes(const double2* H, int h, const uint64_t* keys, const uint32_t* groups, int64_t n_keys,
                               uint64_t tail_mask, const int* open_q, const uint64_t* bits, int64_t n, void* out,
                               int dtype, unsigned long long* status, cudaStream_t s, const int64_t* seg_end = nullptr,
-                              int n_seg = 1);
+                              int n_seg = 1, HeadReport* rep = nullptr, const unsigned int* plan_status = nullptr);
 
-// per-group squared norms Z[g] (chunked warp order) and the total N
-cudaError_t launch_group_norms(const double2* H, int64_t L, int h, double* Z, double* N, cudaStream_t s);
+// per-group squared norms Z[g] and their total (into *N and the report, where given)
+cudaError_t launch_group_norms(const double2* H, int64_t L, int h, double* Z, double* N, double* scratch,
+                               cudaStream_t s, HeadReport* rep = nullptr, const unsigned int* plan_status = nullptr);
 
-// sums[0] = sum |a_i|^2, sums[1] = sum log |a_i|^2 over n complex128 amplitudes
-// (FP64; `part` holds xeb_partials(n) doubles of scratch)
-cudaError_t launch_xeb_sums(const double2* amp, int64_t n, double* part, double* sums, cudaStream_t s);
-int64_t xeb_partials(int64_t n);
+// rep->sum = sum |a_i|^2 and sum log |a_i|^2 over the amplitudes a_i of n samples
+cudaError_t launch_xeb(const double2* H, int h, const uint64_t* keys, const uint32_t* groups, int64_t n_keys,
+                       uint64_t tail_mask, const int* open_q, const uint64_t* samples, int64_t n, double* scratch,
+                       HeadReport* rep, cudaStream_t s);
 
 struct SampleParams {
   const double2* H; int64_t L; int h;
@@ -153,7 +165,11 @@ struct SampleParams {
   uint64_t* out;
   int method;                 // 0 exact inverse CDF, 1 Metropolis chain, 2 frugal rejection
   int64_t param;              // chain length (1) or the bound M (2)
+  double* carry = nullptr;    // scratch of sample_scratch_doubles() doubles (prefix sums)
+  HeadReport* rep = nullptr;  // may be null, as may plan_status
+  const unsigned int* plan_status = nullptr;
 };
+size_t sample_scratch_doubles(int64_t L, int h, int64_t n, int method);
 cudaError_t launch_sample(const SampleParams& p, cudaStream_t s);
 
 }  // namespace tn

@@ -20,10 +20,11 @@ void set_last_error(const std::string& msg);
 
 namespace {
 
-// Per-group partial sums; every GPU that loads the library holds this array
-// (1 MiB) until the process exits.
+// Partial sums; every GPU that loads the library holds this array (1 MiB and
+// 19 KiB) until the process exits.
 constexpr int64_t kMaxGroups = TN_NOALLOC_MAX_GROUPS;
-static __device__ __align__(256) double g_group_sums[kMaxGroups];
+// the groups' sums, then the reduction's partial sums
+static __device__ __align__(256) double g_group_sums[kMaxGroups + 2 * tn::kHeadParts];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -69,7 +70,8 @@ extern "C" int tn_head_norm_noalloc(const void* head_c128, int64_t n_groups, int
   }
   // every entry read by the sum is first written by the per-group pass, so
   // nothing left by an earlier call needs clearing
-  e = tn::launch_group_norms((const double2*)head_c128, n_groups, n_open, scratch, norm_out, (cudaStream_t)stream);
+  e = tn::launch_group_norms((const double2*)head_c128, n_groups, n_open, scratch, norm_out, scratch + kMaxGroups,
+                             (cudaStream_t)stream);
   if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("norm launch: ") + cudaGetErrorString(e));
   return TN_OK;
 }

@@ -194,7 +194,8 @@ int enqueue_op(Slot& s, Request* q, Circuit& c) {
   tn_plan_t* p = c.plan;
   const int h = (int)p->P.open_qubits.size();
   const size_t n = (size_t)r.n;
-  if (ensure_slot_buffers(s, std::max<size_t>(n * 8, 256), std::max<size_t>(n * 8, 256)))
+  const size_t scratch = 8 * tn::sample_scratch_doubles((int64_t)p->P.tails_raw.size(), h, r.n, r.method);
+  if (ensure_slot_buffers(s, std::max<size_t>(n * 8 + scratch, 256), std::max<size_t>(n * 8, 256)))
     return fail(TN_ERR_OOM, "server: slot staging allocation failed");
   cudaStream_t st = s.stream;
   if (c.state == C_BUILDING && !s.building) cudaStreamWaitEvent(st, c.ready, 0);
@@ -218,6 +219,7 @@ int enqueue_op(Slot& s, Request* q, Circuit& c) {
   sp.method = r.method;
   sp.param = r.param != 0 ? r.param
                           : (r.method == TN_SAMPLE_METROPOLIS ? ((int64_t)1 << h) : (r.method == TN_SAMPLE_FRUGAL ? 10 : 0));
+  sp.carry = scratch ? (double*)d + n : nullptr;
   cudaError_t e = tn::launch_sample(sp, st);
   if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("server: sample: ") + cudaGetErrorString(e));
   if (cudaMemcpyAsync(s.h_buf, d, n * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
