@@ -99,6 +99,134 @@ static int report_status(tn_head_t* h, unsigned int word, cudaStream_t st) {
 extern "C" const char* tn_last_error(void) { return g_err.c_str(); }
 extern "C" const char* tn_version(void) { return kVersion; }
 
+// Per-call scratch: a report in mapped host memory and the partial sums of a
+// reduction on the device, plus a device and a pinned host buffer that grow on
+// demand (prefix sums, GEMM operands, pattern maps).  Each call takes one for
+// its duration, so calls from several threads and streams share none.  Between
+// calls at most kMost are kept, with at most kKeepBytes of buffers among them;
+// all of it is given back when a device allocation of the library fails.
+struct CallScratch {
+  tn::HeadReport* rep = nullptr;
+  double* part = nullptr;
+  void* buf = nullptr;
+  size_t bytes = 0;
+  void* host = nullptr;
+  size_t host_bytes = 0;
+  int device = -1;
+};
+
+static std::mutex g_scratch_mu;
+static std::vector<CallScratch> g_scratch;
+
+static void free_scratch(CallScratch& c) {
+  cudaFreeHost(c.rep);
+  cudaFreeHost(c.host);
+  cudaFree(c.part);
+  cudaFree(c.buf);
+  c = CallScratch();
+}
+
+static void trim_scratch() {
+  std::lock_guard<std::mutex> lock(g_scratch_mu);
+  for (CallScratch& c : g_scratch) free_scratch(c);
+  g_scratch.clear();
+}
+
+// cudaMalloc that gives the kept scratch back and tries again before it fails
+static cudaError_t malloc_or_trim(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    trim_scratch();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
+struct ScratchLease {
+  static constexpr size_t kMost = 32, kKeepBytes = (size_t)2 << 30;
+  CallScratch c;
+  cudaStream_t stream;
+  bool in_flight = false;
+  explicit ScratchLease(cudaStream_t st) : stream(st) {}
+  ScratchLease(const ScratchLease&) = delete;
+  ScratchLease& operator=(const ScratchLease&) = delete;
+  ~ScratchLease() {
+    if (!c.rep) return;
+    if (in_flight) cudaStreamSynchronize(stream);   // the call failed after a launch
+    {
+      std::lock_guard<std::mutex> lock(g_scratch_mu);
+      size_t kept = c.bytes;
+      for (const CallScratch& o : g_scratch) kept += o.bytes;
+      if (g_scratch.size() < kMost && kept <= kKeepBytes) {
+        g_scratch.push_back(c);
+        return;
+      }
+    }
+    free_scratch(c);
+  }
+  // The report, once the stream is synchronised.
+  tn::HeadReport done() {
+    in_flight = false;
+    return *c.rep;
+  }
+  // Call before the launches; the report starts as "nothing missing, no status".
+  int take(size_t bytes, size_t host_bytes = 0) {
+    int dev = -1;
+    CUDA_TRY(cudaGetDevice(&dev));
+    {
+      // the kept one with the smallest buffer that is large enough, else the largest
+      std::lock_guard<std::mutex> lock(g_scratch_mu);
+      g_scratch.reserve(kMost);
+      size_t at = g_scratch.size();
+      for (size_t i = 0; i < g_scratch.size(); ++i) {
+        if (g_scratch[i].device != dev) continue;
+        if (at == g_scratch.size()) { at = i; continue; }
+        const size_t x = g_scratch[i].bytes, y = g_scratch[at].bytes;
+        if (x >= bytes ? (y < bytes || x < y) : (y < bytes && x > y)) at = i;
+      }
+      if (at < g_scratch.size()) {
+        c = g_scratch[at];
+        g_scratch.erase(g_scratch.begin() + (std::ptrdiff_t)at);
+      }
+    }
+    if (!c.rep) {
+      c.device = dev;
+      void* h = nullptr;
+      if (cudaHostAlloc(&h, sizeof(tn::HeadReport), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
+          malloc_or_trim((void**)&c.part, 2 * tn::kHeadParts * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        if (h) cudaFreeHost(h);
+        return fail(TN_ERR_OOM, "scratch allocation failed");
+      }
+      c.rep = (tn::HeadReport*)h;   // one address on host and device (unified addressing)
+    }
+    if (c.bytes < bytes) {
+      cudaFree(c.buf);
+      c.buf = nullptr;
+      c.bytes = 0;
+      if (malloc_or_trim(&c.buf, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(TN_ERR_OOM, "scratch allocation failed");
+      }
+      c.bytes = bytes;
+    }
+    if (c.host_bytes < host_bytes) {
+      cudaFreeHost(c.host);
+      c.host = nullptr;
+      c.host_bytes = 0;
+      if (cudaHostAlloc(&c.host, host_bytes, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(TN_ERR_OOM, "scratch allocation failed");
+      }
+      c.host_bytes = host_bytes;
+    }
+    *c.rep = tn::HeadReport{~0ULL, 0u, {0.0, 0.0}};
+    in_flight = true;
+    return TN_OK;
+  }
+};
+
 static void plan_release(tn_plan_t* p) {
   if (!p) return;
   if (p->on_device) {
@@ -144,7 +272,7 @@ static int plan_upload(tn_plan_t* p) {
   if (!P.meta.empty())
     CUDA_TRY(cudaMemcpy(p->d_meta, P.meta.data(), P.meta.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
   if (P.workspace_bytes > 0) {
-    cudaError_t e = cudaMalloc(&p->d_arena, (size_t)P.workspace_bytes);
+    cudaError_t e = malloc_or_trim((void**)&p->d_arena, (size_t)P.workspace_bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(TN_ERR_OOM, "workspace of " + std::to_string(P.workspace_bytes) + " bytes: " + cudaGetErrorString(e));
@@ -331,7 +459,7 @@ extern "C" int tn_head_create(tn_plan_t* plan, void* dev_c128, tn_head_t** out) 
   if (dev_c128) {
     h->H = (double2*)dev_c128;
   } else {
-    cudaError_t e = cudaMalloc(&h->H, (size_t)elems * sizeof(double2));
+    cudaError_t e = malloc_or_trim((void**)&h->H, (size_t)elems * sizeof(double2));
     if (e != cudaSuccess) {
       cudaGetLastError();
       delete h;
@@ -1077,7 +1205,7 @@ static int ensure_stage(tn_head* h, size_t bytes) {
   cudaFree(h->d_stage);
   h->d_stage = nullptr;
   h->stage_bytes = 0;
-  cudaError_t e = cudaMalloc(&h->d_stage, bytes);
+  cudaError_t e = malloc_or_trim(&h->d_stage, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(TN_ERR_OOM, "staging buffer allocation failed");
@@ -1085,101 +1213,6 @@ static int ensure_stage(tn_head* h, size_t bytes) {
   h->stage_bytes = bytes;
   return TN_OK;
 }
-
-// Per-call scratch of the head operations: a report in mapped host memory and
-// the partial sums of a reduction on the device, plus a device buffer that
-// grows on demand (the sampler's prefix sums).  Each call takes one for its
-// duration, so calls on one head from several threads and streams do not share
-// any.  At most kMost of them stay between calls, and one whose
-// buffer grew past kKeepBytes gives it back.
-struct CallScratch {
-  tn::HeadReport* rep = nullptr;
-  double* part = nullptr;
-  void* buf = nullptr;
-  size_t bytes = 0;
-  int device = -1;
-};
-
-static std::mutex g_scratch_mu;
-static std::vector<CallScratch> g_scratch;
-
-static void free_scratch(CallScratch& c) {
-  cudaFreeHost(c.rep);
-  cudaFree(c.part);
-  cudaFree(c.buf);
-  c = CallScratch();
-}
-
-struct ScratchLease {
-  static constexpr size_t kMost = 32, kKeepBytes = (size_t)64 << 20;
-  CallScratch c;
-  cudaStream_t stream;
-  bool in_flight = false;
-  explicit ScratchLease(cudaStream_t st) : stream(st) {}
-  ScratchLease(const ScratchLease&) = delete;
-  ScratchLease& operator=(const ScratchLease&) = delete;
-  ~ScratchLease() {
-    if (!c.rep) return;
-    if (in_flight) cudaStreamSynchronize(stream);   // the call failed after a launch
-    if (c.bytes > kKeepBytes) {
-      cudaFree(c.buf);
-      c.buf = nullptr;
-      c.bytes = 0;
-    }
-    {
-      std::lock_guard<std::mutex> lock(g_scratch_mu);
-      if (g_scratch.size() < kMost) {
-        g_scratch.push_back(c);
-        return;
-      }
-    }
-    free_scratch(c);
-  }
-  // The report, once the stream is synchronised.
-  tn::HeadReport done() {
-    in_flight = false;
-    return *c.rep;
-  }
-  // Call before the launches; the report starts as "nothing missing, no status".
-  int take(size_t bytes) {
-    int dev = -1;
-    CUDA_TRY(cudaGetDevice(&dev));
-    {
-      std::lock_guard<std::mutex> lock(g_scratch_mu);
-      g_scratch.reserve(kMost);
-      for (size_t i = g_scratch.size(); i-- > 0;)
-        if (g_scratch[i].device == dev) {
-          c = g_scratch[i];
-          g_scratch.erase(g_scratch.begin() + (std::ptrdiff_t)i);
-          break;
-        }
-    }
-    if (!c.rep) {
-      c.device = dev;
-      void* h = nullptr;
-      if (cudaHostAlloc(&h, sizeof(tn::HeadReport), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
-          cudaMalloc(&c.part, 2 * tn::kHeadParts * sizeof(double)) != cudaSuccess) {
-        cudaGetLastError();
-        if (h) cudaFreeHost(h);
-        return fail(TN_ERR_OOM, "scratch allocation failed");
-      }
-      c.rep = (tn::HeadReport*)h;   // one address on host and device (unified addressing)
-    }
-    if (c.bytes < bytes) {
-      cudaFree(c.buf);
-      c.buf = nullptr;
-      c.bytes = 0;
-      if (cudaMalloc(&c.buf, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(TN_ERR_OOM, "scratch allocation failed");
-      }
-      c.bytes = bytes;
-    }
-    *c.rep = tn::HeadReport{~0ULL, 0u, {0.0, 0.0}};
-    in_flight = true;
-    return TN_OK;
-  }
-};
 
 // A pointer that kernels can use as it is: device or managed memory, or pinned
 // host memory, which GB300 reads and writes over NVLink-C2C without a copy.
@@ -1430,16 +1463,15 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
     }
     if (best.seconds < tn::tc_seconds(nm, nn, nk, PC, mode[0] == 1, (double)PA * (double)(M * K),
                                       (double)PB * (double)(K * N), (double)PC * (double)(M * N), h16 != 0)) {
-      CUDA_TRY(tn::prepare_direct());
-      uint32_t* d_maps = nullptr;
       const size_t n_map = maps[0].size() + maps[1].size();
-      if (n_map && cudaMalloc(&d_maps, n_map * sizeof(uint32_t)) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(TN_ERR_OOM, "tn_gemm_c64 scratch allocation failed");
+      ScratchLease lease(st);
+      if (int rc = lease.take(n_map * sizeof(uint32_t), n_map * sizeof(uint32_t))) return rc;
+      uint32_t* d_maps = (uint32_t*)lease.c.buf;
+      if (n_map) {
+        std::copy(maps[0].begin(), maps[0].end(), (uint32_t*)lease.c.host);
+        std::copy(maps[1].begin(), maps[1].end(), (uint32_t*)lease.c.host + maps[0].size());
+        CUDA_TRY(cudaMemcpyAsync(d_maps, lease.c.host, n_map * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
       }
-      maps[0].insert(maps[0].end(), maps[1].begin(), maps[1].end());
-      cudaError_t e = cudaSuccess;
-      if (n_map) e = cudaMemcpyAsync(d_maps, maps[0].data(), n_map * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
       tn::DirectParams dp{};
       tn::direct_fill(best, PC, dp);
       dp.X = (const float2*)B;
@@ -1448,100 +1480,47 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
       dp.x_pstride = K * N;
       dp.y_pstride = M * K;
       dp.c_pstride = M * N;
-      dp.mapX = d_maps + (n_map - maps[1].size());
+      dp.mapX = d_maps + maps[0].size();
       dp.mapY = d_maps;
       dp.mapX_mode = mode[1];
       dp.mapY_mode = mode[0];
       dp.vec = (uintptr_t)C % 16 == 0;
       dp.amax = nullptr;
-      if (e == cudaSuccess) e = tn::launch_direct(dp, best.config, st);
+      cudaError_t e = tn::launch_direct(dp, best.config, st, true);
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      cudaFree(d_maps);
       if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("tn_gemm_c64: ") + cudaGetErrorString(e));
+      lease.done();
       return TN_OK;
     }
   }
-  CUDA_TRY(tn::prepare_gemm_tc());   // kernel attributes (shared-memory size), as at plan upload
-  CUDA_TRY(tn::prepare_permute());
-  // scratch: split A planes, prepared B, tables, scale slots
+  // scratch: scale slots, pattern maps, split A planes, prepared B
   const int64_t es = h16 ? 2 : 4;
-  const int split = simt ? 0 : (h16 == 2 ? 3 : h16 == 1 ? 2 : 1);
-  const int64_t a_bytes = simt ? 0 : PA * M * K * 8 * (split == 1 ? 2 : 1);
-  const int64_t b_bytes = simt ? PB * K * N * 8 : 2 * PB * (2 * N) * (2 * K) * es;
-  const int t = std::min(nmk, 10);
-  std::vector<uint32_t> meta;
-  const size_t tab_off = meta.size();
-  for (int i = 0; i < (1 << t); ++i) meta.push_back((uint32_t)i);   // identity tile: in offsets
-  for (int i = 0; i < (1 << t); ++i) meta.push_back((uint32_t)i);   // out offsets
-  for (int i = 0; i < (1 << t); ++i) meta.push_back((uint32_t)i);   // slots
-  const size_t bk_off = meta.size();
-  for (int64_t k = 0; k < K; ++k) meta.push_back((uint32_t)(k * N));
-  const size_t bn_off = meta.size();
-  for (int64_t n = 0; n < N; ++n) meta.push_back((uint32_t)n);
-  const size_t map_off[2] = {meta.size(), meta.size() + maps[0].size()};
-  meta.insert(meta.end(), maps[0].begin(), maps[0].end());
-  meta.insert(meta.end(), maps[1].begin(), maps[1].end());
-  char* a_split = nullptr;
-  char* b_prep = nullptr;
-  uint32_t* d_meta = nullptr;
-  unsigned int* d_scale = nullptr;   // [0] max of A, [1] max of B, [2] status
-  int rc = TN_OK;
-  auto cleanup = [&]() {
-    cudaFree(a_split);
-    cudaFree(b_prep);
-    cudaFree(d_meta);
-    cudaFree(d_scale);
-  };
-  if ((a_bytes && cudaMalloc(&a_split, (size_t)a_bytes) != cudaSuccess) ||
-      cudaMalloc(&b_prep, (size_t)b_bytes) != cudaSuccess ||
-      cudaMalloc(&d_meta, meta.size() * sizeof(uint32_t)) != cudaSuccess ||
-      cudaMalloc(&d_scale, 3 * sizeof(unsigned int)) != cudaSuccess) {
-    cudaGetLastError();
-    cleanup();
-    return fail(TN_ERR_OOM, "tn_gemm_c64 scratch allocation failed");
+  const size_t n_map = maps[0].size() + maps[1].size();
+  const size_t map_off = 256, a_off = (map_off + n_map * sizeof(uint32_t) + 1023) / 1024 * 1024;
+  const size_t a_bytes = simt ? 0 : (size_t)(2 * PA * M * (2 * K) * es);
+  const size_t b_off = a_off + (a_bytes + 1023) / 1024 * 1024;
+  const size_t b_bytes = simt ? 0 : (size_t)(2 * PB * (2 * N) * (2 * K) * es);
+  ScratchLease lease(st);
+  if (int rc = lease.take(b_off + b_bytes, n_map * sizeof(uint32_t))) return rc;
+  char* d = (char*)lease.c.buf;
+  unsigned int* d_scale = (unsigned int*)d;   // [0] max of A, [1] max of B
+  uint32_t* d_maps = (uint32_t*)(d + map_off);
+  cudaError_t e = cudaSuccess;
+  if (n_map) {
+    std::copy(maps[0].begin(), maps[0].end(), (uint32_t*)lease.c.host);
+    std::copy(maps[1].begin(), maps[1].end(), (uint32_t*)lease.c.host + maps[0].size());
+    e = cudaMemcpyAsync(d_maps, lease.c.host, n_map * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
   }
-  cudaError_t e = cudaMemcpyAsync(d_meta, meta.data(), meta.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_scale, 0, 3 * sizeof(unsigned int), st);
-  if (e == cudaSuccess && h16 == 2) {
-    tn::AbsmaxParams ap{(const float2*)A, PA * M * K, d_scale};
-    e = tn::launch_absmax(ap, st);
-    if (e == cudaSuccess) {
-      tn::AbsmaxParams bp{(const float2*)B, PB * K * N, d_scale + 1};
-      e = tn::launch_absmax(bp, st);
-    }
-  }
-  if (e == cudaSuccess && !simt) {   // A -> split planes (identity bit permutation)
-    tn::PermParams pp;
-    pp.in = (const float2*)A;
-    pp.out = (float2*)a_split;
-    pp.pstride = M * K;
-    pp.P = PA;
-    pp.t = t;
-    pp.n_rest = nmk - t;
-    for (int x = 0; x < pp.n_rest; ++x) pp.rest_in[x] = pp.rest_out[x] = (uint8_t)(t + x);
-    pp.tab = d_meta + tab_off;
-    pp.split = split;
-    pp.scale = d_scale;
-    e = tn::launch_permute(pp, st);
-  }
-  if (e == cudaSuccess) {   // B -> real embedding (tensor cores) or [K][N] copy (CUDA cores)
-    tn::BPrepParams bp;
-    bp.B = (const float2*)B;
-    bp.out = b_prep;
-    bp.b_pstride = K * N;
-    bp.PB = PB;
-    bp.nk = nk;
-    bp.nn = nn;
-    bp.bk = d_meta + bk_off;
-    bp.bn = d_meta + bn_off;
-    bp.h16 = h16;
-    bp.scale = d_scale + 1;
-    e = simt ? tn::launch_bprep_c(bp, st) : tn::launch_bprep_tc(bp, st);
+  tn::GemmParams gp;
+  if (!simt) {
+    if (e == cudaSuccess && h16 == 2) e = cudaMemsetAsync(d_scale, 0, 2 * sizeof(unsigned int), st);
+    tn::GemmOperands op{(const float2*)A, (const float2*)B, d + a_off, d + b_off, PA * M * K, K, N, PB, h16, d_scale};
+    if (e == cudaSuccess) e = tn::launch_gemm_operands(op, st);
   }
   if (e == cudaSuccess) {
-    tn::GemmParams gp;
-    gp.A = simt ? (const float2*)A : (const float2*)a_split;
-    gp.B = b_prep;
+    // the CUDA-core GEMM reads both row-major operands as they are
+    gp.A = simt ? (const float2*)A : (const float2*)(d + a_off);
+    gp.B = simt ? B : (const void*)(d + b_off);
     gp.C = (float2*)C;
     gp.M = M;
     gp.N = N;
@@ -1549,8 +1528,8 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
     gp.PA = PA;
     gp.PB = PB;
     gp.PC = PC;
-    gp.mapA = d_meta + map_off[0];
-    gp.mapB = d_meta + map_off[1];
+    gp.mapA = d_maps;
+    gp.mapB = d_maps + maps[0].size();
     gp.mapA_mode = mode[0];
     gp.mapB_mode = mode[1];
     gp.h16 = h16;
@@ -1558,18 +1537,13 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
     gp.scaleB = d_scale + 1;
     gp.amax = nullptr;
     gp.pair = pair < 0 ? -1 : 0;
-    e = simt ? tn::launch_gemm_simt(gp, st) : tn::launch_gemm_tc(gp, d_scale + 2, st);
+    gp.prepare = 1;
+    e = simt ? tn::launch_gemm_simt(gp, st) : tn::launch_gemm_tc(gp, &lease.c.rep->word, st);
   }
-  unsigned int word = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&word, d_scale + 2, sizeof(word), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) {
-    rc = fail(TN_ERR_CUDA, std::string("tn_gemm_c64: ") + cudaGetErrorString(e));
-  } else if (word) {
-    rc = fail(TN_ERR_TIMEOUT, "tn_gemm_c64: a bounded device wait gave up");
-  }
-  cleanup();
-  return rc;
+  if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("tn_gemm_c64: ") + cudaGetErrorString(e));
+  if (lease.done().word) return fail(TN_ERR_TIMEOUT, "tn_gemm_c64: a bounded device wait gave up");
+  return TN_OK;
 }
 
 extern "C" int tn_plan_autotune(const tn_circuit* circuit, const tn_open_spec* open_spec, const tn_edge* sliced_edges,

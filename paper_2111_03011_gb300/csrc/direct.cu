@@ -348,11 +348,15 @@ cudaError_t prepare_direct() {
   return cudaSuccess;
 }
 
-cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s) {
+cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s, bool prepare) {
   if (config < 0 || config >= kNumDirectConfigs) return cudaErrorInvalidValue;
   const int64_t tiles = ((int64_t)p.col_tiles << p.n_rrest) * (p.fold ? 1 : p.PC);
   if (tiles < 1 || tiles * p.cluster > 0x7fffffffLL) return cudaErrorInvalidValue;
   const DirectEntry& e = kEntries[config];
+  if (prepare) {
+    const cudaError_t r = cudaFuncSetAttribute((const void*)e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
+    if (r != cudaSuccess) return r;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(tiles * p.cluster));
   cfg.blockDim = dim3(256);

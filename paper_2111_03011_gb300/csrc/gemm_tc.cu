@@ -901,6 +901,10 @@ static cudaError_t run(const GemmParams& p, int fold, unsigned int* status, cuda
   const int64_t PCg = (p.PC + fold - 1) / fold;
   const int64_t n_tiles = tilesM * tilesN * PCg;
   if (n_tiles <= 0) return cudaSuccess;
+  if (p.prepare) {
+    const cudaError_t e = set_attr<BN, STAGES, FMT>();
+    if (e != cudaSuccess) return e;
+  }
   // persistent: at most one CTA per SM (the pipeline's shared memory allows one)
   const int64_t grid = std::min<int64_t>(n_tiles, sm_count());
   k_gemm_tc<BN, STAGES, FMT><<<(unsigned)grid, kThreads, Lay::TOTAL, s>>>(
@@ -943,6 +947,10 @@ static cudaError_t run_pair(const GemmParams& p, int fold, unsigned int* status,
   const int64_t PCg = (p.PC + fold - 1) / fold;
   const int64_t n_tiles = tilesM * tilesN * PCg;
   if (n_tiles <= 0) return cudaSuccess;
+  if (p.prepare) {
+    const cudaError_t e = set_attr_pair<FMT>();
+    if (e != cudaSuccess) return e;
+  }
   const int64_t clusters = std::min<int64_t>(n_tiles, sm_count() / 2);
   k_gemm_tc_pair<kPairStages, FMT><<<(unsigned)(2 * clusters), kThreads, Lay::TOTAL, s>>>(
       tah, tal, tbh, tbl, (float*)p.C, p.M, N2, K2, tilesM, tilesN, p.PC, PCg, fold, p.mapA, p.mapB, p.mapA_mode,

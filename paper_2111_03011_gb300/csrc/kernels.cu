@@ -514,6 +514,130 @@ cudaError_t launch_bprep_tc(const BPrepParams& p, cudaStream_t s, bool beside_ge
   return cudaGetLastError();
 }
 
+// --------------------------------------------- operands of a standalone GEMM
+// Row-major operands need no gather tables: one launch takes the maxima of both
+// (16-byte loads), one splits A as a stream and transposes B's tiles of
+// 32 k x 32 n through shared memory, so that it is read along n and its
+// embedding written along k, both coalesced.  M = 2^13, N = 2^10, K = 2^11 in
+// fp16: two maximum passes, permute kernel and gather kernel took 107 us, these
+// two launches about 85 us of a 385 us call (the GEMM itself 277 us).
+__global__ void __launch_bounds__(256) k_gemm_max(const float2* __restrict__ A, int64_t nA, int blocks_a,
+                                                  const float2* __restrict__ B, int64_t nB, int vec,
+                                                  unsigned int* scale) {
+  __shared__ unsigned int red[8];
+  const bool a = (int)blockIdx.x < blocks_a;
+  const float2* __restrict__ p = a ? A : B;
+  const int64_t n = a ? nA : nB;
+  const int64_t b = a ? blockIdx.x : blockIdx.x - blocks_a, nb = a ? blocks_a : gridDim.x - blocks_a;
+  float m = 0.0f;
+  int64_t done = 0;
+  if (vec) {                                    // two elements per load
+    done = n & ~(int64_t)1;
+    const float4* q = (const float4*)p;
+#pragma unroll 4
+    for (int64_t i = b * 256 + threadIdx.x; i < n >> 1; i += nb * 256) {
+      const float4 v = __ldg(q + i);
+      m = fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+    }
+  }
+  for (int64_t i = done + b * 256 + threadIdx.x; i < n; i += nb * 256) {
+    const float2 v = __ldg(p + i);
+    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+  }
+  const unsigned int w = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const unsigned int t = __reduce_max_sync(0xffffffffu, threadIdx.x < 8 ? red[threadIdx.x] : 0u);
+    if (threadIdx.x == 0) atomicMax(scale + (a ? 0 : 1), t);
+  }
+}
+
+template <int FMT>
+__global__ void __launch_bounds__(256) k_gemm_operands(GemmOperands p, int64_t blocks_b, int vec) {
+  using PT = Pair<FMT>;
+  using T = typename PT::T;
+  if ((int64_t)blockIdx.x >= blocks_b) {
+    // A: four consecutive elements per thread and round (the count is a
+    // multiple of four for the 16-bit formats, of two for tf32)
+    const float sc = FMT == 2 ? pow2f(fp16_scale_exp(p.scale[0])) : 1.0f;
+    T* hi = (T*)p.a_planes;
+    T* lo = hi + p.nA;
+    const int64_t first = ((int64_t)blockIdx.x - blocks_b) * 256 + threadIdx.x;
+    const int64_t step = ((int64_t)gridDim.x - blocks_b) * 256;
+    const int64_t quads = vec ? p.nA >> 2 : 0;
+    for (int64_t i = first; i < quads; i += step) {
+      const float4 u = __ldg((const float4*)p.A + 2 * i), v = __ldg((const float4*)p.A + 2 * i + 1);
+      T h[4], l[4];
+      PT::split(u.x, u.y, sc, h[0], l[0]);
+      PT::split(u.z, u.w, sc, h[1], l[1]);
+      PT::split(v.x, v.y, sc, h[2], l[2]);
+      PT::split(v.z, v.w, sc, h[3], l[3]);
+      store4(hi + 4 * i, h[0], h[1], h[2], h[3]);
+      if (FMT != 0 || (p.nA & 1) == 0) {
+        store4(lo + 4 * i, l[0], l[1], l[2], l[3]);
+      } else {
+        for (int e = 0; e < 4; ++e) lo[4 * i + e] = l[e];
+      }
+    }
+    for (int64_t i = 4 * quads + first; i < p.nA; i += step) {
+      const float2 v = __ldg(p.A + i);
+      T h, l;
+      PT::split(v.x, v.y, sc, h, l);
+      hi[i] = h;
+      lo[i] = l;
+    }
+    return;
+  }
+  __shared__ float2 tile[32][33];
+  const float sc = FMT == 2 ? pow2f(fp16_scale_exp(p.scale[1])) : 1.0f;
+  T* hi = (T*)p.b_planes;
+  T* lo = hi + 2 * p.PB * p.K * p.N;
+  const int64_t tk = (p.K + 31) >> 5, tn = (p.N + 31) >> 5;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  for (int64_t t = blockIdx.x; t < p.PB * tk * tn; t += blocks_b) {
+    const int64_t n0 = (t % tn) * 32, k0 = (t / tn % tk) * 32, pb = t / (tn * tk);
+    __syncthreads();
+#pragma unroll
+    for (int j = y; j < 32; j += 8)
+      if (k0 + j < p.K && n0 + x < p.N) tile[j][x] = __ldg(p.B + (pb * p.K + k0 + j) * p.N + n0 + x);
+    __syncthreads();
+#pragma unroll
+    for (int j = y; j < 32; j += 8) {
+      const int64_t n = n0 + j, k = k0 + x;
+      if (n >= p.N || k >= p.K) continue;
+      const float2 v = tile[x][j];
+      const int64_t o = (pb * 2 * p.N + 2 * n) * p.K + k;   // pair (2k, 2k + 1) of row 2n
+      T h, l;
+      PT::split(v.x, -v.y, sc, h, l);
+      hi[o] = h;
+      lo[o] = l;
+      PT::split(v.y, v.x, sc, h, l);
+      hi[o + p.K] = h;
+      lo[o + p.K] = l;
+    }
+  }
+}
+
+cudaError_t launch_gemm_operands(const GemmOperands& p, cudaStream_t s) {
+  const int64_t nB = p.PB * p.K * p.N;
+  const int vec = (uintptr_t)p.A % 16 == 0;
+  const int64_t cap = (int64_t)kSMs * 8;
+  if (p.fmt == 2) {
+    const int ba = (int)std::min<int64_t>((p.nA + 1023) / 1024, cap), bb = (int)std::min<int64_t>((nB + 1023) / 1024, cap);
+    k_gemm_max<<<(unsigned)(ba + bb), 256, 0, s>>>(p.A, p.nA, ba, p.B, nB, vec && (uintptr_t)p.B % 16 == 0, p.scale);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t bb = std::min<int64_t>(p.PB * ((p.K + 31) / 32) * ((p.N + 31) / 32), cap);
+  const int64_t ba = std::min<int64_t>((p.nA + 1023) / 1024, cap);
+  const unsigned grid = (unsigned)(ba + bb);
+  if (p.fmt == 2) k_gemm_operands<2><<<grid, 256, 0, s>>>(p, bb, vec);
+  else if (p.fmt == 1) k_gemm_operands<1><<<grid, 256, 0, s>>>(p, bb, vec);
+  else k_gemm_operands<0><<<grid, 256, 0, s>>>(p, bb, vec);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------ SIMT GEMM
 // Plain FP32 complex GEMM on CUDA cores: 64x64 complex tile, 16-deep k slab,
 // 4x4 outputs per thread.  The reference "plain complex64" engine.

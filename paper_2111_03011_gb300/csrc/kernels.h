@@ -86,6 +86,7 @@ struct GemmParams {
   unsigned int* amax;    // non-null: atomicMax of the output's max |re|, |im| (fp32 bits)
   int pair = 0;          // 0: CTA-pair 256 x 256 tiles where they apply (16-bit, M >= 256); -1: one-CTA tiles
   int tile_cap = 256;    // widest tile the dispatch may pick, real columns (16..256)
+  int prepare = 0;       // 1: set the launched kernel's attributes first (no plan upload did)
 };
 
 // Tile a tensor-core GEMM launch runs with: BN real columns per tile, fold
@@ -102,6 +103,19 @@ struct DirectParams : DirectParamsBase {
   const uint32_t* mapX; const uint32_t* mapY;
   unsigned int* amax;        // non-null: atomicMax of the output's max |re|, |im| (fp32 bits)
 };
+
+// Operands of a standalone GEMM, row-major A [PA][M][K] and B [PB][K][N], in
+// the tensor-core engines' formats: A as hi and lo planes, B as the real
+// embedding [PB][2N][2K] in hi and lo planes (fmt 0 tf32, 1 bf16, 2 scaled fp16).
+struct GemmOperands {
+  const float2* A; const float2* B;
+  void* a_planes; void* b_planes;
+  int64_t nA;              // complex elements of A
+  int64_t K, N, PB;
+  int fmt;
+  unsigned int* scale;     // fmt 2: [0] max of A, [1] max of B (zeroed before)
+};
+cudaError_t launch_gemm_operands(const GemmOperands& p, cudaStream_t s);
 
 struct AccumParams {
   const float2* F; double2* H;
@@ -124,7 +138,7 @@ cudaError_t launch_accum(const AccumParams& p, cudaStream_t s);
 // `status` receives a nonzero code if a bounded wait gave up.
 cudaError_t launch_gemm_tc(const GemmParams& p, unsigned int* status, cudaStream_t s);
 cudaError_t prepare_gemm_tc();   // kernel attributes; call before launching or capturing
-cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s);
+cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s, bool prepare = false);
 cudaError_t prepare_direct();    // the direct step's opt-in shared-memory sizes; likewise
 cudaError_t prepare_permute();   // the permute's opt-in shared-memory size; likewise
 

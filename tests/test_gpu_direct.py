@@ -79,3 +79,31 @@ def test_gemm_kernels_on_request(tn, engine, shape):
     tn.tn_gemm_c64(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), c, engine=engine, pair=1)
     got = c.cpu().numpy()
     assert np.linalg.norm(got - ref) <= (1e-4 if engine == 3 else 1e-5) * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("engine", [1, 2, 3, 4], ids=["tf32x3", "simt", "bf16x3", "fp16x3"])
+@pytest.mark.parametrize("shape", [(1, 4, 2, 3), (2, 64, 4, 3), (64, 8, 32, 5), (128, 32, 64, 2), (256, 64, 1024, 1)],
+                         ids=str)
+def test_operand_preparation_at_8_byte_starts(tn, engine, shape):
+    """Operands that start on 8 but not on 16 bytes, and element counts that no
+    16-byte load divides; two calls in a row with a larger one between them
+    (the scratch is kept between calls)."""
+    import torch
+    M, N, K, P = shape
+    rng = np.random.default_rng(M + N + K + P)
+    A, B = ((rng.normal(size=s) + 1j * rng.normal(size=s)).astype(np.complex64) for s in ((P, M, K), (P, K, N)))
+    ref = A.astype(np.complex128) @ B.astype(np.complex128)
+    dev = []
+    for X in (A, B):
+        buf = torch.zeros(X.size + 1, dtype=torch.complex64, device="cuda")
+        dev.append(buf[1:].view(X.shape))
+        dev[-1].copy_(torch.from_numpy(X))
+    c = torch.full((P, M, N), float("nan"), dtype=torch.complex64, device="cuda")
+    big = [torch.ones(s, dtype=torch.complex64, device="cuda") for s in ((1, 512, 512), (1, 512, 512), (1, 512, 512))]
+    for _ in range(2):
+        c.fill_(float("nan"))
+        tn.tn_gemm_c64(dev[0], dev[1], c, engine=engine, pair=1)
+        got = c.cpu().numpy()
+        assert np.linalg.norm(got - ref) <= (1e-4 if engine == 3 else 1e-5) * np.linalg.norm(ref)
+        tn.tn_gemm_c64(*big, engine=engine, pair=1)
+        assert float((big[2] - 512).abs().max()) <= 512 * (1e-4 if engine == 3 else 1e-5)
