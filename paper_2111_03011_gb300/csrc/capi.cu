@@ -664,6 +664,11 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
       gp.amax = scale_ptr(p, x.max_slot);
       gp.pair = P.gemm_pair < 0 ? -1 : x.pair;
       gp.tile_cap = x.tile_cap;
+      if (x.grp_fold > 0) {
+        gp.grp = p->d_meta + x.grp_off;
+        gp.grp_fold = x.grp_fold;
+        gp.n_groups = x.n_groups;
+      }
       e = x.kind == tn::ST_GEMM_SIMT ? tn::launch_gemm_simt(gp, st) : tn::launch_gemm_tc(gp, p->d_status, st);
       break;
     }

@@ -191,13 +191,52 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
       : "r"(taddr));
 }
 
+// Writing a tile out.  A drain warp holds 32 rows, one per lane; stored from
+// there, every 16-byte store instruction touches 32 rows and writes half a sector
+// of each, and the load/store unit's 32 lines per instruction cap the kernel
+// at 2.4 TB/s of output.  The warp therefore turns 32 rows x 16 columns at a
+// time through its own 2 KB of shared memory (16-byte pieces, XOR-swizzled: no
+// bank conflicts either way) and stores 8 rows x 64 bytes per instruction.
+// 2^27 outputs from K = 16 (BF16x3): 453 -> 254 us, 4.2 TB/s of output; 2^25 x
+// 2^13 x 2^9: 4.22 -> 3.53 ms, as the drain warps leave the MMAs waiting less.
+constexpr int OUT_BYTES = 32 * 64;
+
+// (The lane is read afresh and the stage's address passed as 32 bits so that
+// nothing of this stays in registers beside the running sums.)
+__device__ __forceinline__ void store_piece(uint32_t stage, const float* w, float* dst, int64_t pitch, int rows) {
+  uint32_t lane;
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  const uint32_t wr = stage + lane * 64, xw = (lane >> 1) & 3;
+  __syncwarp();                              // the previous piece has been read
+#pragma unroll
+  for (uint32_t q = 0; q < 4; ++q)
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(wr + ((q ^ xw) << 4)), "f"(w[4 * q]),
+                 "f"(w[4 * q + 1]), "f"(w[4 * q + 2]), "f"(w[4 * q + 3])
+                 : "memory");
+  __syncwarp();
+  const uint32_t r0 = lane >> 2, q = lane & 3;
+  const uint32_t rd = stage + r0 * 64 + ((q ^ ((r0 >> 1) & 3)) << 4);   // rows 8 apart share the XOR
+  float* p = dst + r0 * pitch + 4 * q;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(rd + 512u * i)
+                 : "memory");
+    if ((int)r0 + 8 * i < rows) *(float4*)p = v;
+    p += 8 * pitch;
+  }
+}
+
 template <int BN, int STAGES, int KB>
 struct Layout {
   static constexpr int A_BYTES = BM * KB;              // one 128-row tile, KB bytes of K per row
   static constexpr int B_BYTES = BN * KB;              // one BN-row tile
   static constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;  // A hi, A lo, B hi, B lo
   static constexpr int DATA = STAGES * STAGE;
-  static constexpr int TOTAL = DATA + 1024 /*align*/ + 256 /*barriers*/;
+  static constexpr int OUT = (BN >= 32 ? 8 : 4) * OUT_BYTES;   // a staging tile per active drain warp
+  static constexpr int TOTAL = DATA + 1024 /*align*/ + 256 /*barriers*/ + OUT;
   static_assert(TOTAL <= 232448, "shared memory per CTA");
   static_assert(2 * STAGES + 8 <= 32, "barrier area");
   // two chunk buffers of BN fp32 columns (ping-pong), a power of two >= 32
@@ -207,36 +246,73 @@ struct Layout {
 // Tile order: groups of GROUP_M m-tiles; inside a group n-tiles and (when A is
 // shared by every pattern) patterns vary before the next group, so the A rows
 // of a group and the B tiles of a wave stay in L2.
-constexpr int64_t GROUP_M = 8;
+//
+// Pattern groups (grp != nullptr): patterns that read the same A pattern, in a
+// table of n_groups x fold pattern ids (kNoPattern: none; padded to an even
+// count), one tile covering a group's columns side by side; then per group the run of groups with that A
+// pattern (first group, count).  Inside a run the order is that of a shared A:
+// m-groups outside, the run's groups inside.  1,024 patterns of 2^11 x 2^6 x
+// 2^11 on 64 A patterns (3xTF32) took 12.0 ms one by one, re-reading 67 MB of A
+// for each 128-column tile, and take 8.4 ms (262 TFLOP/s) in pairs; 92 patterns
+// of 2^13 x 2^5 x 2^9 on 8 (FP16x3) 424 -> 274 us.
+constexpr uint32_t GROUP_M = 8;
+constexpr uint32_t kNoPattern = 0xffffffffu;
 
-__device__ __forceinline__ void tile_coords(int64_t t, int64_t tilesM, int64_t tilesN, int64_t PC, bool a_shared,
-                                            int64_t& pc, int64_t& tm, int64_t& tn) {
-  const int64_t P_in = a_shared ? PC : 1;
-  int64_t outer = 0;
-  if (!a_shared) {
-    outer = t / (tilesM * tilesN);
-    t -= outer * tilesM * tilesN;
+struct TileGrid {
+  uint32_t tilesM, tilesN, groups;           // groups: pattern groups (patterns without folding)
+  int fold, br_log2;                         // patterns per tile; log2 of a pattern's B rows in the tile
+  int a_shared;
+  const uint32_t* grp;                       // or nullptr
+  uint32_t n_tiles;
+};
+
+__device__ __forceinline__ void tile_coords(const TileGrid& g, uint32_t t, uint32_t& pg, uint32_t& tm, uint32_t& tn) {
+  uint32_t mg, r;
+  if (g.grp) {
+    const uint32_t gm = min(GROUP_M, g.tilesM), mgroups = g.tilesM / gm;   // powers of two
+    const uint32_t u = t / (gm * g.tilesN);
+    r = t - u * gm * g.tilesN;
+    const uint2 run = __ldg((const uint2*)(g.grp + ((g.groups * (uint32_t)g.fold + 1) & ~1u)) + u / mgroups);
+    const uint32_t w = u - run.x * mgroups;
+    mg = w / run.y;
+    pg = run.x + w - mg * run.y;
+    tn = r / gm;
+    tm = mg * GROUP_M + r - tn * gm;
+    return;
   }
-  const int64_t per_full = GROUP_M * tilesN * P_in;
-  const int64_t mg = t / per_full;
-  int64_t r = t - mg * per_full;
-  const int64_t gm = min(GROUP_M, tilesM - mg * GROUP_M);
-  const int64_t mi = r % gm;
-  r /= gm;
-  tn = r % tilesN;
-  const int64_t pin = r / tilesN;
-  tm = mg * GROUP_M + mi;
-  pc = a_shared ? pin : outer;
+  uint32_t outer = 0;
+  if (!g.a_shared) {
+    outer = t / (g.tilesM * g.tilesN);
+    t -= outer * g.tilesM * g.tilesN;
+  }
+  const uint32_t per_full = GROUP_M * g.tilesN * (g.a_shared ? g.groups : 1);
+  mg = t / per_full;
+  r = t - mg * per_full;
+  const uint32_t gm = min(GROUP_M, g.tilesM - mg * GROUP_M);
+  const uint32_t q = r / gm, pin = q / g.tilesN;
+  tm = mg * GROUP_M + r - q * gm;
+  tn = q - pin * g.tilesN;
+  pg = g.a_shared ? pin : outer;
+}
+
+// Pattern f of group pg, or -1
+__device__ __forceinline__ int64_t tile_pattern(const TileGrid& g, uint32_t pg, int f, int64_t PC) {
+  if (g.grp) {
+    const uint32_t v = __ldg(g.grp + pg * (uint32_t)g.fold + f);
+    return v == kNoPattern ? -1 : (int64_t)v;
+  }
+  const int64_t pc = (int64_t)pg * g.fold + f;
+  return pc < PC ? pc : -1;
 }
 
 template <int BN, int STAGES, int FMT>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmAlo,
               const __grid_constant__ CUtensorMap tmBhi, const __grid_constant__ CUtensorMap tmBlo,
-              float* __restrict__ C, int64_t M, int64_t N2, int64_t K2, int64_t tilesM, int64_t tilesN, int64_t PC,
-              int64_t PCg, int fold, const uint32_t* __restrict__ mapA, const uint32_t* __restrict__ mapB,
-              int mapA_mode, int mapB_mode, const unsigned int* scaleA, const unsigned int* scaleB,
-              unsigned int* amax_out, unsigned int* status) {
+              float* __restrict__ C, int64_t M, int64_t N2, int64_t K2, int64_t PC,
+              const __grid_constant__ TileGrid grid, const uint32_t* __restrict__ mapA,
+              const uint32_t* __restrict__ mapB, int mapA_mode, int mapB_mode, const unsigned int* scaleA,
+              const unsigned int* scaleB, unsigned int* amax_out, unsigned int* status, int vec) {
   constexpr int KB = kb_bytes(BN, FMT);
   constexpr int CH = chunk_bytes(FMT) / KB;   // k-blocks per chunk
   using Lay = Layout<BN, STAGES, KB>;
@@ -253,20 +329,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   unsigned int* s_amax = (unsigned int*)(bars + 2 * STAGES + 7);   // CTA maximum of its output tiles
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool a_shared = mapA_mode == 1 && PC > 1;
-  const int64_t n_tiles = tilesM * tilesN * PCg;
-  const int br = BN / fold;                 // B rows per pattern box (2N when folded)
+  const uint32_t n_tiles = grid.n_tiles;
+  const int fold = grid.fold;
+  const int br = 1 << grid.br_log2;         // B rows per pattern box (2N when folded)
   constexpr bool H16 = FMT != 0;
   constexpr int BKE = KB / (H16 ? 2 : 4);   // K elements per k-block
   constexpr int KK = KBlock<KB>::KK;
   const int nkb = (int)((K2 + BKE - 1) / BKE);
   const int nch = (nkb + CH - 1) / CH;
-  // tile t -> first pattern pc0 of its group, m-tile, n-tile
-  auto coords = [&](int64_t t, int64_t& pc0, int64_t& tm, int64_t& tn_) {
-    int64_t pg;
-    tile_coords(t, tilesM, tilesN, PCg, a_shared, pg, tm, tn_);
-    pc0 = pg * fold;
-  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -297,9 +367,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       uint32_t it = 0;          // k-blocks issued by this CTA (all tiles)
       bool ok = true;
-      for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-        int64_t pc0, tm, tn_;
-        coords(t, pc0, tm, tn_);
+      for (uint32_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        uint32_t pg, tm, tn_;
+        tile_coords(grid, t, pg, tm, tn_);
+        const int64_t pc0 = tile_pattern(grid, pg, 0, PC);
         const int64_t pa = mapA_mode == 0 ? pc0 : (mapA_mode == 1 ? 0 : (int64_t)mapA[pc0]);
         for (int kb = 0; kb < nkb; ++kb) {
           const int s = (int)(it % STAGES);
@@ -310,9 +381,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           tma_load_3d(st, &tmAhi, &full[s], kb * BKE, (int)(tm * BM), (int)pa);
           tma_load_3d(st + Lay::A_BYTES, &tmAlo, &full[s], kb * BKE, (int)(tm * BM), (int)pa);
           for (int f = 0; f < fold; ++f) {
-            // a pattern past the last one loads pattern PC - 1 again: its
-            // columns are computed but never stored
-            const int64_t pcf = pc0 + f < PC ? pc0 + f : PC - 1;
+            // where a group has no further pattern its first is loaded
+            // again: those columns are computed but never stored
+            int64_t pcf = f ? tile_pattern(grid, pg, f, PC) : pc0;
+            if (pcf < 0) pcf = pc0;
             const int64_t pb = mapB_mode == 0 ? pcf : (mapB_mode == 1 ? 0 : (int64_t)mapB[pcf]);
             uint8_t* sb = st + 2 * Lay::A_BYTES + f * br * KB;
             tma_load_3d(sb, &tmBhi, &full[s], kb * BKE, (int)(tn_ * br), (int)pb);
@@ -332,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t idesc = idesc_mma<BN, FMT>();
       uint32_t it = 0, cc = 0;   // k-blocks and chunks consumed by this CTA (all tiles)
       bool ok = true, issued = false;
-      for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+      for (uint32_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
         for (int kb = 0; kb < nkb; ++kb) {
           // chunk cc accumulates in TMEM buffer b = cc & 1 from zero
           const int s = (int)(it % STAGES);
@@ -386,15 +458,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool active = BN >= 32 || half == 0;
     const int col0 = BN >= 32 ? half * NCOL : 0;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+    const uint32_t stage = smem_u32(smem + Lay::DATA + 256 + warp * OUT_BYTES);   // used by active warps only
     // FP16 engine: undo the operands' power-of-two scales (two exact multiplies)
     const float ua = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleA)) : 1.0f;
     const float ub = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleB)) : 1.0f;
     float tmax = 0.0f;
     uint32_t cc = 0;
     bool ok = true;
-    for (int64_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-      int64_t pc0, tm, tn_;
-      coords(t, pc0, tm, tn_);
+    for (uint32_t t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+      uint32_t pg, tm, tn_;
+      tile_coords(grid, t, pg, tm, tn_);
       float acc[NCOL];
 #pragma unroll
       for (int e = 0; e < NCOL; ++e) acc[e] = 0.0f;
@@ -428,32 +501,31 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok || !active) continue;
       // the tile's rows go out from registers while the MMAs of the next
       // tile fill the (now drained) TMEM buffers
-      const int64_t row = tm * BM + q * 32 + lane;
-      if (row >= M) continue;
+      const int64_t row0 = (int64_t)tm * BM + q * 32;
+      const int rows = (int)min((int64_t)32, M - row0);
+      if (rows <= 0) continue;
+      if (amax_out) {
+        // rows past M and columns past 2N are zero, repeated patterns repeat
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) tmax = fmaxf(tmax, fabsf(acc[e]));
+      }
 #pragma unroll
       for (int pp = 0; pp < NPIECE; ++pp) {
         const int cl = col0 + 16 * pp;             // column within the tile
-        const int f = cl / br;                     // pattern of the fold
-        const int64_t pc = pc0 + f;
-        const int64_t col = tn_ * br + (cl - f * br);
-        if (pc >= PC) continue;
-        float* crow = C + (pc * M + row) * N2;
+        const int f = cl >> grid.br_log2;          // pattern of the fold
+        const int64_t pc = tile_pattern(grid, pg, f, PC);
+        const int64_t col = ((int64_t)tn_ << grid.br_log2) + (cl & (br - 1));
+        if (pc < 0) continue;
+        float* dst = C + (pc * M + row0) * N2 + col;
         float w[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
-        if (amax_out) {
+        if (vec && col + 16 <= N2) {
+          store_piece(stage, w, dst, N2, rows);
+        } else if (lane < rows) {
 #pragma unroll
           for (int e = 0; e < 16; ++e)
-            if (col + e < N2) tmax = fmaxf(tmax, fabsf(acc[16 * pp + e]));
-        }
-        if (col + 16 <= N2) {
-          float4* dst = (float4*)(crow + col);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) dst[e] = make_float4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (col + e < N2) crow[col + e] = w[e];
+            if (col + e < N2) dst[lane * N2 + e] = w[e];
         }
       }
     }
@@ -556,7 +628,7 @@ struct LayoutPair {
   static constexpr int B_BYTES = 128 * KB;        // this CTA's half of the 256-row B tile
   static constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;
   static constexpr int DATA = STAGES * STAGE;
-  static constexpr int TOTAL = DATA + 1024 + 256;
+  static constexpr int TOTAL = DATA + 1024 + 256 + 8 * OUT_BYTES;
   static_assert(TOTAL <= 232448, "shared memory per CTA");
   static_assert(2 * STAGES + 8 <= 32, "barrier area");
   static constexpr uint32_t TMEM_COLS = 512;     // two chunk buffers of 256 fp32 columns
@@ -573,10 +645,10 @@ template <int STAGES, int FMT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_gemm_tc_pair(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmAlo,
                    const __grid_constant__ CUtensorMap tmBhi, const __grid_constant__ CUtensorMap tmBlo,
-                   float* __restrict__ C, int64_t M, int64_t N2, int64_t K2, int64_t tilesM, int64_t tilesN,
-                   int64_t PC, int64_t PCg, int fold, const uint32_t* __restrict__ mapA,
-                   const uint32_t* __restrict__ mapB, int mapA_mode, int mapB_mode, const unsigned int* scaleA,
-                   const unsigned int* scaleB, unsigned int* amax_out, unsigned int* status) {
+                   float* __restrict__ C, int64_t M, int64_t N2, int64_t K2, int64_t PC,
+                   const __grid_constant__ TileGrid grid, const uint32_t* __restrict__ mapA, const uint32_t* __restrict__ mapB, int mapA_mode,
+                   int mapB_mode, const unsigned int* scaleA, const unsigned int* scaleB, unsigned int* amax_out,
+                   unsigned int* status, int vec) {
   static_assert(FMT == 1 || FMT == 2, "pair MMAs use kind::f16 operands");
   constexpr int BN = 256;
   using Lay = LayoutPair<STAGES>;
@@ -596,21 +668,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
-  const int64_t cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-  const bool a_shared = mapA_mode == 1 && PC > 1;
-  const int64_t n_tiles = tilesM * tilesN * PCg;
-  const int br = BN / fold;                 // B rows per pattern box (2N when folded)
+  const uint32_t cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
+  const uint32_t n_tiles = grid.n_tiles;
+  const int fold = grid.fold;
+  const int br = 1 << grid.br_log2;         // B rows per pattern box (2N when folded)
   const int half_boxes = fold >= 2 ? fold / 2 : 1;   // B boxes this CTA loads per stage
   const int box_rows = fold >= 2 ? br : 128;
   constexpr int BKE = KB / 2;               // K elements (16-bit) per k-block
   constexpr int CH = chunk_bytes(FMT) / KB, KK = KBlock<KB>::KK;
   const int nkb = (int)((K2 + BKE - 1) / BKE);
   const int nch = (nkb + CH - 1) / CH;
-  auto coords = [&](int64_t t, int64_t& pc0, int64_t& tm, int64_t& tn_) {
-    int64_t pg;
-    tile_coords(t, tilesM, tilesN, PCg, a_shared, pg, tm, tn_);
-    pc0 = pg * fold;
-  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -642,9 +709,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int64_t t = cluster; t < n_tiles && ok; t += n_clusters) {
-        int64_t pc0, tm, tn_;
-        coords(t, pc0, tm, tn_);
+      for (uint32_t t = cluster; t < n_tiles && ok; t += n_clusters) {
+        uint32_t pg, tm, tn_;
+        tile_coords(grid, t, pg, tm, tn_);
+        const int64_t pc0 = tile_pattern(grid, pg, 0, PC);
         const int64_t pa = mapA_mode == 0 ? pc0 : (mapA_mode == 1 ? 0 : (int64_t)mapA[pc0]);
         const int row0 = (int)(tm * 2 * BM + rank * BM);
         for (int kb = 0; kb < nkb; ++kb) {
@@ -660,8 +728,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             int64_t pcf = pc0;
             int nrow = (int)(tn_ * BN + rank * 128);
             if (fold >= 2) {
-              const int f = (int)rank * half_boxes + h;
-              pcf = pc0 + f < PC ? pc0 + f : PC - 1;
+              pcf = tile_pattern(grid, pg, (int)rank * half_boxes + h, PC);
+              if (pcf < 0) pcf = pc0;
               nrow = 0;
             }
             const int64_t pb = mapB_mode == 0 ? pcf : (mapB_mode == 1 ? 0 : (int64_t)mapB[pcf]);
@@ -691,7 +759,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const uint32_t idesc = idesc_pair<FMT>();
       uint32_t it = 0, cc = 0;
       bool ok = true;
-      for (int64_t t = cluster; t < n_tiles && ok; t += n_clusters) {
+      for (uint32_t t = cluster; t < n_tiles && ok; t += n_clusters) {
         for (int kb = 0; kb < nkb; ++kb) {
           const int s = (int)(it % STAGES);
           const uint32_t r = it / STAGES;
@@ -736,6 +804,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int q = warp & 3, half = warp >> 2;
     const int col0 = half * NCOL;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+    const uint32_t stage = smem_u32(smem + Lay::DATA + 256 + warp * OUT_BYTES);
     const float ua = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleA)) : 1.0f;
     const float ub = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleB)) : 1.0f;
     // the leader's release barriers: acce[b] sits 8 bytes past acce[0] there
@@ -745,9 +814,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     float tmax = 0.0f;
     uint32_t cc = 0;
     bool ok = true;
-    for (int64_t t = cluster; t < n_tiles && ok; t += n_clusters) {
-      int64_t pc0, tm, tn_;
-      coords(t, pc0, tm, tn_);
+    for (uint32_t t = cluster; t < n_tiles && ok; t += n_clusters) {
+      uint32_t pg, tm, tn_;
+      tile_coords(grid, t, pg, tm, tn_);
       float acc[NCOL];
 #pragma unroll
       for (int e = 0; e < NCOL; ++e) acc[e] = 0.0f;
@@ -775,32 +844,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         ++cc;
       }
       if (!ok) continue;
-      const int64_t row = tm * 2 * BM + (int64_t)rank * BM + q * 32 + lane;
-      if (row >= M) continue;
+      const int64_t row0 = (int64_t)tm * 2 * BM + (int64_t)rank * BM + q * 32;
+      const int rows = (int)min((int64_t)32, M - row0);
+      if (rows <= 0) continue;
+      if (amax_out) {
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) tmax = fmaxf(tmax, fabsf(acc[e]));
+      }
 #pragma unroll
       for (int pp = 0; pp < NPIECE; ++pp) {
         const int cl = col0 + 16 * pp;
-        const int f = cl / br;
-        const int64_t pc = pc0 + f;
-        const int64_t col = tn_ * br + (cl - f * br);
-        if (pc >= PC) continue;
-        float* crow = C + (pc * M + row) * N2;
+        const int f = cl >> grid.br_log2;
+        const int64_t pc = tile_pattern(grid, pg, f, PC);
+        const int64_t col = ((int64_t)tn_ << grid.br_log2) + (cl & (br - 1));
+        if (pc < 0) continue;
+        float* dst = C + (pc * M + row0) * N2 + col;
         float w[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
-        if (amax_out) {
+        if (vec && col + 16 <= N2) {
+          store_piece(stage, w, dst, N2, rows);
+        } else if (lane < rows) {
 #pragma unroll
           for (int e = 0; e < 16; ++e)
-            if (col + e < N2) tmax = fmaxf(tmax, fabsf(acc[16 * pp + e]));
-        }
-        if (col + 16 <= N2) {
-          float4* dst = (float4*)(crow + col);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) dst[e] = make_float4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (col + e < N2) crow[col + e] = w[e];
+            if (col + e < N2) dst[lane * N2 + e] = w[e];
         }
       }
     }
@@ -884,7 +951,8 @@ static cudaError_t run(const GemmParams& p, int fold, unsigned int* status, cuda
   using Lay = Layout<BN, STAGES, KB>;
   const int64_t K2 = 2 * p.K, N2 = 2 * p.N;
   const int br = BN / fold;
-  if (fold > 1 && (br != N2 || br < 16 || p.mapA_mode != 1)) return cudaErrorInvalidValue;
+  const uint32_t* grp = p.grp_fold == fold ? p.grp : nullptr;
+  if (fold > 1 && (br != N2 || br < 16 || (p.mapA_mode != 1 && !grp))) return cudaErrorInvalidValue;
   const uint32_t BKE = KB / (FMT ? 2 : 4);
   const int64_t es = FMT ? 2 : 4;
   // A: hi plane then lo plane, each [PA][M][2K]; B: hi plane then lo plane, each [PB][2N][2K]
@@ -898,18 +966,22 @@ static cudaError_t run(const GemmParams& p, int fold, unsigned int* status, cuda
   if (!encode3d(&tbh, bhi, (uint64_t)K2, (uint64_t)N2, (uint64_t)p.PB, BKE, br, FMT, KB)) return cudaErrorInvalidValue;
   if (!encode3d(&tbl, blo, (uint64_t)K2, (uint64_t)N2, (uint64_t)p.PB, BKE, br, FMT, KB)) return cudaErrorInvalidValue;
   const int64_t tilesM = (p.M + BM - 1) / BM, tilesN = fold > 1 ? 1 : (N2 + BN - 1) / BN;
-  const int64_t PCg = (p.PC + fold - 1) / fold;
+  const int64_t PCg = grp ? p.n_groups : (p.PC + fold - 1) / fold;
   const int64_t n_tiles = tilesM * tilesN * PCg;
   if (n_tiles <= 0) return cudaSuccess;
+  if (n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  TileGrid grid{(uint32_t)tilesM, (uint32_t)tilesN, (uint32_t)PCg, fold, 0, p.mapA_mode == 1 && p.PC > 1, grp,
+                (uint32_t)n_tiles};
+  while ((1 << grid.br_log2) < br) ++grid.br_log2;
   if (p.prepare) {
     const cudaError_t e = set_attr<BN, STAGES, FMT>();
     if (e != cudaSuccess) return e;
   }
   // persistent: at most one CTA per SM (the pipeline's shared memory allows one)
-  const int64_t grid = std::min<int64_t>(n_tiles, sm_count());
-  k_gemm_tc<BN, STAGES, FMT><<<(unsigned)grid, kThreads, Lay::TOTAL, s>>>(
-      tah, tal, tbh, tbl, (float*)p.C, p.M, N2, K2, tilesM, tilesN, p.PC, PCg, fold, p.mapA, p.mapB, p.mapA_mode,
-      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status);
+  const int64_t ctas = std::min<int64_t>(n_tiles, sm_count());
+  k_gemm_tc<BN, STAGES, FMT><<<(unsigned)ctas, kThreads, Lay::TOTAL, s>>>(
+      tah, tal, tbh, tbl, (float*)p.C, p.M, N2, K2, p.PC, grid, p.mapA, p.mapB, p.mapA_mode,
+      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status, (uintptr_t)p.C % 16 == 0);
   return cudaGetLastError();
 }
 
@@ -928,7 +1000,8 @@ static cudaError_t run_pair(const GemmParams& p, int fold, unsigned int* status,
   constexpr int BN = 256, KB = Lay::KB;
   const int64_t K2 = 2 * p.K, N2 = 2 * p.N;
   const int br = BN / fold;
-  if (fold > 1 && (br != N2 || br < 16 || p.mapA_mode != 1 || fold % 2)) return cudaErrorInvalidValue;
+  const uint32_t* grp = p.grp_fold == fold ? p.grp : nullptr;
+  if (fold > 1 && (br != N2 || br < 16 || (p.mapA_mode != 1 && !grp) || fold % 2)) return cudaErrorInvalidValue;
   const uint32_t BKE = KB / 2;
   const int64_t es = 2;
   const char* ahi = (const char*)p.A;
@@ -944,17 +1017,21 @@ static cudaError_t run_pair(const GemmParams& p, int fold, unsigned int* status,
   if (!encode3d(&tbl, blo, (uint64_t)K2, (uint64_t)N2, (uint64_t)p.PB, BKE, box_rows, FMT, KB))
     return cudaErrorInvalidValue;
   const int64_t tilesM = (p.M + 2 * BM - 1) / (2 * BM), tilesN = fold > 1 ? 1 : (N2 + BN - 1) / BN;
-  const int64_t PCg = (p.PC + fold - 1) / fold;
+  const int64_t PCg = grp ? p.n_groups : (p.PC + fold - 1) / fold;
   const int64_t n_tiles = tilesM * tilesN * PCg;
   if (n_tiles <= 0) return cudaSuccess;
+  if (n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  TileGrid grid{(uint32_t)tilesM, (uint32_t)tilesN, (uint32_t)PCg, fold, 0, p.mapA_mode == 1 && p.PC > 1, grp,
+                (uint32_t)n_tiles};
+  while ((1 << grid.br_log2) < br) ++grid.br_log2;
   if (p.prepare) {
     const cudaError_t e = set_attr_pair<FMT>();
     if (e != cudaSuccess) return e;
   }
   const int64_t clusters = std::min<int64_t>(n_tiles, sm_count() / 2);
   k_gemm_tc_pair<kPairStages, FMT><<<(unsigned)(2 * clusters), kThreads, Lay::TOTAL, s>>>(
-      tah, tal, tbh, tbl, (float*)p.C, p.M, N2, K2, tilesM, tilesN, p.PC, PCg, fold, p.mapA, p.mapB, p.mapA_mode,
-      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status);
+      tah, tal, tbh, tbl, (float*)p.C, p.M, N2, K2, p.PC, grid, p.mapA, p.mapB, p.mapA_mode,
+      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status, (uintptr_t)p.C % 16 == 0);
   return cudaGetLastError();
 }
 
@@ -989,8 +1066,27 @@ GemmTile gemm_tc_tile(const GemmParams& p) {
 namespace tc {
 
 template <int FMT>
-static cudaError_t dispatch(const GemmParams& p, unsigned int* status, cudaStream_t s) {
-  const GemmTile t = gemm_tc_tile(p);
+static cudaError_t dispatch(const GemmParams& q, unsigned int* status, cudaStream_t s) {
+  GemmParams p = q;
+  // Every pattern has its own A and all share B: one GEMM over the PC x M rows,
+  // which lie one after another in A's planes and in C.  Small M then fills the
+  // 128-row tiles, and a wave's row tiles share each B tile.
+  if (p.mapA_mode == 0 && p.mapB_mode == 1 && p.PA == p.PC && p.PC > 1 && p.PC * p.M <= 0x7fffffffLL) {
+    p.M *= p.PC;
+    p.PA = p.PC = 1;
+    p.mapA_mode = 1;
+  }
+  GemmTile t = gemm_tc_tile(p);
+  // Groups of patterns with one A pattern, where a table of them is given, for
+  // the widest tiles; other tile choices take the patterns one by one.
+  if (p.grp && p.tile_cap >= 256) {
+    t.fold = p.grp_fold;
+    t.bn = (int)std::min<int64_t>(256, 2 * p.N * p.grp_fold);
+    t.paired = FMT != 0 && t.bn == 256 && p.M >= 2 * BM && p.pair >= 0;
+  } else {
+    p.grp = nullptr;
+    p.grp_fold = 0;
+  }
   const int fold = t.fold;
   if (t.bn == 16) return run<16, kb_stages(16, kb_bytes(16, FMT)), FMT>(p, fold, status, s);
   if (t.bn == 32) return run<32, kb_stages(32, kb_bytes(32, FMT)), FMT>(p, fold, status, s);

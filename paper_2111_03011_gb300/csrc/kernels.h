@@ -86,6 +86,10 @@ struct GemmParams {
   unsigned int* amax;    // non-null: atomicMax of the output's max |re|, |im| (fp32 bits)
   int pair = 0;          // 0: CTA-pair 256 x 256 tiles where they apply (16-bit, M >= 256); -1: one-CTA tiles
   int tile_cap = 256;    // widest tile the dispatch may pick, real columns (16..256)
+  // table of pattern groups (see gemm_tc.cu) of grp_fold patterns, or null
+  const uint32_t* grp = nullptr;
+  int grp_fold = 0;
+  int64_t n_groups = 0;
   int prepare = 0;       // 1: set the launched kernel's attributes first (no plan upload did)
 };
 

@@ -919,10 +919,34 @@ static void add_permute(Plan& plan, const VTensor& X, const std::vector<int>& ta
   plan.steps.push_back(s);
 }
 
+// Patterns of a tensor-core GEMM grouped by the A pattern they read (mapA:
+// a table): the group table that gemm_tc.cu describes, for groups of `fold`.
+static std::vector<uint32_t> group_patterns(const std::vector<uint32_t>& mapA, int fold, int64_t& n_groups) {
+  std::vector<uint32_t> by(mapA.size());
+  for (size_t p = 0; p < by.size(); ++p) by[p] = (uint32_t)p;
+  std::stable_sort(by.begin(), by.end(), [&](uint32_t x, uint32_t y) { return mapA[x] < mapA[y]; });
+  std::vector<uint32_t> ids, runs;
+  for (size_t p = 0; p < by.size();) {
+    size_t e = p;
+    while (e < by.size() && mapA[by[e]] == mapA[by[p]]) ++e;
+    const uint32_t first = (uint32_t)(ids.size() / fold), count = (uint32_t)((e - p + fold - 1) / fold);
+    for (uint32_t i = 0; i < count * (uint32_t)fold; ++i) ids.push_back(p + i < e ? by[p + i] : 0xffffffffu);
+    for (uint32_t i = 0; i < count; ++i) {
+      runs.push_back(first);
+      runs.push_back(count);
+    }
+    p = e;
+  }
+  n_groups = (int64_t)(ids.size() / fold);
+  if (ids.size() % 2) ids.push_back(0xffffffffu);
+  ids.insert(ids.end(), runs.begin(), runs.end());
+  return ids;
+}
+
 // Modelled time of a contraction as split permute, B preparation and
 // tensor-core GEMM, to set against the direct form's (plan_direct).  Measured
 // on GB300: about 4 us per launch; the passes stream at 5 TB/s and a
-// GEMM writes C at 2.4 TB/s; it runs
+// GEMM writes C at 3.7 TB/s; it runs
 // its tiles of 128 rows x BN real columns in whole waves of 152, each SM at
 // its share of 280 (3xTF32) or 560 (16-bit) TFLOP/s for BN >= 256, where an
 // MMA narrower than 128 columns takes as long as one of 128.
@@ -939,7 +963,7 @@ double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, double a, d
   const double tile_flops = 8.0 * 128.0 * std::max(bn, 128.0) / 2.0 * std::ldexp(1.0, nk);
   const double mma = std::ceil(tiles / 152.0) * tile_flops * 152.0 / peak;
   const double plane = h16 ? 8.0 : 16.0;
-  const double gemm = std::max(mma, plane * a / 5.0e12 + 8.0 * c / 2.4e12);
+  const double gemm = std::max(mma, plane * a / 5.0e12 + 8.0 * c / 3.7e12);
   return gemm + (8.0 + plane) * a / 5.0e12 + (8.0 + 2.0 * plane) * b / 5.0e12 + 12e-6;
 }
 
@@ -1176,6 +1200,27 @@ static int layout_steps(Plan& plan, std::string& err) {
       g.nk = nk; g.nm = nm; g.nn = nn;
       g.mapA_mode = mapA_mode; g.mapA_off = mapA_off;
       g.mapB_mode = mapB_mode; g.mapB_off = mapB_off;
+      if (tc && mapA_mode == 2 && big.P < C.P && C.P < (1LL << 24)) {
+        // patterns with one A pattern side by side, up to 256 columns: the
+        // width with the least MMA time (a tile of 128 columns takes 0.77 of
+        // one of 256, narrower ones as long as one of 128)
+        const std::vector<uint32_t> ma(plan.meta.begin() + mapA_off, plan.meta.begin() + mapA_off + C.P);
+        double best = 1e300;
+        std::vector<uint32_t> tab;
+        for (int fold = 1; fold == 1 || ((2LL << nn) >= 16 && ((2LL << nn) * fold) <= 256); fold *= 2) {
+          int64_t ng = 0;
+          std::vector<uint32_t> t = group_patterns(ma, fold, ng);
+          const double cols = (double)(2LL << nn) * fold;
+          const double cost = (double)ng * (cols >= 256 ? cols / 256.0 : 0.77);
+          if (cost < best) {
+            best = cost;
+            tab.swap(t);
+            g.grp_fold = fold;
+            g.n_groups = ng;
+          }
+        }
+        g.grp_off = meta_push(plan, tab);
+      }
       g.macs = macs;
       g.bytes = 8.0 * (double)(vt_elems(big) + eC) + (double)bprep_bytes;
       const int st = (int)plan.steps.size();
@@ -1673,7 +1718,7 @@ std::string describe_plan(const Plan& plan, bool with_data) {
     for (int v = 0; v < 16; ++v) o << (v ? "," : "") << st.boffN[v];
     o << "],\"mapA\":[" << st.mapA_mode << "," << st.mapA_off << "],\"mapB\":[" << st.mapB_mode << ","
       << st.mapB_off << "],\"bk_off\":" << st.bk_off << ",\"bn_off\":" << st.bn_off << ",\"bprep_embed0\":" << st.bprep_embed0 << ",\"variant\":" << st.variant
-      << ",\"direct\":" << (st.direct ? 1 : 0);
+      << ",\"grp\":[" << st.grp_fold << "," << st.n_groups << "," << st.grp_off << "],\"direct\":" << (st.direct ? 1 : 0);
     if (st.direct) {
       const DirectPlan& d = st.dp;
       auto list = [&o](const char* name, const uint8_t* v, int n) {

@@ -128,6 +128,10 @@ struct Step {
   // not (-1), as chosen by a plan tuner (default: the dispatch rule's widest)
   int tile_cap = 256;
   int pair = 0;
+  // GEMM_TC with gathered A patterns: meta offset of the pattern groups' table
+  // (gemm_tc.cu), patterns per group (0: no table), number of groups
+  int64_t grp_off = 0, n_groups = 0;
+  int grp_fold = 0;
   int variant = 0;         // index of the chosen variant (0: default)
   // BPREP: gather tables bk[K], bn[N] in meta (uint32)
   int64_t bk_off = 0, bn_off = 0;
