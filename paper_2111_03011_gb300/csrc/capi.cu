@@ -298,7 +298,7 @@ static int plan_upload(tn_plan_t* p) {
   if (h) CUDA_TRY(cudaMemcpy(p->d_open, P.open_qubits.data(), h * sizeof(int), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMalloc(&p->d_status, sizeof(unsigned int)));
   CUDA_TRY(cudaMemset(p->d_status, 0, sizeof(unsigned int)));
-  const size_t n_static = P.scale_static.size(), n_slots = n_static + (size_t)P.n_scale_slots;
+  const size_t n_static = P.scale_static.size(), n_slots = n_static + (size_t)P.n_scale_slots * P.batch_max;
   if (n_slots > 0) {
     CUDA_TRY(cudaMalloc(&p->d_scale, n_slots * sizeof(unsigned int)));
     CUDA_TRY(cudaMemset(p->d_scale, 0, n_slots * sizeof(unsigned int)));
@@ -520,30 +520,59 @@ extern "C" int tn_head_set_fidelity(tn_head_t* h, double f) {
 
 // -------------------------------------------------------- slice execution
 
-static inline const float2* ref_ptr(const tn_plan_t* p, const tn::Ref& r, int64_t s) {
+// b: the pass's place in its chunk, which selects its copies of batched
+// buffers and of the scale slots
+static inline float2* buf_ptr(const tn_plan_t* p, const tn::Ref& r, int b) {
+  const tn::BufInfo& bi = p->P.bufs[r.id];
+  return (float2*)(p->d_arena + bi.off + (bi.batch ? b * p->P.batch_stride : 0));
+}
+
+static inline const float2* ref_ptr(const tn_plan_t* p, const tn::Ref& r, int64_t s, int b) {
   if (r.kind == 0) {
     const tn::LeafInfo& li = p->P.leaf_info[r.id];
     int64_t v = 0;
     for (size_t t = 0; t < li.var_slice_bits.size(); ++t) v |= ((s >> li.var_slice_bits[t]) & 1) << t;
     return p->d_leaves + li.off + v * li.size;
   }
-  return (const float2*)(p->d_arena + p->P.bufs[r.id].off);
-}
-
-static inline float2* buf_ptr(const tn_plan_t* p, const tn::Ref& r) {
-  return (float2*)(p->d_arena + p->P.bufs[r.id].off);
+  return buf_ptr(p, r, b);
 }
 
 // FP16x3 scale slot -> device address (static slots first, then the per-pass ones)
-static unsigned int* scale_ptr(const tn_plan_t* p, int slot) {
+static unsigned int* scale_ptr(const tn_plan_t* p, int slot, int b) {
   if (slot == -1) return nullptr;
   const int64_t n_static = (int64_t)p->P.scale_static.size();
-  return p->d_scale + (slot >= 0 ? n_static + slot : (int64_t)(-(slot + 2)));
+  return p->d_scale + (slot >= 0 ? n_static + (int64_t)b * p->P.n_scale_slots + slot : (int64_t)(-(slot + 2)));
+}
+
+// An operand of a batched launch: base address of batch element 0 and how the others follow.
+static const float2* batch_operand(const tn_plan_t* p, const tn::Ref& r, tn::BatchOperand& o) {
+  o = tn::BatchOperand();
+  if (r.kind == 1) {
+    o.stride = p->P.batch_stride / (int64_t)sizeof(float2);
+    return buf_ptr(p, r, 0);
+  }
+  const tn::LeafInfo& li = p->P.leaf_info[r.id];
+  o.var_size = li.size;
+  o.n_bits = (int)li.var_slice_bits.size();
+  for (int t = 0; t < o.n_bits; ++t) o.bits[t] = (uint8_t)li.var_slice_bits[t];
+  return p->d_leaves + li.off;
+}
+
+// Passes q0 .. q0 + n - 1 for a launch of them all.
+static void batch_range(const tn_plan_t* p, int64_t q0, int n, tn::BatchParams& q) {
+  q.n_batch = n;
+  q.q0 = q0;
+  q.ni = p->P.n_internal;
+  q.k = p->P.n_sliced;
+  q.amax_stride = p->P.n_scale_slots;
 }
 
 // Launch one step of the launch list for the full slice id s on stream st
-// (`side`: a B-prep beside a running GEMM, launched with one block per SM).
-static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaStream_t st, bool side) {
+// (`side`: a B-prep beside a running GEMM, launched with one block per SM); b is
+// the pass's place in its chunk.  n_batch > 1: a batched step, for the passes
+// q0 .. q0 + n_batch - 1 at once.
+static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaStream_t st, bool side, int b,
+                               int n_batch = 1, int64_t q0 = 0) {
   const tn::Plan& P = p->P;
   NvtxRange range(step_range_name(x.kind));
   cudaError_t e = cudaSuccess;
@@ -553,9 +582,9 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
         const tn::Ref &rx = x.dp.swap ? x.b : x.a, &ry = x.dp.swap ? x.a : x.b;
         tn::DirectParams dp{};
         tn::direct_fill(x.dp, x.PC, dp);
-        dp.X = ref_ptr(p, rx, s);
-        dp.Y = ref_ptr(p, ry, s);
-        dp.C = buf_ptr(p, x.c);
+        dp.X = ref_ptr(p, rx, s, b);
+        dp.Y = ref_ptr(p, ry, s, b);
+        dp.C = buf_ptr(p, x.c, b);
         dp.x_pstride = 1LL << (x.dp.swap ? x.rB : x.rA);
         dp.y_pstride = 1LL << (x.dp.swap ? x.rA : x.rB);
         dp.c_pstride = 1LL << x.rC;
@@ -564,14 +593,20 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
         dp.mapX_mode = x.dp.swap ? x.mapB_mode : x.mapA_mode;
         dp.mapY_mode = x.dp.swap ? x.mapA_mode : x.mapB_mode;
         dp.vec = 1;                      // buffers start on 256 bytes, rows pair up from even ones
-        dp.amax = scale_ptr(p, x.max_slot);
+        dp.amax = scale_ptr(p, x.max_slot, b);
+        if (n_batch > 1) {
+          batch_range(p, q0, n_batch, dp);
+          dp.X = batch_operand(p, rx, dp.bA);
+          dp.Y = batch_operand(p, ry, dp.bB);
+          batch_operand(p, x.c, dp.bC);
+        }
         e = tn::launch_direct(dp, x.dp.config, st);
         break;
       }
       tn::SmallParams sp;
-      sp.A = ref_ptr(p, x.a, s);
-      sp.B = ref_ptr(p, x.b, s);
-      sp.C = buf_ptr(p, x.c);
+      sp.A = ref_ptr(p, x.a, s, b);
+      sp.B = ref_ptr(p, x.b, s, b);
+      sp.C = buf_ptr(p, x.c, b);
       sp.a_pstride = 1LL << x.rA;
       sp.b_pstride = 1LL << x.rB;
       sp.c_pstride = 1LL << x.rC;
@@ -587,14 +622,20 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
       sp.mapB = p->d_meta + x.mapB_off;
       sp.mapA_mode = x.mapA_mode;
       sp.mapB_mode = x.mapB_mode;
-      sp.amax = scale_ptr(p, x.max_slot);
+      sp.amax = scale_ptr(p, x.max_slot, b);
+      if (n_batch > 1) {
+        batch_range(p, q0, n_batch, sp);
+        sp.A = batch_operand(p, x.a, sp.bA);
+        sp.B = batch_operand(p, x.b, sp.bB);
+        batch_operand(p, x.c, sp.bC);
+      }
       e = tn::launch_small(sp, st);
       break;
     }
     case tn::ST_PERMUTE: {
       tn::PermParams pp;
-      pp.in = ref_ptr(p, x.a, s);
-      pp.out = buf_ptr(p, x.c);
+      pp.in = ref_ptr(p, x.a, s, b);
+      pp.out = buf_ptr(p, x.c, b);
       pp.pstride = 1LL << x.rA;
       pp.P = x.PA;
       pp.t = x.t_bits;
@@ -603,7 +644,7 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
       std::memcpy(pp.rest_out, x.rest_out, sizeof(pp.rest_out));
       pp.tab = p->d_meta + x.tab_off;
       pp.split = x.split;
-      pp.scale = scale_ptr(p, x.slot);
+      pp.scale = scale_ptr(p, x.slot, b);
       pp.vec4 = x.vec4;
       e = tn::launch_permute(pp, st);
       break;
@@ -613,8 +654,8 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
       if (x.kind == tn::ST_BPREP_TC && !x.alts.empty() && (x.variant == 0) == (x.bprep_embed0 != 0)) {
         // the permute kernel onto [N][K] order, writing the real embedding
         tn::PermParams pp;
-        pp.in = ref_ptr(p, x.a, s);
-        pp.out = buf_ptr(p, x.c);
+        pp.in = ref_ptr(p, x.a, s, b);
+        pp.out = buf_ptr(p, x.c, b);
         pp.pstride = 1LL << x.rA;
         pp.P = x.PA;
         pp.t = x.t_bits;
@@ -623,14 +664,14 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
         std::memcpy(pp.rest_out, x.rest_out, sizeof(pp.rest_out));
         pp.tab = p->d_meta + x.tab_off;
         pp.split = 4 + x.h16;
-        pp.scale = scale_ptr(p, x.slot);
+        pp.scale = scale_ptr(p, x.slot, b);
         pp.embed_nk = x.nk;
         e = tn::launch_permute(pp, st);
         break;
       }
       tn::BPrepParams bp;
-      bp.B = ref_ptr(p, x.a, s);
-      bp.out = buf_ptr(p, x.c);
+      bp.B = ref_ptr(p, x.a, s, b);
+      bp.out = buf_ptr(p, x.c, b);
       bp.b_pstride = 1LL << x.rA;
       bp.PB = x.PA;
       bp.nk = x.nk;
@@ -638,16 +679,16 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
       bp.bk = p->d_meta + x.bk_off;
       bp.bn = p->d_meta + x.bn_off;
       bp.h16 = x.h16;
-      bp.scale = scale_ptr(p, x.slot);
+      bp.scale = scale_ptr(p, x.slot, b);
       e = x.kind == tn::ST_BPREP_C ? tn::launch_bprep_c(bp, st) : tn::launch_bprep_tc(bp, st, side);
       break;
     }
     case tn::ST_GEMM_SIMT:
     case tn::ST_GEMM_TC: {
       tn::GemmParams gp;
-      gp.A = ref_ptr(p, x.a, s);
-      gp.B = (const void*)ref_ptr(p, x.b, s);
-      gp.C = buf_ptr(p, x.c);
+      gp.A = ref_ptr(p, x.a, s, b);
+      gp.B = (const void*)ref_ptr(p, x.b, s, b);
+      gp.C = buf_ptr(p, x.c, b);
       gp.M = 1LL << x.nm;
       gp.N = 1LL << x.nn;
       gp.K = 1LL << x.nk;
@@ -659,9 +700,9 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
       gp.mapA_mode = x.mapA_mode;
       gp.mapB_mode = x.mapB_mode;
       gp.h16 = x.h16;
-      gp.scaleA = scale_ptr(p, x.slot);
-      gp.scaleB = scale_ptr(p, x.slotB);
-      gp.amax = scale_ptr(p, x.max_slot);
+      gp.scaleA = scale_ptr(p, x.slot, b);
+      gp.scaleB = scale_ptr(p, x.slotB, b);
+      gp.amax = scale_ptr(p, x.max_slot, b);
       gp.pair = P.gemm_pair < 0 ? -1 : x.pair;
       gp.tile_cap = x.tile_cap;
       if (x.grp_fold > 0) {
@@ -674,9 +715,9 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
     }
     case tn::ST_ABSMAX: {
       tn::AbsmaxParams ap;
-      ap.in = ref_ptr(p, x.a, s);
+      ap.in = ref_ptr(p, x.a, s, b);
       ap.n = x.PA << x.rA;
-      ap.out = scale_ptr(p, x.slot);
+      ap.out = scale_ptr(p, x.slot, b);
       e = tn::launch_absmax(ap, st);
       break;
     }
@@ -686,16 +727,31 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
   return e;
 }
 
+static tn::AccumParams accum_params(const tn_plan_t* p, double2* H) {
+  const tn::Plan& P = p->P;
+  tn::AccumParams ap;
+  ap.H = H;
+  ap.f_pstride = 1LL << P.fin.rF;
+  ap.L = (int64_t)P.tails_raw.size();
+  ap.h = (int)P.open_qubits.size();
+  ap.pidx = p->d_meta + P.fin.pidx_off;
+  for (int j = 0; j < ap.h && j < 32; ++j) ap.open_pos[j] = P.fin.open_pos[j];
+  return ap;
+}
+
 // One pass of the launch list for the full slice id s (user bits, then the
 // bits of automatically sliced edges).  With per-launch timing events (ev)
 // every step runs in order on st; otherwise a B-prep step with fork f is
 // launched on the plan's side stream just before step f (after everything
 // before f is done) and step f + ... waits for it right before the GEMM that
 // consumes its output.
-static int run_pass(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st, cudaEvent_t* ev) {
+// chunk_pass >= 0: this pass of a chunk, whose batched steps have run and whose
+// scale slots were zeroed; -1: the whole launch list.
+static int run_pass(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st, cudaEvent_t* ev, int chunk_pass = -1) {
   const tn::Plan& P = p->P;
   NvtxRange range("tn pass");
-  if (P.n_scale_slots > 0) {
+  const int b = std::max(chunk_pass, 0);
+  if (P.n_scale_slots > 0 && chunk_pass < 0) {
     cudaError_t e = cudaMemsetAsync(p->d_scale + P.scale_static.size(), 0,
                                     (size_t)P.n_scale_slots * sizeof(unsigned int), st);
     if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("scale reset: ") + cudaGetErrorString(e));
@@ -709,11 +765,15 @@ static int run_pass(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st, cudaEv
   int si = 0;
   for (const tn::Step& x : P.steps) {
     cudaError_t e = cudaSuccess;
+    if (chunk_pass >= 0 && x.batch) {
+      ++si;
+      continue;
+    }
     if (use_side && !p->forks_at[si].empty()) {
       e = cudaEventRecord(p->side_fork[si], st);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(p->side_stream, p->side_fork[si], 0);
       for (int j : p->forks_at[si]) {
-        if (e == cudaSuccess) e = launch_step(p, P.steps[j], s, p->side_stream, true);
+        if (e == cudaSuccess) e = launch_step(p, P.steps[j], s, p->side_stream, true, b);
         if (e == cudaSuccess) e = cudaEventRecord(p->side_join[j], p->side_stream);
         if (e == cudaSuccess) pending.push_back(j);
       }
@@ -728,7 +788,7 @@ static int run_pass(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st, cudaEv
       e = cudaStreamWaitEvent(st, p->side_join[si], 0);
       pending.erase(std::remove(pending.begin(), pending.end(), si), pending.end());
     } else {
-      e = launch_step(p, x, s, st, false);
+      e = launch_step(p, x, s, st, false, b);
     }
     if (e == cudaErrorInvalidValue && (x.kind < 0 || x.kind > tn::ST_ABSMAX)) {
       join_pending();
@@ -743,36 +803,78 @@ static int run_pass(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st, cudaEv
   }
   join_pending();
   if (ev) cudaEventRecord(ev[2 * si], st);
-  tn::AccumParams ap;
-  ap.F = ref_ptr(p, P.fin.ref, s);
-  ap.H = H;
-  ap.f_pstride = 1LL << P.fin.rF;
-  ap.L = (int64_t)P.tails_raw.size();
-  ap.h = (int)P.open_qubits.size();
-  ap.pidx = p->d_meta + P.fin.pidx_off;
-  for (int j = 0; j < ap.h && j < 32; ++j) ap.open_pos[j] = P.fin.open_pos[j];
+  tn::AccumParams ap = accum_params(p, H);
+  ap.F = ref_ptr(p, P.fin.ref, s, b);
   cudaError_t e = tn::launch_accum(ap, st);
   if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("accumulate launch: ") + cudaGetErrorString(e));
   if (ev) cudaEventRecord(ev[2 * si + 1], st);
   return TN_OK;
 }
 
-// User slice s: every value t of the automatically sliced edges, slice id
-// s | t << k, each pass accumulating into H.  *passes_done (if given) counts
-// the passes enqueued whole: a failing pass fails before its accumulation
-// launch, so exactly those passes reach H.
-static int run_slice(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st, int64_t* passes_done = nullptr) {
-  const int64_t ni = 1LL << p->P.n_internal;
-  for (int64_t t = 0; t < ni; ++t) {
-    if (passes_done) *passes_done = t;
-    if (tn::fault_slice(s, t))
-      return fail(TN_ERR_CUDA, "injected failure before pass " + std::to_string(t) + " of slice " + std::to_string(s) +
-                                   " (TN_FAULT_INJECT)");
-    int rc = run_pass(p, s | (t << p->P.n_sliced), H, st, nullptr);
-    if (rc) return rc;
+// Passes [q, q_end) of the plan (pass q: user slice q >> n_internal, value
+// q & (2^n_internal - 1) of the automatically sliced edges), each accumulating
+// into H, in chunks whose batched steps are launched for all their passes at
+// once.  *done (if given) receives the end of the passes enqueued whole: a
+// failing pass fails before its accumulation launch, so exactly those reach H.
+static int run_passes(tn_plan_t* p, int64_t q, int64_t q_end, double2* H, cudaStream_t st, int64_t* done = nullptr) {
+  const tn::Plan& P = p->P;
+  const int ni = P.n_internal;
+  auto slice_id = [&](int64_t x) { return (x >> ni) | ((x & ((1LL << ni) - 1)) << P.n_sliced); };
+  auto injected = [&](int64_t x) {
+    const int64_t s = x >> ni, t = x & ((1LL << ni) - 1);
+    if (!tn::fault_slice(s, t)) return (int)TN_OK;
+    return fail(TN_ERR_CUDA, "injected failure before pass " + std::to_string(t) + " of slice " + std::to_string(s) +
+                                 " (TN_FAULT_INJECT)");
+  };
+  bool all_batched = true;
+  for (const tn::Step& x : P.steps) all_batched = all_batched && x.batch;
+  if (done) *done = q;
+  while (q < q_end) {
+    const int n = (int)std::min<int64_t>(P.batch_max, q_end - q);
+    if (n == 1) {
+      if (int rc = injected(q)) return rc;
+      if (int rc = run_pass(p, slice_id(q), H, st, nullptr)) return rc;
+      ++q;
+      if (done) *done = q;
+      continue;
+    }
+    NvtxRange range("tn chunk");
+    if (P.n_scale_slots > 0) {
+      const cudaError_t e = cudaMemsetAsync(p->d_scale + P.scale_static.size(), 0,
+                                            (size_t)n * P.n_scale_slots * sizeof(unsigned int), st);
+      if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("scale reset: ") + cudaGetErrorString(e));
+    }
+    for (const tn::Step& x : P.steps) {
+      if (!x.batch) continue;
+      const cudaError_t e = launch_step(p, x, 0, st, false, 0, n, q);
+      if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
+    }
+    if (all_batched) {
+      int rc = TN_OK, m = 0;
+      while (m < n && (rc = injected(q + m)) == TN_OK) ++m;
+      if (m > 0) {
+        tn::AccumParams ap = accum_params(p, H);
+        batch_range(p, q, m, ap);
+        ap.F = batch_operand(p, P.fin.ref, ap.bA);
+        const cudaError_t e = tn::launch_accum(ap, st);
+        if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("accumulate launch: ") + cudaGetErrorString(e));
+      }
+      q += m;
+      if (done) *done = q;
+      if (rc) return rc;
+      continue;
+    }
+    for (int b = 0; b < n; ++b, ++q) {
+      if (int rc = injected(q)) return rc;
+      if (int rc = run_pass(p, slice_id(q), H, st, nullptr, b)) return rc;
+      if (done) *done = q + 1;
+    }
   }
-  if (passes_done) *passes_done = ni;
   return TN_OK;
+}
+
+static int run_slice(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st) {
+  return run_passes(p, s << p->P.n_internal, (s + 1) << p->P.n_internal, H, st);
 }
 
 static int check_range(tn_plan_t* plan, tn_range r, tn_head_t* head) {
@@ -1105,8 +1207,8 @@ static int capture_items(const std::vector<tn_plan_t*>& plans, const std::vector
   for (int b = 0; b < n_branches && ce == cudaSuccess; ++b) ce = cudaStreamWaitEvent(streams[1 + b], ev[0], 0);
   if (ce != cudaSuccess) rc = fail(TN_ERR_CUDA, std::string("graph fork: ") + cudaGetErrorString(ce));
   for (size_t i = 0; i < plans.size() && rc == TN_OK; ++i)
-    for (int64_t s = ranges[i].begin; s < ranges[i].end && rc == TN_OK; ++s)
-      rc = run_slice(plans[i], s, heads[i]->H, streams[1 + branch_of[i]]);
+    rc = run_passes(plans[i], ranges[i].begin << plans[i]->P.n_internal, ranges[i].end << plans[i]->P.n_internal,
+                    heads[i]->H, streams[1 + branch_of[i]]);
   for (int b = 0; b < n_branches && rc == TN_OK; ++b) {
     ce = cudaEventRecord(ev[1 + b], streams[1 + b]);
     if (ce == cudaSuccess) ce = cudaStreamWaitEvent(main, ev[1 + b], 0);
@@ -1382,16 +1484,11 @@ static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t
 
 namespace tn {
 int enqueue_slices(tn_plan_t* plan, tn_range r, double2* H, cudaStream_t stream, int64_t* done_end) {
-  for (int64_t s = r.begin; s < r.end; ++s) {
-    int64_t t = 0;
-    int rc = run_slice(plan, s, H, stream, &t);
-    if (rc) {
-      if (done_end) *done_end = t == 0 ? s : -1;
-      return rc;
-    }
-  }
-  if (done_end) *done_end = r.end;
-  return TN_OK;
+  const int ni = plan->P.n_internal;
+  int64_t q = 0;
+  const int rc = run_passes(plan, r.begin << ni, r.end << ni, H, stream, &q);
+  if (done_end) *done_end = q & ((1LL << ni) - 1) ? -1 : q >> ni;   // -1: a slice is partly accumulated
+  return rc;
 }
 int check_slice_range(tn_plan_t* plan, tn_range r, tn_head_t* head) { return check_range(plan, r, head); }
 void mark_slices_done(tn_head_t* head, tn_range r) { mark_done(head, r); }

@@ -46,6 +46,7 @@
 
 #include <algorithm>
 
+#include "batch.cuh"
 #include "direct.h"
 #include "kernels.h"
 
@@ -140,7 +141,8 @@ __global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectPa
   auto map_of = [](int mode, const uint32_t* tab, int64_t q) {
     return mode == 0 ? q : (mode == 1 ? (int64_t)0 : (int64_t)__ldg(tab + q));
   };
-  const float2* Xp = p.X + (p.fold ? 0 : map_of(p.mapX_mode, p.mapX, pc) * p.x_pstride) +
+  const int bz = blockIdx.y;
+  const float2* Xp = p.X + batch_offset(p, p.bA, bz) + (p.fold ? 0 : map_of(p.mapX_mode, p.mapX, pc) * p.x_pstride) +
                      scatter_warp(rt, p.rrest, p.n_rrest);
   const uint32_t ybase = scatter_warp(ctl, p.crest, p.n_crest);
 
@@ -168,6 +170,7 @@ __global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectPa
       }
   }
   const float2* yp[NY];
+  const float2* Yb = p.Y + batch_offset(p, p.bB, bz);
   uint32_t yse[NY];
 #pragma unroll
   for (int e = 0; e < NY; ++e) {
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectPa
       }
     int64_t q = pc0;
     if (p.fold) q = min(pc0 + ((tid + 256 * e) >> (tcb + tkb)), p.PC - 1);   // past the last pattern: read, never stored
-    yp[e] = p.Y + map_of(p.mapY_mode, p.mapY, q) * p.y_pstride + ybase + o;
+    yp[e] = Yb + map_of(p.mapY_mode, p.mapY, q) * p.y_pstride + ybase + o;
     yse[e] = u;
   }
 
@@ -250,7 +253,7 @@ __global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectPa
   // C[pattern][column][row], rows lowest; with folded patterns the column
   // index runs on across patterns, which is the same address
   const int64_t rows = 1LL << p.nr;
-  float2* Cp = p.C + (p.fold ? 0 : pc * p.c_pstride);
+  float2* Cp = p.C + batch_offset(p, p.bC, bz) + (p.fold ? 0 : pc * p.c_pstride);
   const int64_t row0 = (int64_t)rt << TRB, col0 = (int64_t)ct << TCB;
   float tmax = 0.0f;
   if (KG == 1 && CL == 1) {
@@ -319,7 +322,7 @@ __global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectPa
     __syncthreads();
     if (lane == 0) atomicMax(&s_amax, m);
     __syncthreads();
-    if (tid == 0 && s_amax) atomicMax(p.amax, s_amax);
+    if (tid == 0 && s_amax) atomicMax(p.amax + bz * p.amax_stride, s_amax);
   }
 }
 
@@ -358,7 +361,7 @@ cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s, boo
     if (r != cudaSuccess) return r;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * p.cluster));
+  cfg.gridDim = dim3((unsigned)(tiles * p.cluster), (unsigned)p.n_batch);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = (size_t)e.smem;
   cfg.stream = s;

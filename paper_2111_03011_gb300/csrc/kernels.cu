@@ -5,6 +5,7 @@
 
 #include <cstdio>
 
+#include "batch.cuh"
 #include "kernels.h"
 
 namespace tn {
@@ -42,6 +43,10 @@ __global__ void __launch_bounds__(256) k_small(SmallParams p) {
       if ((k >> j) & 1) o |= 1LL << p.kpos[j];
     offK[k] = o;
   }
+  const int bz = blockIdx.z;
+  const float2* __restrict__ A0 = p.A + batch_offset(p, p.bA, bz);
+  const float2* __restrict__ B0 = p.B + batch_offset(p, p.bB, bz);
+  float2* __restrict__ C0 = p.C + batch_offset(p, p.bC, bz);
   const int64_t rowsC = p.M;  // C stride of the n index
   __shared__ unsigned int s_amax;
   if (threadIdx.x == 0) s_amax = 0u;
@@ -52,11 +57,11 @@ __global__ void __launch_bounds__(256) k_small(SmallParams p) {
     __syncthreads();
     for (int i = threadIdx.x; i < KK * NNN; i += blockDim.x) {
       const int k = i / NNN, n = i % NNN;
-      Bs[k][n] = p.B[pb * p.b_pstride + p.boffK[k] + p.boffN[n]];
+      Bs[k][n] = B0[pb * p.b_pstride + p.boffK[k] + p.boffN[n]];
     }
     __syncthreads();
-    const float2* __restrict__ Ap = p.A + pa * p.a_pstride;
-    float2* __restrict__ Cp = p.C + pc * p.c_pstride;
+    const float2* __restrict__ Ap = A0 + pa * p.a_pstride;
+    float2* __restrict__ Cp = C0 + pc * p.c_pstride;
     for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < p.M; m += (int64_t)gridDim.x * blockDim.x) {
       int64_t x = m;
 #pragma unroll
@@ -83,7 +88,7 @@ __global__ void __launch_bounds__(256) k_small(SmallParams p) {
     __syncthreads();
     if ((threadIdx.x & 31) == 0) atomicMax(&s_amax, b);
     __syncthreads();
-    if (threadIdx.x == 0) atomicMax(p.amax, s_amax);
+    if (threadIdx.x == 0) atomicMax(p.amax + bz * p.amax_stride, s_amax);
   }
 }
 
@@ -95,7 +100,7 @@ static cudaError_t launch_small_t(const SmallParams& p, cudaStream_t s) {
   int64_t by = p.PC < 65535 ? p.PC : 65535;
   if (bx * by > cap * 4) bx = std::max<int64_t>(1, (cap * 4) / by);
   if (bx < 1) bx = 1;
-  k_small<NK, NN><<<dim3((unsigned)bx, (unsigned)by), threads, 0, s>>>(p);
+  k_small<NK, NN><<<dim3((unsigned)bx, (unsigned)by, (unsigned)p.n_batch), threads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -716,10 +721,14 @@ __global__ void k_accum(AccumParams p) {
     int64_t off = (int64_t)__ldg(p.pidx + g) * p.f_pstride;
     for (int j = 0; j < p.h; ++j)
       if ((mu >> j) & 1) off |= 1LL << p.open_pos[j];
-    const float2 v = __ldg(p.F + off);
+    // the passes of a batch are added one after another, as single launches would
     double2 hv = p.H[e];
-    hv.x += (double)v.x;
-    hv.y += (double)v.y;
+#pragma unroll 4
+    for (int b = 0; b < p.n_batch; ++b) {
+      const float2 v = __ldg(p.F + batch_offset(p, p.bA, b) + off);
+      hv.x += (double)v.x;
+      hv.y += (double)v.y;
+    }
     p.H[e] = hv;
   }
 }

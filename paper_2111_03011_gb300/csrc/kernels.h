@@ -34,8 +34,26 @@ struct AbsmaxParams {
   unsigned int* out;     // scale slot (fp32 bits of the running maximum; zeroed per pass)
 };
 
+// A launch for the passes q0 .. q0 + n_batch - 1 of a range at once: pass q is
+// slice id (q >> ni) | (q & (2^ni - 1)) << k, ni the bits of automatically
+// sliced edges, k the user's.  An operand of batch element b lies at
+// b * stride elements from its base, or, for a leaf, at its variant: bit t
+// of the variant's index is bit bits[t] of the slice id.  n_batch = 1 with zero
+// strides and no bits: a plain launch.
+struct BatchOperand {
+  int64_t stride = 0, var_size = 0;
+  int n_bits = 0;
+  uint8_t bits[8] = {0};
+};
+struct BatchParams {
+  int n_batch = 1, ni = 0, k = 0;
+  int64_t q0 = 0;
+  BatchOperand bA, bB, bC;     // operands (direct step: X, Y) and result; accumulation: bA is F
+  int64_t amax_stride = 0;     // scale slots between the passes' copies
+};
+
 // C[p][m + (n << (rA-nk))] = sum_k A[mapA(p)][insert_K(m) + k-offset] * B[mapB(p)][boffK[k] + boffN[n]]
-struct SmallParams {
+struct SmallParams : BatchParams {
   const float2* A; const float2* B; float2* C;
   int64_t a_pstride, b_pstride, c_pstride;
   int64_t M;            // rows per pattern = 2^(rA - nk)
@@ -102,7 +120,7 @@ struct GemmTile {
 GemmTile gemm_tc_tile(const GemmParams& p);
 
 // C[p][c][r] = sum_k X[mapX(p)][r, k] Y[mapY(p)][k, c], operands where they lie
-struct DirectParams : DirectParamsBase {
+struct DirectParams : DirectParamsBase, BatchParams {
   const float2* X; const float2* Y; float2* C;
   const uint32_t* mapX; const uint32_t* mapY;
   unsigned int* amax;        // non-null: atomicMax of the output's max |re|, |im| (fp32 bits)
@@ -121,7 +139,7 @@ struct GemmOperands {
 };
 cudaError_t launch_gemm_operands(const GemmOperands& p, cudaStream_t s);
 
-struct AccumParams {
+struct AccumParams : BatchParams {
   const float2* F; double2* H;
   int64_t f_pstride;
   int64_t L; int h;

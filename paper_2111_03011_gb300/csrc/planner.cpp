@@ -1293,9 +1293,52 @@ static void schedule_side_bprep(Plan& plan) {
   }
 }
 
-static void plan_arena(Plan& plan) {
-  std::vector<int> idx(plan.bufs.size());
-  for (size_t i = 0; i < idx.size(); ++i) idx[i] = (int)i;
+// Steps that run once for a whole chunk of passes (slices, or the passes of
+// automatically sliced edges).  The streaming steps near the leaves work on a few
+// thousand elements, so a pass is a chain of launches that each take
+// microseconds and leave the chip idle.  A streaming step whose operands are
+// leaves or results of such steps, with a result of at most 2^18 elements, is
+// launched for all passes of a chunk at once, before the rest of any of them;
+// each pass has its own copy of its result.  The copies take at most 64 MB, half
+// of L2, so that a pass still finds its own there.  16 slices of a 16-qubit
+// circuit (6 launches each) take 62 us, with the reset and the lookup, where 16
+// chains of launches took 420 us.
+constexpr double kBatchElems = 0x1p18;
+constexpr int64_t kBatchBytes = 64LL << 20;
+constexpr int kBatchMost = 64;
+
+static void mark_batched(Plan& plan) {
+  plan.batch_max = 1;
+  const int bits = plan.n_sliced + plan.n_internal;
+  if (bits == 0) return;
+  auto ready = [&](const Ref& r) {
+    return r.kind == 0 ? plan.leaf_info[r.id].var_slice_bits.size() <= 8 : plan.bufs[r.id].batch;
+  };
+  bool any = plan.steps.empty();
+  for (Step& x : plan.steps) {
+    x.batch = x.kind == ST_SMALL && ready(x.a) && ready(x.b) &&
+              (double)x.PC * std::exp2((double)x.rC) <= kBatchElems;
+    if (x.batch) plan.bufs[x.c.id].batch = true;
+    any = any || x.batch;
+  }
+  if (!any || (plan.steps.empty() && !ready(plan.fin.ref))) return;
+  // what a later, unbatched step or the accumulation reads lives to the end
+  const int end = (int)plan.steps.size();
+  auto keep = [&](const Ref& r) {
+    if (r.kind == 1 && plan.bufs[r.id].batch) plan.bufs[r.id].last = end;
+  };
+  for (const Step& x : plan.steps)
+    if (!x.batch) {
+      keep(x.a);
+      keep(x.b);
+    }
+  keep(plan.fin.ref);
+  plan.batch_max = (int)std::min<int64_t>(kBatchMost, bits >= 6 ? kBatchMost : 1LL << bits);
+}
+
+// Offsets of the buffers `idx` whose lifetimes overlap, largest first at the
+// lowest free offset; returns the size.
+static int64_t place_buffers(Plan& plan, std::vector<int> idx) {
   std::sort(idx.begin(), idx.end(), [&](int a, int b) {
     if (plan.bufs[a].bytes != plan.bufs[b].bytes) return plan.bufs[a].bytes > plan.bufs[b].bytes;
     return a < b;
@@ -1320,7 +1363,19 @@ static void plan_arena(Plan& plan) {
     peak = std::max(peak, off + B.bytes);
     placed.push_back(b);
   }
-  plan.workspace_bytes = peak;
+  return peak;
+}
+
+// The arena: the buffers of a pass, then the copies of the batched ones.
+static void plan_arena(Plan& plan) {
+  std::vector<int> own, batched;
+  for (size_t i = 0; i < plan.bufs.size(); ++i) (plan.bufs[i].batch ? batched : own).push_back((int)i);
+  const int64_t base = place_buffers(plan, own);
+  plan.batch_stride = place_buffers(plan, batched);
+  for (int b : batched) plan.bufs[b].off += base;
+  if (plan.batch_stride > 0)
+    plan.batch_max = (int)std::max<int64_t>(1, std::min<int64_t>(plan.batch_max, kBatchBytes / plan.batch_stride));
+  plan.workspace_bytes = base + plan.batch_max * plan.batch_stride;
 }
 
 // --------------------------------------------------------------------- driver
@@ -1645,6 +1700,7 @@ int build_plan(const PlanInput& in, Plan& plan, std::string& err) {
   plan.fin.pidx_off = meta_push(plan, pidx);
   touch(plan, F.ref, (int)plan.steps.size());
   if (in.side_bprep) schedule_side_bprep(plan);
+  mark_batched(plan);
   plan_arena(plan);
   return TN_OK;
 }
@@ -1718,7 +1774,7 @@ std::string describe_plan(const Plan& plan, bool with_data) {
     for (int v = 0; v < 16; ++v) o << (v ? "," : "") << st.boffN[v];
     o << "],\"mapA\":[" << st.mapA_mode << "," << st.mapA_off << "],\"mapB\":[" << st.mapB_mode << ","
       << st.mapB_off << "],\"bk_off\":" << st.bk_off << ",\"bn_off\":" << st.bn_off << ",\"bprep_embed0\":" << st.bprep_embed0 << ",\"variant\":" << st.variant
-      << ",\"grp\":[" << st.grp_fold << "," << st.n_groups << "," << st.grp_off << "],\"direct\":" << (st.direct ? 1 : 0);
+      << ",\"batch\":" << (st.batch ? 1 : 0) << ",\"grp\":[" << st.grp_fold << "," << st.n_groups << "," << st.grp_off << "],\"direct\":" << (st.direct ? 1 : 0);
     if (st.direct) {
       const DirectPlan& d = st.dp;
       auto list = [&o](const char* name, const uint8_t* v, int n) {
@@ -1770,7 +1826,8 @@ std::string describe_plan(const Plan& plan, bool with_data) {
     o << "]";
   }
   o << ",\"tc_macs\":" << plan.tc_macs << ",\"alg_bytes\":" << plan.alg_bytes << ",\"max_log2\":" << plan.max_log2
-    << ",\"workspace_bytes\":" << plan.workspace_bytes << "}";
+    << ",\"workspace_bytes\":" << plan.workspace_bytes << ",\"batch\":[" << plan.batch_max << "," << plan.batch_stride
+    << "]}";
   return o.str();
 }
 

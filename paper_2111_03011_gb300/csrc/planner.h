@@ -75,6 +75,7 @@ struct BufInfo {
   int64_t bytes = 0;
   int64_t off = 0;
   int first = 0, last = 0;  // step lifetime (inclusive)
+  bool batch = false;       // written by a batched step: one copy per pass of a chunk, Plan::batch_stride apart
 };
 
 // Tile schedule of a permute step: tile bits, its tables in meta and the
@@ -100,6 +101,8 @@ struct Step {
   // SMALL
   int kposA[4] = {0, 0, 0, 0};
   uint32_t boffK[16] = {0}, boffN[16] = {0};
+  // SMALL: run once for all passes of a chunk (see mark_batched)
+  bool batch = false;
   // SMALL in the direct form (direct.cu): small or narrow contractions of any K
   bool direct = false;
   DirectPlan dp;
@@ -193,6 +196,8 @@ struct Plan {
   FinalInfo fin;
   int64_t n_patterns_final = 1;
   int64_t workspace_bytes = 0;
+  int batch_max = 1;               // passes per chunk (1: no step is batched)
+  int64_t batch_stride = 0;        // bytes between the copies of a batched buffer
   double tc_macs = 0, alg_bytes = 0, max_log2 = 0;
   int n_contractions = 0;
 
