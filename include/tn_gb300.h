@@ -265,9 +265,10 @@ int  tn_contract_slices(tn_plan_t* plan, tn_range slice_range, tn_head_t* head, 
  * graph (cached per plan, range and head buffer) and replayed on `stream`.
  * tn_contract_batch: items (plans[i], ranges[i], heads[i]) as parallel
  * branches of one graph (items of the same plan share a branch, since they
- * share its workspace), so many small contractions overlap on the GPU; the
- * last batch's graph is cached per thread and replayed when the same batch is
- * submitted again.  Both asynchronous on `stream`; both reject slices already
+ * share its workspace), so many small contractions overlap on the GPU.  The
+ * first time a thread submits a batch it is launched on branch streams; from
+ * the second time on its captured graph is replayed (the last 8 batches'
+ * graphs are kept per thread).  Both asynchronous on `stream`; both reject slices already
  * accumulated into a head, and a batch rejects a head listed twice.  Items
  * with an empty range record nothing.  tn_contract_slices_graph keeps at most
  * 16 captured ranges per plan and drops the least recently replayed one. */

@@ -553,7 +553,7 @@ static const float2* batch_operand(const tn_plan_t* p, const tn::Ref& r, tn::Bat
   }
   const tn::LeafInfo& li = p->P.leaf_info[r.id];
   o.var_size = li.size;
-  o.n_bits = (int)li.var_slice_bits.size();
+  o.n_bits = std::min((int)li.var_slice_bits.size(), 8);   // at most 8 (mark_batched)
   for (int t = 0; t < o.n_bits; ++t) o.bits[t] = (uint8_t)li.var_slice_bits[t];
   return p->d_leaves + li.off;
 }
@@ -1187,42 +1187,62 @@ extern "C" int tn_contract_slices(tn_plan_t* plan, tn_range r, tn_head_t* head, 
 
 // ---------------------------------------------------------- CUDA graphs
 
-// Capture the launches of `slices` of every (plan, head) item, item i on branch
-// stream branch_of[i], into one graph (fork/join through events).
-static int capture_items(const std::vector<tn_plan_t*>& plans, const std::vector<tn_range>& ranges,
-                         const std::vector<tn_head_t*>& heads, const std::vector<int>& branch_of, int n_branches,
-                         cudaGraphExec_t* exec_out) {
+// Branch streams of this thread (and the stream that captures): one set, reused.
+static int branch_streams(int n, std::vector<cudaStream_t>** out) {
   static thread_local std::vector<cudaStream_t> streams;
-  while ((int)streams.size() < n_branches + 1) {
+  while ((int)streams.size() < n) {
     cudaStream_t st;
     CUDA_TRY(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
     streams.push_back(st);
   }
-  cudaStream_t main = streams[0];
-  std::vector<cudaEvent_t> ev(n_branches + 1);
-  for (auto& e : ev) CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  CUDA_TRY(cudaStreamBeginCapture(main, cudaStreamCaptureModeThreadLocal));
+  *out = &streams;
+  return TN_OK;
+}
+
+// Enqueue the slices of every (plan, head) item, item i on branch stream
+// 1 + branch_of[i], between a fork from `main` and a join into it (events).
+static int fork_items(const std::vector<tn_plan_t*>& plans, const std::vector<tn_range>& ranges,
+                      const std::vector<tn_head_t*>& heads, const std::vector<int>& branch_of, int n_branches,
+                      cudaStream_t main, const std::vector<cudaStream_t>& streams) {
+  static thread_local std::vector<cudaEvent_t> ev;
+  while ((int)ev.size() < n_branches + 1) {
+    cudaEvent_t e;
+    CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    ev.push_back(e);
+  }
   int rc = TN_OK;
   cudaError_t ce = cudaEventRecord(ev[0], main);
   for (int b = 0; b < n_branches && ce == cudaSuccess; ++b) ce = cudaStreamWaitEvent(streams[1 + b], ev[0], 0);
-  if (ce != cudaSuccess) rc = fail(TN_ERR_CUDA, std::string("graph fork: ") + cudaGetErrorString(ce));
+  if (ce != cudaSuccess) rc = fail(TN_ERR_CUDA, std::string("fork: ") + cudaGetErrorString(ce));
   for (size_t i = 0; i < plans.size() && rc == TN_OK; ++i)
     rc = run_passes(plans[i], ranges[i].begin << plans[i]->P.n_internal, ranges[i].end << plans[i]->P.n_internal,
                     heads[i]->H, streams[1 + branch_of[i]]);
-  for (int b = 0; b < n_branches && rc == TN_OK; ++b) {
+  // joined on failure too, so that what was enqueued stays ordered before the caller's next work
+  for (int b = 0; b < n_branches; ++b) {
     ce = cudaEventRecord(ev[1 + b], streams[1 + b]);
     if (ce == cudaSuccess) ce = cudaStreamWaitEvent(main, ev[1 + b], 0);
-    if (ce != cudaSuccess) rc = fail(TN_ERR_CUDA, std::string("graph join: ") + cudaGetErrorString(ce));
+    if (rc == TN_OK && ce != cudaSuccess) rc = fail(TN_ERR_CUDA, std::string("join: ") + cudaGetErrorString(ce));
   }
+  return rc;
+}
+
+// The same, captured into an executable graph.
+static int capture_items(const std::vector<tn_plan_t*>& plans, const std::vector<tn_range>& ranges,
+                         const std::vector<tn_head_t*>& heads, const std::vector<int>& branch_of, int n_branches,
+                         cudaGraphExec_t* exec_out) {
+  std::vector<cudaStream_t>* streams = nullptr;
+  if (int rc = branch_streams(n_branches + 1, &streams)) return rc;
+  cudaStream_t main = (*streams)[0];
+  CUDA_TRY(cudaStreamBeginCapture(main, cudaStreamCaptureModeThreadLocal));
+  int rc = fork_items(plans, ranges, heads, branch_of, n_branches, main, *streams);
   cudaGraph_t graph = nullptr;
-  ce = cudaStreamEndCapture(main, &graph);
+  cudaError_t ce = cudaStreamEndCapture(main, &graph);
   if (rc == TN_OK && ce != cudaSuccess) rc = fail(TN_ERR_CUDA, std::string("end capture: ") + cudaGetErrorString(ce));
   if (rc == TN_OK) {
     ce = cudaGraphInstantiate(exec_out, graph, 0);
     if (ce != cudaSuccess) rc = fail(TN_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
   }
   if (graph) cudaGraphDestroy(graph);
-  for (auto& e : ev) cudaEventDestroy(e);
   cudaGetLastError();
   return rc;
 }
@@ -1280,27 +1300,72 @@ extern "C" int tn_contract_batch(tn_plan_t* const* plans, const tn_range* ranges
   }
   const int n_branches = std::min<int>((int)branch_of_plan.size(), 32);
   for (int i = 0; i < n; ++i) branch[i] %= n_branches;
-  // single-entry cache: the same batch again replays the same graph.  Keyed
-  // on the handles' serials (never reused), not on their addresses.
-  static thread_local std::vector<uint64_t> last_p;
-  static thread_local std::vector<int64_t> last_r;
-  static thread_local std::vector<uint64_t> last_h;
-  static thread_local cudaGraphExec_t last_exec = nullptr;
-  std::vector<int64_t> rr;
-  for (auto& x : R) { rr.push_back(x.begin); rr.push_back(x.end); }
-  std::vector<uint64_t> sp, sh;
-  for (auto* x : P) sp.push_back(x->serial);
-  for (auto* x : Hs) sh.push_back(x->serial);
-  if (!(last_exec && last_p == sp && last_r == rr && last_h == sh)) {
-    if (last_exec) cudaGraphExecDestroy(last_exec);
-    last_exec = nullptr;
-    int rc = capture_items(P, R, Hs, branch, n_branches, &last_exec);
-    if (rc) { last_exec = nullptr; return rc; }
-    last_p = sp;
-    last_r = rr;
-    last_h = sh;
+  // A batch is known by its handles' serials (never reused) and ranges.  The
+  // first time one is seen its launches go straight to the branch streams,
+  // which takes less host time than capturing and instantiating a graph; from
+  // the second time on a captured graph is replayed.  Per thread, the graphs
+  // of the kBatchGraphs batches replayed last are kept, and the keys of the
+  // kBatchSeen seen last.
+  struct Batch {
+    std::vector<uint64_t> p, h;
+    std::vector<int64_t> r;
+    cudaGraphExec_t exec = nullptr;
+    uint64_t last_use = 0;
+    bool same(const Batch& o) const { return p == o.p && h == o.h && r == o.r; }
+  };
+  constexpr size_t kBatchGraphs = 8, kBatchSeen = 32;
+  static thread_local std::vector<Batch> known;
+  static thread_local uint64_t clock = 0;
+  Batch key;
+  for (auto* x : P) key.p.push_back(x->serial);
+  for (auto* x : Hs) key.h.push_back(x->serial);
+  for (auto& x : R) { key.r.push_back(x.begin); key.r.push_back(x.end); }
+  auto it = std::find_if(known.begin(), known.end(), [&](const Batch& b) { return b.same(key); });
+  const bool seen = it != known.end();
+  if (!seen) {
+    if (known.size() >= kBatchSeen) {
+      auto lru = std::min_element(known.begin(), known.end(),
+                                  [](const Batch& a, const Batch& b) { return a.last_use < b.last_use; });
+      if (lru->exec) cudaGraphExecDestroy(lru->exec);
+      known.erase(lru);
+    }
+    known.push_back(key);
+    it = std::prev(known.end());
   }
-  CUDA_TRY(cudaGraphLaunch(last_exec, (cudaStream_t)stream));
+  it->last_use = ++clock;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CUDA_TRY(cudaStreamIsCapturing((cudaStream_t)stream, &cap));
+  // into a capture of the caller's, and with a fault armed (which must leave
+  // every head as it was), only as a graph
+  if (!seen && cap == cudaStreamCaptureStatusNone && !std::getenv("TN_FAULT_INJECT")) {
+    std::vector<cudaStream_t>* streams = nullptr;
+    if (int rc = branch_streams(n_branches + 1, &streams)) return rc;
+    const int rc = fork_items(P, R, Hs, branch, n_branches, (cudaStream_t)stream, *streams);
+    if (rc) {   // a launch failed: which passes reached the heads is not recorded
+      for (int i = 0; i < n; ++i)
+        if (R[i].begin < R[i].end) Hs[i]->invalid = true;
+      g_err += "; the heads of the batch are invalid until tn_head_reset";
+      return rc;
+    }
+  } else {
+    if (!it->exec) {
+      size_t graphs = 0;
+      for (const Batch& b : known) graphs += b.exec != nullptr;
+      if (graphs >= kBatchGraphs) {
+        auto lru = known.end();
+        for (auto b = known.begin(); b != known.end(); ++b)
+          if (b->exec && (lru == known.end() || b->last_use < lru->last_use)) lru = b;
+        cudaGraphExecDestroy(lru->exec);
+        lru->exec = nullptr;
+      }
+      const int rc = capture_items(P, R, Hs, branch, n_branches, &it->exec);
+      if (rc) {
+        it->exec = nullptr;
+        return rc;
+      }
+    }
+    CUDA_TRY(cudaGraphLaunch(it->exec, (cudaStream_t)stream));
+  }
   for (int i = 0; i < n; ++i) mark_done(Hs[i], R[i]);
   return TN_OK;
 }

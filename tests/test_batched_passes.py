@@ -99,3 +99,45 @@ def test_failure_inside_a_chunk_keeps_the_passes_before_it(tn, monkeypatch):
     tn.tn_contract_slices(p, 5, 16, head)
     torch.cuda.synchronize()
     assert np.array_equal(buf.cpu().numpy(), _head(tn, p, [(0, 16)]))
+
+
+@pytest.mark.gpu
+def test_batches_first_seen_and_replayed(tn, monkeypatch):
+    """A batch's first submission (branch streams), its second (captured) and
+    later ones (replayed, also after enough other batches to drop its graph)
+    give the heads of plain calls, bit for bit; a failing submission leaves every
+    head as it was."""
+    import torch
+    cfgs = [ci.config_small(4, 4, 6 + i, seed=20 + i, n_open=5, L=6, n_cut_gates=i % 2, tail_seed=30 + i)
+            for i in range(12)]
+    plans = [tn.tn_plan(c["circuit"], c["open_qubits"], c["tails"], c["edges"], gemm=[1, 4][i % 2])
+             for i, c in enumerate(cfgs)]
+    ends = [1 << tn.tn_plan_get_stats(p)["n_sliced"] for p in plans]
+    ref = [_head(tn, p, [(0, e)]) for p, e in zip(plans, ends)]
+    bufs = [torch.zeros(r.shape, dtype=torch.complex128, device="cuda") for r in ref]
+    heads = [tn.tn_head_create(p, b) for p, b in zip(plans, bufs)]
+
+    def submit(idx):
+        for i in idx:
+            tn.tn_head_reset(heads[i])
+        tn.tn_contract_batch([plans[i] for i in idx], [(0, ends[i]) for i in idx], [heads[i] for i in idx])
+        torch.cuda.synchronize()
+        for i in idx:
+            assert np.array_equal(bufs[i].cpu().numpy(), ref[i])
+
+    batches = [[i, (i + 1) % 12, (i + 5) % 12] for i in range(10)]
+    for _ in range(3):
+        for b in batches:
+            submit(b)
+    submit(list(range(12)))
+    for i in range(3):
+        tn.tn_head_reset(heads[i])
+    torch.cuda.synchronize()
+    monkeypatch.setenv("TN_FAULT_INJECT", "slice:0")
+    with pytest.raises(tn.TNError):
+        tn.tn_contract_batch(plans[:3], [(0, e) for e in ends[:3]], heads[:3])
+    monkeypatch.delenv("TN_FAULT_INJECT")
+    torch.cuda.synchronize()
+    assert all(float(b.abs().max()) == 0.0 for b in bufs[:3])
+    assert all(tn.tn_head_fidelity(h)[1] == 0 for h in heads[:3])
+    submit([0, 1, 2])
