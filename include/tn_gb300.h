@@ -96,9 +96,9 @@ typedef struct {
   int    max_host_absorb_log2;/* size cap of host-side absorption of order<=2 tensors (0: 12)*/
   int    small_max_bits;      /* contractions with <= this many contracted and new legs use the
                                  streaming small-operand kernel (0: 4; -1: none, all GEMM steps).  With 4,
-                                 other steps that are small or narrow run as one direct FP32 kernel
-                                 where that is modelled faster than permute, B preparation and GEMM
-                                 (not the bf16 steps of BF16X3 plans, not SIMT_FP32 plans) */
+                                 other steps that are small or narrow run as one direct kernel on the
+                                 CUDA cores where that is modelled faster than permute, B preparation
+                                 and GEMM (not in SIMT_FP32 plans) */
   int    auto_slice;          /* 0: off.  Otherwise, when no order fits the cap, slice up to this
                                  many more wires (at most 24), chosen on the best over-cap order:
                                  each is the bond carried by the most over-cap intermediates
@@ -420,8 +420,8 @@ int  tn_head_norm_noalloc(const void* head_c128, int64_t n_groups, int n_open, d
  * arrays of PC pattern indices, or NULL for the identity (P = PC) or pattern 0
  * (P = 1).  The operands pass through the same kernels as a plan's steps
  * (engine TN_GEMM_*): split permute, B preparation and GEMM, or, with pair = 0
- * and a tensor-core engine, the direct FP32 kernel where it is modelled faster
- * (small or narrow shapes; not in bf16).  pair = -1: one-CTA GEMM tiles,
+ * and a tensor-core engine, the direct kernel (FP32 products; BF16x3 ones for
+ * that engine) where it is modelled faster (small or narrow shapes).  pair = -1: one-CTA GEMM tiles,
  * pair > 0: the GEMM kernels with CTA pairs where they apply.  Its
  * scratch (split planes, prepared B, maps) comes from a bounded pool that the
  * library keeps between calls (at most 2 GiB, given back when an allocation

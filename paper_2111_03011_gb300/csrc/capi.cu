@@ -592,6 +592,7 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
         dp.mapY = p->d_meta + (x.dp.swap ? x.mapA_off : x.mapB_off);
         dp.mapX_mode = x.dp.swap ? x.mapB_mode : x.mapA_mode;
         dp.mapY_mode = x.dp.swap ? x.mapA_mode : x.mapB_mode;
+        dp.bf16 = P.gemm_engine == TN_GEMM_TC_BF16X3 && x.nk >= 2;   // K = 2 GEMM steps run in tf32
         dp.vec = 1;                      // buffers start on 256 bytes, rows pair up from even ones
         dp.amax = scale_ptr(p, x.max_slot, b);
         if (n_batch > 1) {
@@ -1604,7 +1605,7 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
   // The direct kernel where it is modelled faster than the three launches
   // below (as the planner chooses; C is row-major, so its rows are N and X is
   // B).  pair != 0 asks for the GEMM kernels themselves.
-  if (!simt && pair == 0 && !(engine == TN_GEMM_TC_BF16X3 && nk >= 2) && nmk <= 31 && nk + nn <= 31) {
+  if (!simt && pair == 0 && nmk <= 31 && nk + nn <= 31) {
     int nm = nmk - nk;
     std::vector<int> xr, xk, yk, yc;
     for (int j = 0; j < nn; ++j) xr.push_back(j);
@@ -1623,6 +1624,7 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
       ds.yc = yc.data();
       ds.PC = PC;
       ds.x_shared = mode[1] == 1;
+      ds.bf16 = h16 == 1;
       ds.x_elems = (double)PB * (double)(K * N);
       ds.y_elems = (double)PA * (double)(M * K);
       const tn::DirectPlan d = tn::plan_direct(ds, fold != 0);
@@ -1651,6 +1653,7 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
       dp.mapY = d_maps;
       dp.mapX_mode = mode[1];
       dp.mapY_mode = mode[0];
+      dp.bf16 = h16 == 1;
       dp.vec = (uintptr_t)C % 16 == 0;
       dp.amax = nullptr;
       cudaError_t e = tn::launch_direct(dp, best.config, st, true);

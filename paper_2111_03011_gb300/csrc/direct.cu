@@ -40,8 +40,14 @@
 // rank order through distributed shared memory.  Every order is fixed, so the
 // same inputs give the same bits.
 //
+// BF16x3 plans.  A step of such a plan that would run in bf16 keeps that
+// engine's arithmetic here: the three products of bf16 parts, in FP32.  With
+// plain FP32 products in some steps the amplitudes move by as much as the
+// engine's own error (2e-5).
+//
 // Folded patterns.  When all patterns share X, the columns run over (pattern,
 // column): one tile serves several patterns and X is read once for all of them.
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -113,7 +119,14 @@ struct DirectTile {
   static_assert(RM % 2 == 0 && NX >= 1 && KG >= 1 && KG <= TK, "tile");
 };
 
-template <int TRB, int TCB, int RM, int RN, int TKB>
+// x as a bf16 (rounded to nearest even) and the bf16 of the remainder
+__device__ __forceinline__ void split_bf16(float2 x, float2& hi, float2& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x.x, x.y);
+  hi = __bfloat1622float2(h);
+  lo = __bfloat1622float2(__floats2bfloat162_rn(x.x - hi.x, x.y - hi.y));
+}
+
+template <int TRB, int TCB, int RM, int RN, int TKB, bool BF16>
 __global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectParams p) {
   using T = DirectTile<TRB, TCB, RM, RN, TKB>;
   constexpr int TR = T::TR, TC = T::TC, KG = T::KG, LDX = T::LDX, LDY = T::LDY, NX = T::NX, NY = T::NY;
@@ -242,10 +255,27 @@ __global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectPa
       } else {
         b[0] = yb[k * LDY + cg];
       }
+      if constexpr (BF16) {
+        // the BF16x3 products, correction terms first
+        float2 al[RM], bl[RN];
 #pragma unroll
-      for (int i = 0; i < RM; ++i)
+        for (int i = 0; i < RM; ++i) split_bf16(a[i], a[i], al[i]);
 #pragma unroll
-        for (int c = 0; c < RN; ++c) cmul_acc(acc[i][c], a[i], b[c]);
+        for (int c = 0; c < RN; ++c) split_bf16(b[c], b[c], bl[c]);
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+#pragma unroll
+          for (int c = 0; c < RN; ++c) {
+            cmul_acc(acc[i][c], a[i], bl[c]);
+            cmul_acc(acc[i][c], al[i], b[c]);
+            cmul_acc(acc[i][c], a[i], b[c]);
+          }
+      } else {
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+#pragma unroll
+          for (int c = 0; c < RN; ++c) cmul_acc(acc[i][c], a[i], b[c]);
+      }
     }
   }
   cp_wait<0>();
@@ -330,23 +360,26 @@ namespace {
 
 typedef void (*DirectKernel)(DirectParams);
 struct DirectEntry {
-  DirectKernel fn;
+  DirectKernel fn[2];      // FP32 products, BF16x3 products
   int smem;
 };
-#define DIRECT_ENTRY(a, b, c, d, e) {k_direct<a, b, c, d, e>, DirectTile<a, b, c, d, e>::SMEM}
+#define DIRECT_ENTRY(a, b, c, d, e) \
+  {{k_direct<a, b, c, d, e, false>, k_direct<a, b, c, d, e, true>}, DirectTile<a, b, c, d, e>::SMEM}
 // in the order of kDirectConfigs (direct.h)
 const DirectEntry kEntries[kNumDirectConfigs] = {
-    DIRECT_ENTRY(6, 6, 4, 4, 4), DIRECT_ENTRY(6, 5, 4, 4, 4), DIRECT_ENTRY(6, 4, 4, 4, 5), DIRECT_ENTRY(6, 2, 4, 2, 5),
+    DIRECT_ENTRY(6, 6, 4, 4, 4), DIRECT_ENTRY(6, 5, 4, 4, 4), DIRECT_ENTRY(6, 4, 4, 4, 5), DIRECT_ENTRY(6, 2, 4, 4, 5),
     DIRECT_ENTRY(6, 0, 4, 1, 5),
-    DIRECT_ENTRY(4, 4, 4, 4, 6), DIRECT_ENTRY(4, 2, 4, 2, 7), DIRECT_ENTRY(4, 0, 4, 1, 7),
+    DIRECT_ENTRY(4, 4, 4, 4, 6), DIRECT_ENTRY(4, 2, 4, 4, 7), DIRECT_ENTRY(4, 0, 4, 1, 7),
 };
 
 }  // namespace
 
 cudaError_t prepare_direct() {
   for (const DirectEntry& e : kEntries) {
-    const cudaError_t r = cudaFuncSetAttribute((const void*)e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
-    if (r != cudaSuccess) return r;
+    for (DirectKernel fn : e.fn) {
+      const cudaError_t r = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
+      if (r != cudaSuccess) return r;
+    }
   }
   return cudaSuccess;
 }
@@ -357,7 +390,8 @@ cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s, boo
   if (tiles < 1 || tiles * p.cluster > 0x7fffffffLL) return cudaErrorInvalidValue;
   const DirectEntry& e = kEntries[config];
   if (prepare) {
-    const cudaError_t r = cudaFuncSetAttribute((const void*)e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
+    const cudaError_t r =
+        cudaFuncSetAttribute((const void*)e.fn[p.bf16 != 0], cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
     if (r != cudaSuccess) return r;
   }
   cudaLaunchConfig_t cfg = {};
@@ -371,7 +405,7 @@ cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s, boo
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = p.cluster > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, e.fn, p);
+  return cudaLaunchKernelEx(&cfg, e.fn[p.bf16 != 0], p);
 }
 
 }  // namespace tn

@@ -56,6 +56,7 @@ struct DirectShape {
   int64_t PC = 1;
   bool x_shared = false;   // every pattern reads X's pattern 0
   double x_elems = 0, y_elems = 0;
+  bool bf16 = false;       // BF16x3 products: three multiply-adds for one
 };
 DirectPlan plan_direct(const DirectShape& s, bool fold);
 
@@ -66,6 +67,7 @@ struct DirectParamsBase {
   uint32_t col_tiles;
   int nr, nk, nc, n_rrest, n_crest, fold, cluster;
   int mapX_mode, mapY_mode;      // 0 identity, 1 zero, 2 table
+  int bf16;                      // 1: BF16x3 products
   int vec;                       // C and its pattern stride allow 16-byte stores of two rows
   uint8_t rrest[32], crest[32], kxrest[32], kyrest[32];
   // per bit of a stage's element index: what it adds to the source offset and

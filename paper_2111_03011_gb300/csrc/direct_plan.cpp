@@ -71,7 +71,7 @@ DirectPlan plan_direct(const DirectShape& s, bool fold) {
   const double fill = std::min(1.0, ctas / (kSmCount * kBusy));
   const double c_elems = (double)s.PC * std::ldexp(1.0, s.nr + s.nc);
   const double l2 = 8.0 * s.x_elems * (double)(d.col_tiles - 1) / (2.0 * kBytesPerSecond);
-  d.seconds = kLaunchSeconds + std::max(padded / (g.rate * fill),
+  d.seconds = kLaunchSeconds + std::max(padded * (s.bf16 ? 3.5 : 1.0) / (g.rate * fill),
                                         8.0 * (s.x_elems + s.y_elems + c_elems) / (kBytesPerSecond * fill) + l2);
   return d;
 }

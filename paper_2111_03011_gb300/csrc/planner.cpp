@@ -1029,12 +1029,10 @@ static int layout_steps(Plan& plan, std::string& err) {
     // patterns fold into the columns where they share that operand; the
     // cheapest of those forms is taken where its modelled time is below the
     // three-launch GEMM's.  Limited to plans whose streaming steps have their
-    // full range, and to operands whose offsets fit 32 bits.  A BF16x3 plan
-    // keeps the GEMM for every step that runs in bf16: FP32 in some of them
-    // moves its amplitudes by as much as that engine's own error (2e-5).
+    // full range, and to operands whose offsets fit 32 bits.
     DirectPlan dp;
     const bool h16_step = nk >= 2 && (plan.gemm_engine == TN_GEMM_TC_BF16X3 || plan.gemm_engine == TN_GEMM_TC_FP16X3);
-    if (!use_small && !(h16_step && plan.gemm_engine == TN_GEMM_TC_BF16X3) && plan.small_max_bits >= 4 && plan.gemm_engine != TN_GEMM_SIMT_FP32 && nm <= 31 &&
+    if (!use_small && plan.small_max_bits >= 4 && plan.gemm_engine != TN_GEMM_SIMT_FP32 && nm <= 31 &&
         big.legs.size() <= 31) {
       std::vector<int> mp, kp, ks, np;
       for (int l : M) mp.push_back(find_pos(big.legs, l));
@@ -1052,6 +1050,7 @@ static int layout_steps(Plan& plan, std::string& err) {
         ds.yk = swap ? kp.data() : ks.data();
         ds.yc = swap ? mp.data() : np.data();
         ds.PC = C.P;
+        ds.bf16 = h16_step && plan.gemm_engine == TN_GEMM_TC_BF16X3;
         ds.x_shared = (swap ? mapB_mode : mapA_mode) == 1;
         ds.x_elems = (double)vt_elems(swap ? sml : big);
         ds.y_elems = (double)vt_elems(swap ? big : sml);

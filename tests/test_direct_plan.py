@@ -75,10 +75,10 @@ def test_direct_steps_describe_their_contraction(tn, case, gemm):
         d = tn.tn_plan_describe(p)
         for s in d["steps"]:
             if s["direct"]:
-                assert s["kind"] == 0 and not (gemm == 3 and s["nk"] >= 2)
+                assert s["kind"] == 0
                 _check_direct(d, s)
                 seen += 1
-    assert seen > 0 or gemm == 3        # BF16x3 plans: K = 2 steps only
+    assert seen > 0
     # plans that ask for the GEMM form, and the plain CUDA-core engine, have none
     for kw in (dict(gemm=gemm, small_max_bits=-1), dict(gemm=gemm, small_max_bits=2), dict(gemm=2)):
         p = tn.tn_plan(cfg["circuit"], cfg["open_qubits"], cfg["tails"], cfg["edges"], host_only=True, **kw)

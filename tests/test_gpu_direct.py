@@ -65,6 +65,35 @@ def test_direct_kernel_against_numpy(tn, engine, shape, shift):
     assert np.isnan(rest[:shift]).all() and np.isnan(rest[shift + PC * M * N:]).all()   # nothing past the output
 
 
+@pytest.mark.parametrize("shape", SHAPES, ids=[f"M{s[0]}N{s[1]}K{s[2]}P{s[3]}x{s[4]}x{s[5]}" for s in SHAPES])
+def test_direct_kernel_bf16_products(tn, shape):
+    """The BF16x3 engine on the direct kernel takes that engine's three products
+    of bf16 parts: equal to them in FP64 up to FP32 rounding of three sums."""
+    import torch
+    M, N, K, PA, PB, PC, ma, mb = shape
+    rng = np.random.default_rng(M * 7 + N * 3 + K + PA + 5 * PB + PC)
+    A, B = (rng.normal(size=s) + 1j * rng.normal(size=s) for s in ((PA, M, K), (PB, K, N)))
+    a, b = (torch.from_numpy(x.astype(np.complex64)) for x in (A, B))
+
+    def parts(x):
+        x = torch.view_as_real(x)
+        hi = x.to(torch.bfloat16).to(torch.float32)
+        lo = (x - hi).to(torch.bfloat16).to(torch.float32)
+        return [torch.view_as_complex(y.contiguous()).to(torch.complex128).numpy() for y in (hi, lo)]
+
+    (ah, al), (bh, bl) = parts(a), parts(b)
+    ia = ma if ma is not None else ([0] * PC if PA == 1 else list(range(PC)))
+    ib = mb if mb is not None else ([0] * PC if PB == 1 else list(range(PC)))
+    if K == 2:                      # tf32 steps in every engine: plain products here
+        ah, bh, al, bl = a.numpy().astype(np.complex128), b.numpy().astype(np.complex128), 0 * al, 0 * bl
+    ref = np.stack([ah[i] @ bh[j] + ah[i] @ bl[j] + al[i] @ bh[j] for i, j in zip(ia, ib)])
+    c = torch.full((PC, M, N), float("nan"), dtype=torch.complex64, device="cuda")
+    tn.tn_gemm_c64(a.cuda(), b.cuda(), c, engine=3, map_a=ma, map_b=mb)
+    got = c.cpu().numpy().astype(np.complex128)
+    tol = 2 * (2 * np.sqrt(K) + 4) * 2.0 ** -24
+    assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("engine", [1, 3, 4], ids=["tf32x3", "bf16x3", "fp16x3"])
 @pytest.mark.parametrize("shape", [(512, 64, 256, 5), (256, 32, 128, 7), (512, 16, 64, 9), (256, 8, 32, 20),
                                    (256, 128, 64, 1)], ids=str)
