@@ -229,6 +229,20 @@ __device__ __forceinline__ void store_piece(uint32_t stage, const float* w, floa
   }
 }
 
+// 16 columns of a row where the columns run over patterns of 2^sub (below 16)
+// reals each: C[pattern][row][2^sub].  A warp's 32 rows of a pattern are one
+// stretch of memory, so each lane stores its own row.
+__device__ __forceinline__ void store_patterns(const float* w, float* C, int64_t col, int sub, int64_t M, int64_t row,
+                                               int64_t cols) {
+#pragma unroll
+  for (int e = 0; e < 16; e += 2) {
+    const int64_t c = col + e;
+    if (c >= cols) return;
+    const int64_t pc = c >> sub, n = c & ((1 << sub) - 1);
+    *(float2*)(C + (((pc * M + row) << sub) + n)) = make_float2(w[e], w[e + 1]);
+  }
+}
+
 template <int BN, int STAGES, int KB>
 struct Layout {
   static constexpr int A_BYTES = BM * KB;              // one 128-row tile, KB bytes of K per row
@@ -264,6 +278,7 @@ struct TileGrid {
   int a_shared;
   const uint32_t* grp;                       // or nullptr
   uint32_t n_tiles;
+  int sub_log2;                              // >= 0: the columns are those of many patterns, 2^sub_log2 reals each
 };
 
 __device__ __forceinline__ void tile_coords(const TileGrid& g, uint32_t t, uint32_t& pg, uint32_t& tm, uint32_t& tn) {
@@ -508,6 +523,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         // rows past M and columns past 2N are zero, repeated patterns repeat
 #pragma unroll
         for (int e = 0; e < NCOL; ++e) tmax = fmaxf(tmax, fabsf(acc[e]));
+      }
+      if (grid.sub_log2 >= 0) {
+#pragma unroll
+        for (int pp = 0; pp < NPIECE; ++pp) {
+          float w[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
+          if (lane < rows)
+            store_patterns(w, C, ((int64_t)tn_ << grid.br_log2) + col0 + 16 * pp, grid.sub_log2, M, row0 + lane, N2);
+        }
+        continue;
       }
 #pragma unroll
       for (int pp = 0; pp < NPIECE; ++pp) {
@@ -851,6 +877,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int e = 0; e < NCOL; ++e) tmax = fmaxf(tmax, fabsf(acc[e]));
       }
+      if (grid.sub_log2 >= 0) {
+#pragma unroll
+        for (int pp = 0; pp < NPIECE; ++pp) {
+          float w[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
+          if (lane < rows)
+            store_patterns(w, C, ((int64_t)tn_ << grid.br_log2) + col0 + 16 * pp, grid.sub_log2, M, row0 + lane, N2);
+        }
+        continue;
+      }
 #pragma unroll
       for (int pp = 0; pp < NPIECE; ++pp) {
         const int cl = col0 + 16 * pp;
@@ -971,7 +1008,7 @@ static cudaError_t run(const GemmParams& p, int fold, unsigned int* status, cuda
   if (n_tiles <= 0) return cudaSuccess;
   if (n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   TileGrid grid{(uint32_t)tilesM, (uint32_t)tilesN, (uint32_t)PCg, fold, 0, p.mapA_mode == 1 && p.PC > 1, grp,
-                (uint32_t)n_tiles};
+                (uint32_t)n_tiles, p.sub_log2};
   while ((1 << grid.br_log2) < br) ++grid.br_log2;
   if (p.prepare) {
     const cudaError_t e = set_attr<BN, STAGES, FMT>();
@@ -1022,7 +1059,7 @@ static cudaError_t run_pair(const GemmParams& p, int fold, unsigned int* status,
   if (n_tiles <= 0) return cudaSuccess;
   if (n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   TileGrid grid{(uint32_t)tilesM, (uint32_t)tilesN, (uint32_t)PCg, fold, 0, p.mapA_mode == 1 && p.PC > 1, grp,
-                (uint32_t)n_tiles};
+                (uint32_t)n_tiles, p.sub_log2};
   while ((1 << grid.br_log2) < br) ++grid.br_log2;
   if (p.prepare) {
     const cudaError_t e = set_attr_pair<FMT>();
@@ -1075,6 +1112,17 @@ static cudaError_t dispatch(const GemmParams& q, unsigned int* status, cudaStrea
     p.M *= p.PC;
     p.PA = p.PC = 1;
     p.mapA_mode = 1;
+  }
+  // All patterns share A and each has its own narrow B: the prepared B is one
+  // matrix of all their columns, so this is one GEMM over PC x N columns whose
+  // results go to their patterns.  53 patterns of one column each (2^18 x 2^6)
+  // took 2.4 ms as 53 passes over A.
+  if (p.mapA_mode == 1 && p.mapB_mode == 0 && p.PB == p.PC && p.PC > 1 && 2 * p.N < 16 &&
+      p.PC * p.N <= 0x3fffffffLL && p.tile_cap >= 256) {
+    p.sub_log2 = p.N == 1 ? 1 : p.N == 2 ? 2 : 3;
+    p.N *= p.PC;
+    p.PB = p.PC = 1;
+    p.mapB_mode = 1;
   }
   GemmTile t = gemm_tc_tile(p);
   // Groups of patterns with one A pattern, where a table of them is given, for

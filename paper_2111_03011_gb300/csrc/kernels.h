@@ -108,6 +108,7 @@ struct GemmParams {
   const uint32_t* grp = nullptr;
   int grp_fold = 0;
   int64_t n_groups = 0;
+  int sub_log2 = -1;     // set by the dispatch: the columns are many patterns', 2^sub_log2 reals each
   int prepare = 0;       // 1: set the launched kernel's attributes first (no plan upload did)
 };
 

@@ -950,8 +950,13 @@ static std::vector<uint32_t> group_patterns(const std::vector<uint32_t>& mapA, i
 // its tiles of 128 rows x BN real columns in whole waves of 152, each SM at
 // its share of 280 (3xTF32) or 560 (16-bit) TFLOP/s for BN >= 256, where an
 // MMA narrower than 128 columns takes as long as one of 128.
-double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, double a, double b, double c, bool h16) {
+double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, bool b_own, double a, double b, double c,
+                  bool h16) {
   int64_t cols = 2LL << nn, groups = PC;
+  if (a_shared && b_own && cols < 16 && PC > 1) {   // one matrix of all patterns' columns
+    cols *= PC;
+    groups = 1;
+  }
   if (a_shared && cols >= 16)
     while (cols < 256 && groups > 1) {
       cols *= 2;
@@ -1059,7 +1064,7 @@ static int layout_steps(Plan& plan, std::string& err) {
         if (d.seconds < dp.seconds) dp = d;
       }
     }
-    const bool direct = dp.seconds < tc_seconds(nm, nn, nk, C.P, mapA_mode == 1, (double)vt_elems(big),
+    const bool direct = dp.seconds < tc_seconds(nm, nn, nk, C.P, mapA_mode == 1, mapB_mode == 0, (double)vt_elems(big),
                                                 (double)vt_elems(sml), (double)C.P * std::exp2(nm + nn), h16_step);
     if (use_small || (direct && !dp.swap)) {
       for (int l : M) cl.push_back(l);

@@ -231,8 +231,10 @@ struct PlanInput {
 };
 
 // Modelled time of a contraction as split permute, B preparation and
-// tensor-core GEMM (a, b, c: elements of the operands and the result).
-double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, double a, double b, double c, bool h16);
+// tensor-core GEMM (a, b, c: elements of the operands and the result; b_own:
+// every pattern has its own B, in order).
+double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, bool b_own, double a, double b, double c,
+                  bool h16);
 int build_plan(const PlanInput& in, Plan& plan, std::string& err);
 void apply_perm_schedule(Step& s, const PermSched& ps);
 std::string describe_plan(const Plan& plan, bool with_data);
