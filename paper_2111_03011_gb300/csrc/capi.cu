@@ -259,7 +259,6 @@ static int plan_upload(tn_plan_t* p) {
   if (tn::fault_alloc()) return fail(TN_ERR_OOM, "device allocation failed (injected: TN_FAULT_INJECT=alloc)");
   CUDA_TRY(cudaGetDevice(&p->device));
   CUDA_TRY(tn::prepare_gemm_tc());
-  CUDA_TRY(tn::prepare_permute());
   CUDA_TRY(tn::prepare_direct());
   std::vector<float2> leaves(P.leaf_arena.size());
   for (size_t i = 0; i < leaves.size(); ++i)

@@ -118,11 +118,16 @@ cudaError_t launch_small(const SmallParams& p, cudaStream_t s) {
 // preimages of the output's low bits (grown to 10 bits with further input
 // bits); it is read with the input's contiguous order and written with the
 // output's, through shared memory.  The tile is padded by one element per 32 so
-// that the strided reads of the write phase fall into different banks.  The
+// that the strided reads of the write phase fall into different banks.
+// Every index table is OR-linear in the tile index (a bit goes to a position),
+// and the padding is additive over disjoint bits, so a thread keeps the entries
+// of its own index in registers and adds those of 256, 512 and 768, which are
+// the same for all threads: no table is read per element, and the shared memory
+// holds tiles only, so that eight CTAs fit an SM instead of four.  The
 // tile's base addresses (the remaining "rest" bits of the tile index scattered
-// to their positions) come from one 256-entry table per byte of the rest bits
-// and direction (only as many as n_rest needs, to keep shared memory small and
-// more blocks, hence more loads, in flight per SM).
+// to their positions) are a warp-wide OR, lane j placing bit j.
+// 2^25 elements, split to bf16 planes: 104-119 us with the tables in shared
+// memory, now 82-91 us (5.9-6.6 TB/s); 2^29: 1,857 -> 1,391 us.
 // SPLIT 1: the output is written as two fp32 planes, tf32-rounded hi and the
 // remainder lo; SPLIT 2: two bf16 planes, bf16 hi and the bf16-rounded
 // remainder; SPLIT 3: two fp16 planes of the value times the operand's power-
@@ -153,8 +158,7 @@ __device__ __forceinline__ void cp_async_wait() {
 // kPermBufs - 1 are in flight.
 constexpr int kPermBufs = 3;
 
-__host__ __device__ inline int perm_levels(int n_rest) { return n_rest > 0 ? (n_rest + 7) >> 3 : 1; }
-// float2 per buffer, even so that the index tables after the buffers start on 16 bytes
+// float2 per buffer
 __host__ __device__ inline int perm_tile_stride(int nt) { return (nt + (nt >> 5) + 3) & ~1; }
 
 // Four consecutive outputs of one plane as one 16-byte store (16-bit formats)
@@ -203,62 +207,106 @@ struct Pair<2> {
   }
 };
 
+// One element v at output index o (of all patterns), in the form SPLIT.
+template <int SPLIT>
+__device__ __forceinline__ void perm_store(const PermParams& p, int64_t planes, float2 v, int64_t o, float sc) {
+  if constexpr (SPLIT >= 4) {
+    // the tensor-core B operand: output index o = k + K n of a pattern
+    // becomes the 2 x 2 block [[re, -im], [im, re]] at pairs (2k, 2k+1)
+    // of rows 2n and 2n + 1 of the [2N][2K] real embedding
+    using PT = Pair<SPLIT - 4>;
+    using T = typename PT::T;
+    T* hi = (T*)p.out;
+    T* lo = hi + 2 * planes;
+    const int64_t K = 1LL << p.embed_nk;
+    const int64_t e0 = 2 * o - (o & (K - 1));
+    T h, l;
+    PT::split(v.x, -v.y, sc, h, l);
+    hi[e0] = h;
+    lo[e0] = l;
+    PT::split(v.y, v.x, sc, h, l);
+    hi[e0 + K] = h;
+    lo[e0 + K] = l;
+  } else if constexpr (SPLIT >= 1) {
+    using PT = Pair<SPLIT - 1>;
+    using T = typename PT::T;
+    T* hi = (T*)p.out;
+    T h, l;
+    PT::split(v.x, v.y, sc, h, l);
+    hi[o] = h;
+    hi[planes + o] = l;
+  } else {
+    p.out[o] = v;
+  }
+}
+
 template <int SPLIT>
 __global__ void __launch_bounds__(256) k_permute(PermParams p) {
   extern __shared__ float2 tile[];
+  const int tid = threadIdx.x, lane = tid & 31;
   const int nt = 1 << p.t;
   const int tstride = perm_tile_stride(nt);
-  uint32_t* s_in = (uint32_t*)(tile + kPermBufs * tstride);
-  uint32_t* s_out = s_in + nt;
-  uint32_t* s_slot = s_out + nt;
-  const int levels = perm_levels(p.n_rest);
-  uint64_t* r_in = (uint64_t*)(((uintptr_t)(s_slot + nt) + 7) & ~(uintptr_t)7);   // [levels][256]
-  uint64_t* r_out = r_in + 256 * levels;
-  for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-    s_in[i] = __ldg(p.tab + i);
-    s_out[i] = __ldg(p.tab + nt + i);
-    s_slot[i] = (uint32_t)pad32((int)__ldg(p.tab + 2 * nt + i));
+  const int ne = nt >> 8;                   // elements per thread (0: fewer than 256, one for the first nt threads)
+  // this thread's tile index and, uniform, the steps by 256 and 512 (their sum is that by 768)
+  uint32_t in0 = 0, out0 = 0, slot0 = 0, in1 = 0, in2 = 0, out1 = 0, out2 = 0, slot1 = 0, slot2 = 0;
+  const bool v4 = SPLIT < 4 && p.vec4;
+  // four-outputs form: thread g takes outputs 4g .. 4g + 3 of the tile
+  const int j0 = v4 ? 4 * tid : tid;
+  if (tid < nt) in0 = __ldg(p.tab + tid);
+  if (j0 < nt) {
+    out0 = __ldg(p.tab + nt + j0);
+    slot0 = (uint32_t)pad32((int)__ldg(p.tab + 2 * nt + j0));
   }
-  for (int e = threadIdx.x; e < 256 * levels; e += blockDim.x) {
-    const int level = e >> 8, v = e & 255;
-    uint64_t bi = 0, bo = 0;
-    for (int k = 0; k < 8; ++k) {
-      const int bit = level * 8 + k;
-      if (bit < p.n_rest && ((v >> k) & 1)) {
-        bi |= 1ULL << p.rest_in[bit];
-        bo |= 1ULL << p.rest_out[bit];
-      }
+  if (p.t > 8) in1 = __ldg(p.tab + 256);
+  if (p.t > 9) in2 = __ldg(p.tab + 512);
+  if (v4) {
+    slot1 = (uint32_t)pad32((int)__ldg(p.tab + 2 * nt + 1));
+    slot2 = (uint32_t)pad32((int)__ldg(p.tab + 2 * nt + 2));
+  } else {
+    if (p.t > 8) {
+      out1 = __ldg(p.tab + nt + 256);
+      slot1 = (uint32_t)pad32((int)__ldg(p.tab + 2 * nt + 256));
     }
-    r_in[e] = bi;
-    r_out[e] = bo;
+    if (p.t > 9) {
+      out2 = __ldg(p.tab + nt + 512);
+      slot2 = (uint32_t)pad32((int)__ldg(p.tab + 2 * nt + 512));
+    }
   }
-  __syncthreads();  // the tables are read below
+  // lane j: where bit j of a tile's index goes in the input and in the output
+  uint64_t bit_in = 0, bit_out = 0;
+  if (lane < p.n_rest) {
+    bit_in = 1ULL << p.rest_in[lane];
+    bit_out = 1ULL << p.rest_out[lane];
+  }
   const uint64_t nrest_mask = (1ULL << p.n_rest) - 1;
   const uint64_t total_tiles = (uint64_t)p.P << p.n_rest;
-  float2* __restrict__ out_lo = p.out + p.P * p.pstride;
+  const int64_t planes = p.P * p.pstride;
   const float sc = (SPLIT == 3 || SPLIT == 6) ? pow2f(fp16_scale_exp(*p.scale)) : 1.0f;
-  // input and output base offsets of tile blk: the pattern's stride plus the
-  // rest bits of the tile index scattered through the per-byte tables
-  auto tile_base = [&](uint64_t blk, int64_t& iofs, int64_t& dofs) {
-    const uint64_t pp = blk >> p.n_rest, b = blk & nrest_mask;
-    uint64_t bi = 0, bo = 0;
-    for (int l = 0; l < levels; ++l) {
-      const int v = (int)((b >> (8 * l)) & 255);
-      bi |= r_in[256 * l + v];
-      bo |= r_out[256 * l + v];
-    }
-    iofs = (int64_t)(pp * p.pstride + bi);
-    dofs = (int64_t)(pp * p.pstride + bo);
+  auto scatter = [&](uint32_t b, uint64_t bit) -> uint64_t {
+    const uint64_t v = (b >> lane) & 1u ? bit : 0ULL;
+    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v);
+    const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
+    return ((uint64_t)hi << 32) | lo;
   };
   // issue the copies of tile blk into buffer buf (an empty group past the
   // end keeps the group count uniform)
+  const uint32_t dst0 = (uint32_t)pad32(tid);
   auto issue = [&](uint64_t blk, int buf) {
     if (blk < total_tiles) {
-      int64_t iofs, dofs;
-      tile_base(blk, iofs, dofs);
-      const float2* src = p.in + iofs;
-      float2* dst = tile + buf * tstride;
-      for (int i = threadIdx.x; i < nt; i += blockDim.x) cp_async8(dst + pad32(i), src + s_in[i]);
+      const uint64_t pp = blk >> p.n_rest;
+      const float2* src = p.in + (pp * p.pstride + scatter((uint32_t)(blk & nrest_mask), bit_in)) + in0;
+      float2* dst = tile + buf * tstride + dst0;
+      if (ne == 4) {
+        cp_async8(dst, src);
+        cp_async8(dst + 264, src + in1);
+        cp_async8(dst + 528, src + in2);
+        cp_async8(dst + 792, src + in1 + in2);
+      } else if (ne == 2) {
+        cp_async8(dst, src);
+        cp_async8(dst + 264, src + in1);
+      } else if (tid < nt) {
+        cp_async8(dst, src);
+      }
     }
     cp_async_commit();
   };
@@ -269,102 +317,46 @@ __global__ void __launch_bounds__(256) k_permute(PermParams p) {
     cp_async_wait<kPermBufs - 2>();   // this thread's copies of tile blk are done
     __syncthreads();                  // ... and everyone's; the buffer written out last round is free
     issue(blk + (uint64_t)(kPermBufs - 1) * gridDim.x, (buf + kPermBufs - 1) % kPermBufs);
-    int64_t iofs, cur_dofs;
-    tile_base(blk, iofs, cur_dofs);
-    const float2* t = tile + buf * tstride;
+    const uint64_t pp = blk >> p.n_rest;
+    const int64_t o = (int64_t)(pp * p.pstride + scatter((uint32_t)(blk & nrest_mask), bit_out)) + out0;
+    const float2* t = tile + buf * tstride + slot0;
     buf = (buf + 1) % kPermBufs;
-    if (SPLIT < 4 && p.vec4) {
-      // output bits 0 and 1 are tile bits 0 and 1: outputs 4g .. 4g + 3 of
-      // the tile are consecutive in memory, from a 4-aligned index.  Fewer,
-      // wider stores, but each warp's shared-memory reads take other tile
-      // bits than in the loop below, so which is faster depends on the
-      // permutation: a schedule variant of its own, chosen by timing.
-      for (int g = threadIdx.x; g < (nt >> 2); g += blockDim.x) {
-        const uint4 sl = *(const uint4*)(s_slot + 4 * g);
-        const int64_t o = cur_dofs + s_out[4 * g];
-        const float2 v0 = t[sl.x], v1 = t[sl.y], v2 = t[sl.z], v3 = t[sl.w];
-        if (SPLIT == 1) {
-          const float2 h0 = make_float2(tf32_rn(v0.x), tf32_rn(v0.y)), h1 = make_float2(tf32_rn(v1.x), tf32_rn(v1.y));
-          const float2 h2 = make_float2(tf32_rn(v2.x), tf32_rn(v2.y)), h3 = make_float2(tf32_rn(v3.x), tf32_rn(v3.y));
-          store4(p.out + o, h0, h1, h2, h3);
-          store4(out_lo + o, make_float2(v0.x - h0.x, v0.y - h0.y), make_float2(v1.x - h1.x, v1.y - h1.y),
-                 make_float2(v2.x - h2.x, v2.y - h2.y), make_float2(v3.x - h3.x, v3.y - h3.y));
-        } else if (SPLIT == 3) {
-          __half2* fh = (__half2*)p.out;
-          __half2* fl = fh + p.P * p.pstride;
-          __half2 h[4], l[4];
-          const float2 v[4] = {v0, v1, v2, v3};
+    if constexpr (SPLIT < 4) {
+      if (v4) {
+        // output bits 0 and 1 are tile bits 0 and 1: outputs 4g .. 4g + 3 of
+        // the tile are consecutive in memory, from a 4-aligned index.  Fewer,
+        // wider stores, but each warp's shared-memory reads take other tile
+        // bits than in the other form, so which is faster depends on the
+        // permutation: a schedule variant of its own, chosen by timing.
+        if (j0 < nt) {
+          const float2 v[4] = {t[0], t[slot1], t[slot2], t[slot1 + slot2]};
+          if constexpr (SPLIT == 0) {
+            store4(p.out + o, v[0], v[1], v[2], v[3]);
+          } else {
+            using PT = Pair<SPLIT - 1>;
+            using T = typename PT::T;
+            T h[4], l[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 w = make_float2(v[e].x * sc, v[e].y * sc);
-            h[e] = __floats2half2_rn(w.x, w.y);
-            const float2 hf = __half22float2(h[e]);
-            l[e] = __floats2half2_rn(w.x - hf.x, w.y - hf.y);
+            for (int e = 0; e < 4; ++e) PT::split(v[e].x, v[e].y, sc, h[e], l[e]);
+            store4((T*)p.out + o, h[0], h[1], h[2], h[3]);
+            store4((T*)p.out + planes + o, l[0], l[1], l[2], l[3]);
           }
-          store4(fh + o, h[0], h[1], h[2], h[3]);
-          store4(fl + o, l[0], l[1], l[2], l[3]);
-        } else if (SPLIT == 2) {
-          __nv_bfloat162* bh = (__nv_bfloat162*)p.out;
-          __nv_bfloat162* bl = bh + p.P * p.pstride;
-          __nv_bfloat162 h[4], l[4];
-          const float2 v[4] = {v0, v1, v2, v3};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            h[e] = __floats2bfloat162_rn(v[e].x, v[e].y);
-            const float2 hf = __bfloat1622float2(h[e]);
-            l[e] = __floats2bfloat162_rn(v[e].x - hf.x, v[e].y - hf.y);
-          }
-          store4(bh + o, h[0], h[1], h[2], h[3]);
-          store4(bl + o, l[0], l[1], l[2], l[3]);
-        } else {
-          store4(p.out + o, v0, v1, v2, v3);
         }
+        continue;
       }
-      continue;
     }
-#pragma unroll 4
-    for (int j = threadIdx.x; j < nt; j += blockDim.x) {
-      const float2 v = t[s_slot[j]];
-      const int64_t o = cur_dofs + s_out[j];
-      if constexpr (SPLIT >= 4) {
-        // the tensor-core B operand: output index o = k + K n of a pattern
-        // becomes the 2 x 2 block [[re, -im], [im, re]] at pairs (2k, 2k+1)
-        // of rows 2n and 2n + 1 of the [2N][2K] real embedding
-        using PT = Pair<SPLIT - 4>;
-        using T = typename PT::T;
-        T* hi = (T*)p.out;
-        T* lo = hi + 2 * p.P * p.pstride;
-        const int64_t K = 1LL << p.embed_nk;
-        const int64_t e0 = 2 * o - (o & (K - 1));
-        T h, l;
-        PT::split(v.x, -v.y, sc, h, l);
-        hi[e0] = h;
-        lo[e0] = l;
-        PT::split(v.y, v.x, sc, h, l);
-        hi[e0 + K] = h;
-        lo[e0 + K] = l;
-      } else if (SPLIT == 1) {
-        const float2 h = make_float2(tf32_rn(v.x), tf32_rn(v.y));
-        p.out[o] = h;
-        out_lo[o] = make_float2(v.x - h.x, v.y - h.y);
-      } else if (SPLIT == 3) {
-        __half2* fh = (__half2*)p.out;
-        __half2* fl = fh + p.P * p.pstride;
-        const float2 w = make_float2(v.x * sc, v.y * sc);
-        const __half2 h = __floats2half2_rn(w.x, w.y);
-        const float2 hf = __half22float2(h);
-        fh[o] = h;
-        fl[o] = __floats2half2_rn(w.x - hf.x, w.y - hf.y);
-      } else if (SPLIT == 2) {
-        __nv_bfloat162* bh = (__nv_bfloat162*)p.out;
-        __nv_bfloat162* bl = bh + p.P * p.pstride;
-        const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
-        const float2 hf = __bfloat1622float2(h);
-        bh[o] = h;
-        bl[o] = __floats2bfloat162_rn(v.x - hf.x, v.y - hf.y);
-      } else {
-        p.out[o] = v;
-      }
+    if (ne == 4) {
+      const float2 a = t[0], b = t[slot1], c = t[slot2], d = t[slot1 + slot2];
+      perm_store<SPLIT>(p, planes, a, o, sc);
+      perm_store<SPLIT>(p, planes, b, o + out1, sc);
+      perm_store<SPLIT>(p, planes, c, o + out2, sc);
+      perm_store<SPLIT>(p, planes, d, o + out1 + out2, sc);
+    } else if (ne == 2) {
+      const float2 a = t[0], b = t[slot1];
+      perm_store<SPLIT>(p, planes, a, o, sc);
+      perm_store<SPLIT>(p, planes, b, o + out1, sc);
+    } else if (tid < nt) {
+      perm_store<SPLIT>(p, planes, t[0], o, sc);
     }
   }
   cp_async_wait<0>();
@@ -398,33 +390,14 @@ cudaError_t launch_absmax(const AbsmaxParams& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Largest dynamic shared memory of a permute launch: kPermBufs tiles of 2^10
-// elements, the three 2^10-entry index tables and four levels of rest-bit
-// tables (about 54 KB), above the 48 KB a launch gets without opting in.
-static size_t perm_smem(int t, int n_rest) {
-  const int nt = 1 << t;
-  return sizeof(float2) * (size_t)kPermBufs * perm_tile_stride(nt) + 3 * sizeof(uint32_t) * (size_t)nt + 8 +
-         2 * 256 * (size_t)perm_levels(n_rest) * sizeof(uint64_t);
-}
-
-cudaError_t prepare_permute() {
-  const int mx = (int)perm_smem(10, 32);
-  cudaError_t e = cudaFuncSetAttribute(k_permute<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_permute<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_permute<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_permute<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_permute<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_permute<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_permute<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  return e;
-}
+static size_t perm_smem(int t) { return sizeof(float2) * (size_t)kPermBufs * perm_tile_stride(1 << t); }
 
 cudaError_t launch_permute(const PermParams& p, cudaStream_t s) {
   if (p.n_rest > 32) return cudaErrorInvalidValue;
   const int64_t blocks = (1LL << p.n_rest) * p.P;
   const int64_t grid = std::min<int64_t>(blocks, (int64_t)kSMs * 8);
   if (p.t < 0 || p.t > 10) return cudaErrorInvalidValue;
-  const size_t smem = perm_smem(p.t, p.n_rest);
+  const size_t smem = perm_smem(p.t);
   if (p.split == 1) k_permute<1><<<(unsigned)grid, 256, smem, s>>>(p);
   else if (p.split == 2) k_permute<2><<<(unsigned)grid, 256, smem, s>>>(p);
   else if (p.split == 3) k_permute<3><<<(unsigned)grid, 256, smem, s>>>(p);

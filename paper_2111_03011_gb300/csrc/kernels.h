@@ -163,7 +163,6 @@ cudaError_t launch_gemm_tc(const GemmParams& p, unsigned int* status, cudaStream
 cudaError_t prepare_gemm_tc();   // kernel attributes; call before launching or capturing
 cudaError_t launch_direct(const DirectParams& p, int config, cudaStream_t s, bool prepare = false);
 cudaError_t prepare_direct();    // the direct step's opt-in shared-memory sizes; likewise
-cudaError_t prepare_permute();   // the permute's opt-in shared-memory size; likewise
 
 // What a head operation reports to the host, in mapped host memory.  The host
 // sets `missing` to ~0 and `word` to 0 before the launch.
