@@ -140,7 +140,9 @@ typedef struct {
   int     n_pinned;           /* PIN edges (each halves F_est) */
   int     n_leaves;           /* device leaves: tensors left after host simplification and folding */
   int     n_contractions;     /* pairwise contractions per slice */
-  int     n_launches;         /* kernel launches per slice (steps incl. permutes/prep + accumulate) */
+  int     n_launches;         /* steps of a slice's launch list (permutes, preparations, accumulate);
+                                 a GEMM's two preparations share a launch, and streaming steps near
+                                 the leaves one for several slices of a range */
   double  tc_macs;            /* T_c: complex multiply-adds per slice (algorithmic) */
   double  alg_bytes;          /* algorithmic HBM bytes per slice (each operand read once, result written once) */
   double  max_log2_elements;  /* largest intermediate */

@@ -566,6 +566,52 @@ static void batch_range(const tn_plan_t* p, int64_t q0, int n, tn::BatchParams& 
   q.amax_stride = p->P.n_scale_slots;
 }
 
+// Launch parameters of a permute step (for a B preparation in the permute form:
+// of its schedule) and of a B preparation by gather.
+static tn::PermParams perm_params(const tn_plan_t* p, const tn::Step& x, int64_t s, int b) {
+  tn::PermParams pp;
+  pp.in = ref_ptr(p, x.a, s, b);
+  pp.out = buf_ptr(p, x.c, b);
+  pp.pstride = 1LL << x.rA;
+  pp.P = x.PA;
+  pp.t = x.t_bits;
+  pp.n_rest = x.n_rest;
+  std::memcpy(pp.rest_in, x.rest_in, sizeof(pp.rest_in));
+  std::memcpy(pp.rest_out, x.rest_out, sizeof(pp.rest_out));
+  pp.tab = p->d_meta + x.tab_off;
+  pp.split = x.split;
+  pp.scale = scale_ptr(p, x.slot, b);
+  pp.vec4 = x.vec4;
+  return pp;
+}
+
+static tn::BPrepParams bprep_params(const tn_plan_t* p, const tn::Step& x, int64_t s, int b) {
+  tn::BPrepParams bp;
+  bp.B = ref_ptr(p, x.a, s, b);
+  bp.out = buf_ptr(p, x.c, b);
+  bp.b_pstride = 1LL << x.rA;
+  bp.PB = x.PA;
+  bp.nk = x.nk;
+  bp.nn = x.nn;
+  bp.bk = p->d_meta + x.bk_off;
+  bp.bn = p->d_meta + x.bn_off;
+  bp.h16 = x.h16;
+  bp.scale = scale_ptr(p, x.slot, b);
+  return bp;
+}
+
+static bool bprep_embeds(const tn::Step& x) {
+  return x.kind == tn::ST_BPREP_TC && !x.alts.empty() && (x.variant == 0) == (x.bprep_embed0 != 0);
+}
+
+// Whether the permute step x and the step y after it are the two operands of one
+// GEMM that launch_operands prepares together (y does not read x's result: it
+// prepares the other operand).
+static bool joined_operands(const tn::Step& x, const tn::Step& y) {
+  return x.kind == tn::ST_PERMUTE && x.split >= 1 && y.kind == tn::ST_BPREP_TC && y.h16 + 1 == x.split &&
+         y.contraction == x.contraction && y.fork < 0 && !bprep_embeds(y);
+}
+
 // Launch one step of the launch list for the full slice id s on stream st
 // (`side`: a B-prep beside a running GEMM, launched with one block per SM); b is
 // the pass's place in its chunk.  n_batch > 1: a batched step, for the passes
@@ -633,53 +679,21 @@ static cudaError_t launch_step(tn_plan_t* p, const tn::Step& x, int64_t s, cudaS
       break;
     }
     case tn::ST_PERMUTE: {
-      tn::PermParams pp;
-      pp.in = ref_ptr(p, x.a, s, b);
-      pp.out = buf_ptr(p, x.c, b);
-      pp.pstride = 1LL << x.rA;
-      pp.P = x.PA;
-      pp.t = x.t_bits;
-      pp.n_rest = x.n_rest;
-      std::memcpy(pp.rest_in, x.rest_in, sizeof(pp.rest_in));
-      std::memcpy(pp.rest_out, x.rest_out, sizeof(pp.rest_out));
-      pp.tab = p->d_meta + x.tab_off;
-      pp.split = x.split;
-      pp.scale = scale_ptr(p, x.slot, b);
-      pp.vec4 = x.vec4;
+      const tn::PermParams pp = perm_params(p, x, s, b);
       e = tn::launch_permute(pp, st);
       break;
     }
     case tn::ST_BPREP_C:
     case tn::ST_BPREP_TC: {
-      if (x.kind == tn::ST_BPREP_TC && !x.alts.empty() && (x.variant == 0) == (x.bprep_embed0 != 0)) {
+      if (bprep_embeds(x)) {
         // the permute kernel onto [N][K] order, writing the real embedding
-        tn::PermParams pp;
-        pp.in = ref_ptr(p, x.a, s, b);
-        pp.out = buf_ptr(p, x.c, b);
-        pp.pstride = 1LL << x.rA;
-        pp.P = x.PA;
-        pp.t = x.t_bits;
-        pp.n_rest = x.n_rest;
-        std::memcpy(pp.rest_in, x.rest_in, sizeof(pp.rest_in));
-        std::memcpy(pp.rest_out, x.rest_out, sizeof(pp.rest_out));
-        pp.tab = p->d_meta + x.tab_off;
+        tn::PermParams pp = perm_params(p, x, s, b);
         pp.split = 4 + x.h16;
-        pp.scale = scale_ptr(p, x.slot, b);
         pp.embed_nk = x.nk;
         e = tn::launch_permute(pp, st);
         break;
       }
-      tn::BPrepParams bp;
-      bp.B = ref_ptr(p, x.a, s, b);
-      bp.out = buf_ptr(p, x.c, b);
-      bp.b_pstride = 1LL << x.rA;
-      bp.PB = x.PA;
-      bp.nk = x.nk;
-      bp.nn = x.nn;
-      bp.bk = p->d_meta + x.bk_off;
-      bp.bn = p->d_meta + x.bn_off;
-      bp.h16 = x.h16;
-      bp.scale = scale_ptr(p, x.slot, b);
+      const tn::BPrepParams bp = bprep_params(p, x, s, b);
       e = x.kind == tn::ST_BPREP_C ? tn::launch_bprep_c(bp, st) : tn::launch_bprep_tc(bp, st, side);
       break;
     }
@@ -787,6 +801,11 @@ static int run_pass(tn_plan_t* p, int64_t s, double2* H, cudaStream_t st, cudaEv
       // launched on the side stream before step x.fork: wait for it here
       e = cudaStreamWaitEvent(st, p->side_join[si], 0);
       pending.erase(std::remove(pending.begin(), pending.end(), si), pending.end());
+    } else if (!ev && si > 0 && joined_operands(P.steps[si - 1], x)) {
+      // launched with the permute before it
+    } else if (!ev && si + 1 < (int)P.steps.size() && joined_operands(x, P.steps[si + 1])) {
+      NvtxRange range("tn operands");
+      e = tn::launch_operands(perm_params(p, x, s, b), bprep_params(p, P.steps[si + 1], s, b), st);
     } else {
       e = launch_step(p, x, s, st, false, b);
     }

@@ -207,6 +207,59 @@ struct Pair<2> {
   }
 };
 
+// Real embedding of B for C_r = A_r B_r with interleaved complex rows:
+// Bt[j][i] (j = 2n + jc output column, i = 2k + ic reduction index) is
+// [[re, -im], [im, re]] in (jc, ic); stored K-major as hi and lo planes in the
+// GEMM engine's operand format (FMT 0: tf32-rounded fp32 hi + fp32 remainder;
+// 1: bf16 hi + bf16 remainder; 2: fp16 of the value times the scale sc).  One
+// thread per complex element of B: it writes the element's 2 x 2 block as two
+// pairs of adjacent reals (rows 2n and 2n + 1) in each plane; consecutive
+// threads take consecutive k, so every row segment is written contiguously.
+// Its loads coalesce only when B's K legs are its low bits; otherwise the
+// plan prepares B with the permute kernel in an embedding mode (split 4-6),
+// which reads through a shared-memory tile.
+template <int FMT>
+__device__ __forceinline__ void bprep_tc(const BPrepParams& p, int64_t block, int64_t blocks) {
+  using T = typename Pair<FMT>::T;
+  const int64_t K = 1LL << p.nk, N = 1LL << p.nn;
+  const int64_t per = K * N;                  // complex elements per pattern
+  const int64_t total = p.PB * per;
+  T* hi = (T*)p.out;                          // pairs: [PB][2N][K] pairs of reals
+  T* lo = hi + 2 * total;
+  const float sc = FMT == 2 ? pow2f(fp16_scale_exp(*p.scale)) : 1.0f;
+  // kU elements per thread and round, their loads issued before any store,
+  // so that a grid of one block per SM (beside a running GEMM) still keeps
+  // enough loads in flight
+  constexpr int kU = 4;
+  const int64_t stride = blocks * 256;
+  for (int64_t e0 = block * 256 + threadIdx.x; e0 < total; e0 += kU * stride) {
+    float2 b[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t e = e0 + u * stride;
+      if (e < total) {
+        const int64_t pb = e / per, r = e - pb * per;
+        b[u] = p.B[pb * p.b_pstride + p.bk[r & (K - 1)] + p.bn[r >> p.nk]];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t e = e0 + u * stride;
+      if (e >= total) break;
+      const int64_t pb = e / per, r = e - pb * per;
+      const int64_t n = r >> p.nk, k = r & (K - 1);
+      const int64_t o0 = (pb * 2 * N + 2 * n) * K + k;   // pair (2k, 2k+1) of row 2n
+      T h, l;
+      Pair<FMT>::split(b[u].x, -b[u].y, sc, h, l);
+      hi[o0] = h;
+      lo[o0] = l;
+      Pair<FMT>::split(b[u].y, b[u].x, sc, h, l);
+      hi[o0 + K] = h;                                    // row 2n + 1
+      lo[o0 + K] = l;
+    }
+  }
+}
+
 // One element v at output index o (of all patterns), in the form SPLIT.
 template <int SPLIT>
 __device__ __forceinline__ void perm_store(const PermParams& p, int64_t planes, float2 v, int64_t o, float sc) {
@@ -241,7 +294,7 @@ __device__ __forceinline__ void perm_store(const PermParams& p, int64_t planes, 
 }
 
 template <int SPLIT>
-__global__ void __launch_bounds__(256) k_permute(PermParams p) {
+__device__ __forceinline__ void permute(const PermParams& p, uint32_t block, uint32_t blocks) {
   extern __shared__ float2 tile[];
   const int tid = threadIdx.x, lane = tid & 31;
   const int nt = 1 << p.t;
@@ -311,12 +364,12 @@ __global__ void __launch_bounds__(256) k_permute(PermParams p) {
     cp_async_commit();
   };
 #pragma unroll
-  for (int k = 0; k < kPermBufs - 1; ++k) issue((uint64_t)blockIdx.x + (uint64_t)k * gridDim.x, k);
+  for (int k = 0; k < kPermBufs - 1; ++k) issue((uint64_t)block + (uint64_t)k * blocks, k);
   int buf = 0;
-  for (uint64_t blk = blockIdx.x; blk < total_tiles; blk += gridDim.x) {
+  for (uint64_t blk = block; blk < total_tiles; blk += blocks) {
     cp_async_wait<kPermBufs - 2>();   // this thread's copies of tile blk are done
     __syncthreads();                  // ... and everyone's; the buffer written out last round is free
-    issue(blk + (uint64_t)(kPermBufs - 1) * gridDim.x, (buf + kPermBufs - 1) % kPermBufs);
+    issue(blk + (uint64_t)(kPermBufs - 1) * blocks, (buf + kPermBufs - 1) % kPermBufs);
     const uint64_t pp = blk >> p.n_rest;
     const int64_t o = (int64_t)(pp * p.pstride + scatter((uint32_t)(blk & nrest_mask), bit_out)) + out0;
     const float2* t = tile + buf * tstride + slot0;
@@ -360,6 +413,20 @@ __global__ void __launch_bounds__(256) k_permute(PermParams p) {
     }
   }
   cp_async_wait<0>();
+}
+
+template <int SPLIT>
+__global__ void __launch_bounds__(256) k_permute(PermParams p) {
+  permute<SPLIT>(p, blockIdx.x, gridDim.x);
+}
+
+// Both operands of a tensor-core GEMM in one launch: the first CTAs prepare B
+// (they are few and start first), the others permute and split A.  The two have
+// nothing to wait for in each other, and a small B's gather hides under A's.
+template <int FMT>
+__global__ void __launch_bounds__(256) k_operands(PermParams a, BPrepParams b, uint32_t blocks_b) {
+  if (blockIdx.x < blocks_b) bprep_tc<FMT>(b, blockIdx.x, blocks_b);
+  else permute<FMT + 1>(a, blockIdx.x - blocks_b, gridDim.x - blocks_b);
 }
 
 // Scale slot of the FP16x3 engine: max over the operand of |re| and |im|.
@@ -408,6 +475,19 @@ cudaError_t launch_permute(const PermParams& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+cudaError_t launch_operands(const PermParams& a, const BPrepParams& b, cudaStream_t s) {
+  if (a.n_rest > 32 || a.t < 0 || a.t > 10 || a.split != b.h16 + 1) return cudaErrorInvalidValue;
+  const int64_t total = b.PB << (b.nk + b.nn);
+  const uint32_t blocks_b = (uint32_t)std::max<int64_t>(std::min<int64_t>((total + 1023) / 1024, kSMs * 4), 1);
+  const uint32_t blocks_a = (uint32_t)std::min<int64_t>((1LL << a.n_rest) * a.P, (int64_t)kSMs * 8);
+  const dim3 grid(blocks_a + blocks_b);
+  const size_t smem = perm_smem(a.t);
+  if (b.h16 == 2) k_operands<2><<<grid, 256, smem, s>>>(a, b, blocks_b);
+  else if (b.h16 == 1) k_operands<1><<<grid, 256, smem, s>>>(a, b, blocks_b);
+  else k_operands<0><<<grid, 256, smem, s>>>(a, b, blocks_b);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ B prep
 __global__ void k_bprep_c(BPrepParams p) {
   const int64_t K = 1LL << p.nk, N = 1LL << p.nn;
@@ -420,57 +500,9 @@ __global__ void k_bprep_c(BPrepParams p) {
   }
 }
 
-// Real embedding of B for C_r = A_r B_r with interleaved complex rows:
-// Bt[j][i] (j = 2n + jc output column, i = 2k + ic reduction index) is
-// [[re, -im], [im, re]] in (jc, ic); stored K-major as hi and lo planes in the
-// GEMM engine's operand format (FMT 0: tf32-rounded fp32 hi + fp32 remainder;
-// 1: bf16 hi + bf16 remainder; 2: fp16 of the value times the scale sc).  One
-// thread per complex element of B: it writes the element's 2 x 2 block as two
-// pairs of adjacent reals (rows 2n and 2n + 1) in each plane; consecutive
-// threads take consecutive k, so every row segment is written contiguously.
-// Its loads coalesce only when B's K legs are its low bits; otherwise the
-// plan prepares B with the permute kernel in an embedding mode (split 4-6),
-// which reads through a shared-memory tile.
 template <int FMT>
-__global__ void k_bprep_tc(BPrepParams p) {
-  using T = typename Pair<FMT>::T;
-  const int64_t K = 1LL << p.nk, N = 1LL << p.nn;
-  const int64_t per = K * N;                  // complex elements per pattern
-  const int64_t total = p.PB * per;
-  T* hi = (T*)p.out;                          // pairs: [PB][2N][K] pairs of reals
-  T* lo = hi + 2 * total;
-  const float sc = FMT == 2 ? pow2f(fp16_scale_exp(*p.scale)) : 1.0f;
-  // kU elements per thread and round, their loads issued before any store,
-  // so that a grid of one block per SM (beside a running GEMM) still keeps
-  // enough loads in flight
-  constexpr int kU = 4;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < total; e0 += kU * stride) {
-    float2 b[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int64_t e = e0 + u * stride;
-      if (e < total) {
-        const int64_t pb = e / per, r = e - pb * per;
-        b[u] = p.B[pb * p.b_pstride + p.bk[r & (K - 1)] + p.bn[r >> p.nk]];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int64_t e = e0 + u * stride;
-      if (e >= total) break;
-      const int64_t pb = e / per, r = e - pb * per;
-      const int64_t n = r >> p.nk, k = r & (K - 1);
-      const int64_t o0 = (pb * 2 * N + 2 * n) * K + k;   // pair (2k, 2k+1) of row 2n
-      T h, l;
-      Pair<FMT>::split(b[u].x, -b[u].y, sc, h, l);
-      hi[o0] = h;
-      lo[o0] = l;
-      Pair<FMT>::split(b[u].y, b[u].x, sc, h, l);
-      hi[o0 + K] = h;                                    // row 2n + 1
-      lo[o0 + K] = l;
-    }
-  }
+__global__ void __launch_bounds__(256) k_bprep_tc(BPrepParams p) {
+  bprep_tc<FMT>(p, blockIdx.x, gridDim.x);
 }
 
 cudaError_t launch_bprep_c(const BPrepParams& p, cudaStream_t s) {

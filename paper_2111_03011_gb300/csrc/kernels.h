@@ -151,6 +151,7 @@ struct AccumParams : BatchParams {
 cudaError_t launch_small(const SmallParams& p, cudaStream_t s);
 cudaError_t launch_absmax(const AbsmaxParams& p, cudaStream_t s);
 cudaError_t launch_permute(const PermParams& p, cudaStream_t s);
+cudaError_t launch_operands(const PermParams& a, const BPrepParams& b, cudaStream_t s);   // A's permute and B's gather
 cudaError_t launch_bprep_c(const BPrepParams& p, cudaStream_t s);
 cudaError_t launch_bprep_tc(const BPrepParams& p, cudaStream_t s, bool beside_gemm = false);
 cudaError_t launch_gemm_simt(const GemmParams& p, cudaStream_t s);

@@ -1185,7 +1185,10 @@ static int layout_steps(Plan& plan, std::string& err) {
       {
         const int st = (int)plan.steps.size();
         touch(plan, sml.ref, st);
-        p.c = Ref{1, new_buf(plan, bprep_bytes, st)};
+        // the two preparations may share a launch (launch_operands): B's result
+        // is written while A's permute still reads its input
+        const bool after_permute = st > 0 && plan.steps.back().kind == ST_PERMUTE && plan.steps.back().contraction == ci;
+        p.c = Ref{1, new_buf(plan, bprep_bytes, after_permute ? st - 1 : st)};
         p.bytes = 8.0 * (double)vt_elems(sml) + (double)bprep_bytes;
         plan.steps.push_back(p);
       }

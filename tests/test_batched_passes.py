@@ -141,3 +141,26 @@ def test_batches_first_seen_and_replayed(tn, monkeypatch):
     assert all(float(b.abs().max()) == 0.0 for b in bufs[:3])
     assert all(tn.tn_head_fidelity(h)[1] == 0 for h in heads[:3])
     submit([0, 1, 2])
+
+
+@pytest.mark.parametrize("gemm", [1, 3, 4])
+def test_joint_preparations_share_no_memory(tn, gemm):
+    """A GEMM's permute and the B preparation right after it may run in one launch:
+    B's result and everything the permute reads or writes are apart."""
+    seen = 0
+    for c, kw in ((ci.config_small(4, 6, 10, seed=13, n_open=6, L=24, n_cut_gates=1), {}),
+                  (ci.config_small(4, 5, 10, seed=13, n_open=7, L=24, n_cut_gates=1), dict(small_max_bits=-1)),
+                  (ci.config_sliced30(), dict(order_trials=64, max_log2_elements=31))):
+        p = tn.tn_plan(c["circuit"], c["open_qubits"], c["tails"], c["edges"], host_only=True, gemm=gemm, **kw)
+        d = tn.tn_plan_describe(p)
+        for x, y in zip(d["steps"], d["steps"][1:]):
+            if x["kind"] != 1 or y["kind"] != 2 or x["contraction"] != y["contraction"]:
+                continue
+            seen += 1
+            assert y["a"] != x["c"]
+            o, n = d["bufs"][y["c"][1]][:2]
+            for kind, rid in (x["a"], x["c"], y["a"]):
+                if kind == 1:
+                    o2, n2 = d["bufs"][rid][:2]
+                    assert o + n <= o2 or o2 + n2 <= o
+    assert seen > 5
