@@ -629,11 +629,18 @@ __device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* m
       : "memory");
 }
 
+template <bool H16>
 __device__ __forceinline__ void mma2(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc));
+  if (H16)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc));
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
 // arrive on barrier `bar` (a local offset) in both CTAs of the pair once the
@@ -660,10 +667,10 @@ struct LayoutPair {
   static constexpr uint32_t TMEM_COLS = 512;     // two chunk buffers of 256 fp32 columns
 };
 
-// Instruction descriptor of a 256 x 256 pair MMA (kind::f16, fp32 accumulate)
+// Instruction descriptor of a 256 x 256 pair MMA (fp32 accumulate)
 template <int FMT>
 __device__ __forceinline__ uint32_t idesc_pair() {
-  const uint32_t f = FMT == 1 ? 1u : 0u;
+  const uint32_t f = FMT == 0 ? 2u : (FMT == 1 ? 1u : 0u);
   return (1u << 4) | (f << 7) | (f << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
 
@@ -675,7 +682,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                    const __grid_constant__ TileGrid grid, const uint32_t* __restrict__ mapA, const uint32_t* __restrict__ mapB, int mapA_mode,
                    int mapB_mode, const unsigned int* scaleA, const unsigned int* scaleB, unsigned int* amax_out,
                    unsigned int* status, int vec) {
-  static_assert(FMT == 1 || FMT == 2, "pair MMAs use kind::f16 operands");
   constexpr int BN = 256;
   using Lay = LayoutPair<STAGES>;
   constexpr int KB = Lay::KB;
@@ -700,7 +706,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int br = 1 << grid.br_log2;         // B rows per pattern box (2N when folded)
   const int half_boxes = fold >= 2 ? fold / 2 : 1;   // B boxes this CTA loads per stage
   const int box_rows = fold >= 2 ? br : 128;
-  constexpr int BKE = KB / 2;               // K elements (16-bit) per k-block
+  constexpr int BKE = KB / (FMT ? 2 : 4);   // K elements per k-block
   constexpr int CH = chunk_bytes(FMT) / KB, KK = KBlock<KB>::KK;
   const int nkb = (int)((K2 + BKE - 1) / BKE);
   const int nch = (nkb + CH - 1) / CH;
@@ -802,13 +808,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int kk = 0; kk < KK; ++kk) {
             const uint32_t o = kk * 32;
-            mma2(d, sdesc<KB>(a_hi + o), sdesc<KB>(b_lo + o), idesc, (first && kk == 0) ? 0u : 1u);
-            mma2(d, sdesc<KB>(a_lo + o), sdesc<KB>(b_hi + o), idesc, 1u);
+            mma2<FMT != 0>(d, sdesc<KB>(a_hi + o), sdesc<KB>(b_lo + o), idesc, (first && kk == 0) ? 0u : 1u);
+            mma2<FMT != 0>(d, sdesc<KB>(a_lo + o), sdesc<KB>(b_hi + o), idesc, 1u);
           }
 #pragma unroll
           for (int kk = 0; kk < KK; ++kk) {
             const uint32_t o = kk * 32;
-            mma2(d, sdesc<KB>(a_hi + o), sdesc<KB>(b_hi + o), idesc, 1u);
+            mma2<FMT != 0>(d, sdesc<KB>(a_hi + o), sdesc<KB>(b_hi + o), idesc, 1u);
           }
           mma_commit_pair(&empty[s]);
           if (last) {
@@ -1039,8 +1045,8 @@ static cudaError_t run_pair(const GemmParams& p, int fold, unsigned int* status,
   const int br = BN / fold;
   const uint32_t* grp = p.grp_fold == fold ? p.grp : nullptr;
   if (fold > 1 && (br != N2 || br < 16 || (p.mapA_mode != 1 && !grp) || fold % 2)) return cudaErrorInvalidValue;
-  const uint32_t BKE = KB / 2;
-  const int64_t es = 2;
+  const uint32_t BKE = KB / (FMT ? 2 : 4);
+  const int64_t es = FMT ? 2 : 4;
   const char* ahi = (const char*)p.A;
   const char* alo = ahi + p.PA * p.M * K2 * es;
   const char* bhi = (const char*)p.B;
@@ -1140,16 +1146,21 @@ static cudaError_t dispatch(const GemmParams& q, unsigned int* status, cudaStrea
   if (t.bn == 32) return run<32, kb_stages(32, kb_bytes(32, FMT)), FMT>(p, fold, status, s);
   if (t.bn == 64) return run<64, kb_stages(64, kb_bytes(64, FMT)), FMT>(p, fold, status, s);
   if (t.bn == 128) return run<128, kb_stages(128, kb_bytes(128, FMT)), FMT>(p, fold, status, s);
-  if (t.paired) return run_pair<FMT == 0 ? 1 : FMT>(p, fold, status, s);
+  // In tf32 a 128 x 256 tile on one CTA already feeds the tensor cores; pairs
+  // load a third less per tile from L2, which is what bounds short K, and pay
+  // once there are tiles for every pair: 53-qubit lattice in 3xTF32 23.3 -> 21.4 ms.
+  if (FMT == 0 && t.bn == 256 && p.M >= 2 * BM && p.pair >= 0) {
+    const int64_t groups = p.grp ? p.n_groups : (p.PC + fold - 1) / fold;
+    t.paired = groups * ((p.M + 2 * BM - 1) / (2 * BM)) * (fold > 1 ? 1 : (2 * p.N + 255) / 256) >= sm_count() / 2;
+  }
+  if (t.paired) return run_pair<FMT>(p, fold, status, s);
   return run<256, kb_stages(256, kb_bytes(256, FMT)), FMT>(p, fold, status, s);
 }
 
 template <int FMT>
 static cudaError_t set_attrs() {
-  if (FMT != 0) {
-    const cudaError_t e = set_attr_pair<FMT == 0 ? 1 : FMT>();
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = set_attr_pair<FMT>();
+  if (e != cudaSuccess) return e;
   const cudaError_t r[5] = {set_attr<16, kb_stages(16, kb_bytes(16, FMT)), FMT>(),
                             set_attr<32, kb_stages(32, kb_bytes(32, FMT)), FMT>(),
                             set_attr<64, kb_stages(64, kb_bytes(64, FMT)), FMT>(),

@@ -97,10 +97,12 @@ def test_direct_kernel_bf16_products(tn, shape):
 @pytest.mark.parametrize("engine", [1, 3, 4], ids=["tf32x3", "bf16x3", "fp16x3"])
 @pytest.mark.parametrize("shape", [(512, 64, 256, 5), (256, 32, 128, 7), (512, 16, 64, 9), (256, 8, 32, 20),
                                    (256, 128, 64, 1), (4096, 1, 64, 53), (256, 2, 16, 70), (512, 4, 128, 33),
-                                   (64, 1, 4, 3), (128, 4, 8, 200)], ids=str)
+                                   (64, 1, 4, 3), (128, 4, 8, 200), (4096, 1024, 32, 1), (8192, 512, 4, 1),
+                                   (2048, 64, 32, 24)], ids=str)
 def test_gemm_kernels_on_request(tn, engine, shape):
     """pair = 1 keeps small shapes on the GEMM kernels: folded CTA-pair tiles, and
-    narrow patterns as the columns of one matrix (ragged last tiles)."""
+    narrow patterns as the columns of one matrix (ragged last tiles), and enough
+    256 x 256 tiles for CTA pairs in tf32 too."""
     import torch
     M, N, K, P = shape
     rng = np.random.default_rng(M + N + K + P)
