@@ -183,64 +183,51 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
+// 16 lanes (rows) x 32 or 16 columns: thread t holds, for each 8 columns, the
+// pair 2 (t % 4), + 1 of row t / 4 and then of row t / 4 + 8.
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
         "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
 }
-
-// Writing a tile out.  A drain warp holds 32 rows, one per lane; stored from
-// there, every 16-byte store instruction touches 32 rows and writes half a sector
-// of each, and the load/store unit's 32 lines per instruction cap the kernel
-// at 2.4 TB/s of output.  The warp therefore turns 32 rows x 16 columns at a
-// time through its own 2 KB of shared memory (16-byte pieces, XOR-swizzled: no
-// bank conflicts either way) and stores 8 rows x 64 bytes per instruction.
-// 2^27 outputs from K = 16 (BF16x3): 453 -> 254 us, 4.2 TB/s of output; 2^25 x
-// 2^13 x 2^9: 4.22 -> 3.53 ms, as the drain warps leave the MMAs waiting less.
-constexpr int OUT_BYTES = 32 * 64;
-
-// (The lane is read afresh and the stage's address passed as 32 bits so that
-// nothing of this stays in registers beside the running sums.)
-__device__ __forceinline__ void store_piece(uint32_t stage, const float* w, float* dst, int64_t pitch, int rows) {
-  uint32_t lane;
-  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
-  const uint32_t wr = stage + lane * 64, xw = (lane >> 1) & 3;
-  __syncwarp();                              // the previous piece has been read
-#pragma unroll
-  for (uint32_t q = 0; q < 4; ++q)
-    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(wr + ((q ^ xw) << 4)), "f"(w[4 * q]),
-                 "f"(w[4 * q + 1]), "f"(w[4 * q + 2]), "f"(w[4 * q + 3])
-                 : "memory");
-  __syncwarp();
-  const uint32_t r0 = lane >> 2, q = lane & 3;
-  const uint32_t rd = stage + r0 * 64 + ((q ^ ((r0 >> 1) & 3)) << 4);   // rows 8 apart share the XOR
-  float* p = dst + r0 * pitch + 4 * q;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(rd + 512u * i)
-                 : "memory");
-    if ((int)r0 + 8 * i < rows) *(float4*)p = v;
-    p += 8 * pitch;
-  }
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(taddr));
 }
 
-// 16 columns of a row where the columns run over patterns of 2^sub (below 16)
-// reals each: C[pattern][row][2^sub].  A warp's 32 rows of a pattern are one
-// stretch of memory, so each lane stores its own row.
-__device__ __forceinline__ void store_patterns(const float* w, float* C, int64_t col, int sub, int64_t M, int64_t row,
-                                               int64_t cols) {
+// One drain warp's 32 rows x NCOL columns of a chunk, from its quarter's first
+// lane at taddr, into (first) or onto the running sums.  Element (half h of 16
+// rows, 8 columns j, register e) is acc[(h NCOL / 8 + j) 4 + e].
+template <int NCOL, bool FIRST>
+__device__ __forceinline__ void drain_loads(uint32_t taddr, float (&acc)[NCOL]) {
+  constexpr int W = NCOL >= 32 ? 32 : 16, NR = W / 2;          // columns and registers of a load
+  constexpr int LOADS = 2 * NCOL / W;
+  constexpr int RPMAX = NCOL >= 128 ? 2 : 4;                    // loads in flight per wait
+  constexpr int RP = LOADS < RPMAX ? LOADS : RPMAX;
 #pragma unroll
-  for (int e = 0; e < 16; e += 2) {
-    const int64_t c = col + e;
-    if (c >= cols) return;
-    const int64_t pc = c >> sub, n = c & ((1 << sub) - 1);
-    *(float2*)(C + (((pc * M + row) << sub) + n)) = make_float2(w[e], w[e + 1]);
+  for (int p0 = 0; p0 < LOADS; p0 += RP) {
+    uint32_t v[RP][NR];
+#pragma unroll
+    for (int j = 0; j < RP; ++j) {
+      const int l = p0 + j;
+      tmem_ld(taddr + (uint32_t)(l / (NCOL / W)) * (16u << 16) + (uint32_t)(l % (NCOL / W) * W), v[j]);
+    }
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < RP; ++j)
+#pragma unroll
+      for (int e = 0; e < NR; ++e) {
+        const float x = __uint_as_float(v[j][e]);
+        if (FIRST) acc[(p0 + j) * NR + e] = x; else acc[(p0 + j) * NR + e] += x;
+      }
   }
+}
+template <int NCOL>
+__device__ __forceinline__ void drain_chunk(uint32_t taddr, float (&acc)[NCOL], bool first) {
+  if (first) drain_loads<NCOL, true>(taddr, acc); else drain_loads<NCOL, false>(taddr, acc);
 }
 
 template <int BN, int STAGES, int KB>
@@ -249,8 +236,7 @@ struct Layout {
   static constexpr int B_BYTES = BN * KB;              // one BN-row tile
   static constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;  // A hi, A lo, B hi, B lo
   static constexpr int DATA = STAGES * STAGE;
-  static constexpr int OUT = (BN >= 32 ? 8 : 4) * OUT_BYTES;   // a staging tile per active drain warp
-  static constexpr int TOTAL = DATA + 1024 /*align*/ + 256 /*barriers*/ + OUT;
+  static constexpr int TOTAL = DATA + 1024 /*align*/ + 256 /*barriers*/;
   static_assert(TOTAL <= 232448, "shared memory per CTA");
   static_assert(2 * STAGES + 8 <= 32, "barrier area");
   // two chunk buffers of BN fp32 columns (ping-pong), a power of two >= 32
@@ -320,6 +306,66 @@ __device__ __forceinline__ int64_t tile_pattern(const TileGrid& g, uint32_t pg, 
   return pc < PC ? pc : -1;
 }
 
+// Writing a drain warp's 32 rows x NCOL columns out, straight from the running
+// sums: every store instruction writes 8 rows x 32 bytes, whole sectors.  (One
+// row per thread, 16 bytes at a time, half a sector of 32 rows per instruction,
+// stopped at 2.4 TB/s of output; turning the rows through shared memory at
+// 3.7 TB/s, bound by the latency of the drain warps' instructions.)
+template <int NCOL, int FMT>
+__device__ __forceinline__ void store_tile(const float (&acc)[NCOL], float* __restrict__ C, const TileGrid& grid,
+                                           uint32_t pg, uint32_t tn, int col0, int64_t row0, int rows, int64_t M,
+                                           int64_t N2, int64_t PC, float ua, float ub) {
+  const int lane = threadIdx.x & 31, r = lane >> 2, q2 = (lane & 3) * 2;
+  // FP16 engine: undo the operands' power-of-two scales (two exact multiplies)
+  auto pair = [&](int j, int g) {             // rows r + 8 g, columns 8 j + q2, + 1
+    const int i = ((g >> 1) * (NCOL / 8) + j) * 4 + (g & 1) * 2;
+    return FMT == 2 ? make_float2((acc[i] * ua) * ub, (acc[i + 1] * ua) * ub) : make_float2(acc[i], acc[i + 1]);
+  };
+  if (grid.sub_log2 >= 0) {
+    // the columns run over patterns of 2^sub reals each: C[pattern][row][2^sub]
+    const int sub = grid.sub_log2;
+#pragma unroll
+    for (int j = 0; j < NCOL / 8; ++j) {
+      const int64_t col = ((int64_t)tn << grid.br_log2) + col0 + 8 * j + q2;
+      float* dst = C + ((((col >> sub) * M + row0 + r) << sub) + (col & ((1 << sub) - 1)));
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        if (col < N2 && r + 8 * g < rows) *(float2*)(dst + ((8 * g) << sub)) = pair(j, g);
+    }
+    return;
+  }
+  const int64_t col = ((int64_t)tn << grid.br_log2) + col0;
+  if (grid.fold == 1 && col + NCOL <= N2) {
+    float* dst = C + ((tile_pattern(grid, pg, 0, PC) * M + row0 + r) * N2 + col + q2);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      if (r + 8 * g < rows) {
+#pragma unroll
+        for (int j = 0; j < NCOL / 8; ++j) *(float2*)(dst + 8 * j) = pair(j, g);
+      }
+      dst += 8 * N2;
+    }
+    return;
+  }
+  const int br = 1 << grid.br_log2;
+#pragma unroll
+  for (int pp = 0; pp < NCOL / 16; ++pp) {
+    const int cl = col0 + 16 * pp;             // column within the tile
+    const int64_t pc = tile_pattern(grid, pg, cl >> grid.br_log2, PC);   // pattern of the fold
+    if (pc < 0) continue;
+    const int64_t c = ((int64_t)tn << grid.br_log2) + (cl & (br - 1)) + q2;
+    float* dst = C + ((pc * M + row0 + r) * N2 + c);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      if (r + 8 * g < rows) {
+        if (c < N2) *(float2*)dst = pair(2 * pp, g);
+        if (c + 8 < N2) *(float2*)(dst + 8) = pair(2 * pp + 1, g);
+      }
+      dst += 8 * N2;
+    }
+  }
+}
+
 template <int BN, int STAGES, int FMT>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmAlo,
@@ -327,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               float* __restrict__ C, int64_t M, int64_t N2, int64_t K2, int64_t PC,
               const __grid_constant__ TileGrid grid, const uint32_t* __restrict__ mapA,
               const uint32_t* __restrict__ mapB, int mapA_mode, int mapB_mode, const unsigned int* scaleA,
-              const unsigned int* scaleB, unsigned int* amax_out, unsigned int* status, int vec) {
+              const unsigned int* scaleB, unsigned int* amax_out, unsigned int* status) {
   constexpr int KB = kb_bytes(BN, FMT);
   constexpr int CH = chunk_bytes(FMT) / KB;   // k-blocks per chunk
   using Lay = Layout<BN, STAGES, KB>;
@@ -466,15 +512,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // drain warps 0-7: TMEM lane quarter = warp % 4, column half = warp / 4;
     // each thread keeps the running sum of its row's NCOL columns in registers.
     constexpr int NCOL = BN >= 32 ? BN / 2 : BN;     // columns per warp
-    constexpr int NPIECE = NCOL / 16;                  // 16-column TMEM loads
-    constexpr int RPMAX = BN >= 256 ? 2 : 4;           // loads in flight per wait
-    constexpr int RP = NPIECE < RPMAX ? NPIECE : RPMAX;
     const int q = warp & 3, half = warp >> 2;
     const bool active = BN >= 32 || half == 0;
     const int col0 = BN >= 32 ? half * NCOL : 0;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const uint32_t stage = smem_u32(smem + Lay::DATA + 256 + warp * OUT_BYTES);   // used by active warps only
-    // FP16 engine: undo the operands' power-of-two scales (two exact multiplies)
     const float ua = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleA)) : 1.0f;
     const float ub = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleB)) : 1.0f;
     float tmax = 0.0f;
@@ -484,28 +525,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t pg, tm, tn_;
       tile_coords(grid, t, pg, tm, tn_);
       float acc[NCOL];
-#pragma unroll
-      for (int e = 0; e < NCOL; ++e) acc[e] = 0.0f;
       for (int c = 0; c < nch; ++c) {
         const int b = (int)(cc & 1);
         const uint32_t u = cc >> 1;
         ok = mbar_wait(&accf[b], u & 1, abort_flag);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
-        if (active) {
-#pragma unroll
-          for (int p0 = 0; p0 < NPIECE; p0 += RP) {
-            uint32_t v[RP][16];
-#pragma unroll
-            for (int j = 0; j < RP; ++j)
-              tmem_ld16(tmem + lane_base + (uint32_t)(b * BN) + (uint32_t)(col0 + 16 * (p0 + j)), v[j]);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int j = 0; j < RP; ++j)
-#pragma unroll
-              for (int e = 0; e < 16; ++e) acc[16 * (p0 + j) + e] += __uint_as_float(v[j][e]);
-          }
-        }
+        if (active) drain_chunk(tmem + lane_base + (uint32_t)(b * BN + col0), acc, c == 0);
         // the warp's TMEM loads are complete (wait::ld above); one lane
         // releases the buffer for the whole warp
         asm volatile("tcgen05.fence::before_thread_sync;");
@@ -524,36 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int e = 0; e < NCOL; ++e) tmax = fmaxf(tmax, fabsf(acc[e]));
       }
-      if (grid.sub_log2 >= 0) {
-#pragma unroll
-        for (int pp = 0; pp < NPIECE; ++pp) {
-          float w[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
-          if (lane < rows)
-            store_patterns(w, C, ((int64_t)tn_ << grid.br_log2) + col0 + 16 * pp, grid.sub_log2, M, row0 + lane, N2);
-        }
-        continue;
-      }
-#pragma unroll
-      for (int pp = 0; pp < NPIECE; ++pp) {
-        const int cl = col0 + 16 * pp;             // column within the tile
-        const int f = cl >> grid.br_log2;          // pattern of the fold
-        const int64_t pc = tile_pattern(grid, pg, f, PC);
-        const int64_t col = ((int64_t)tn_ << grid.br_log2) + (cl & (br - 1));
-        if (pc < 0) continue;
-        float* dst = C + (pc * M + row0) * N2 + col;
-        float w[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
-        if (vec && col + 16 <= N2) {
-          store_piece(stage, w, dst, N2, rows);
-        } else if (lane < rows) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (col + e < N2) dst[lane * N2 + e] = w[e];
-        }
-      }
+      store_tile<NCOL, FMT>(acc, C, grid, pg, tn_, col0, row0, rows, M, N2, PC, ua, ub);
     }
     if (amax_out && active) {
       // warp maximum, then the CTA maximum in shared memory (one global
@@ -661,7 +658,7 @@ struct LayoutPair {
   static constexpr int B_BYTES = 128 * KB;        // this CTA's half of the 256-row B tile
   static constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;
   static constexpr int DATA = STAGES * STAGE;
-  static constexpr int TOTAL = DATA + 1024 + 256 + 8 * OUT_BYTES;
+  static constexpr int TOTAL = DATA + 1024 + 256;
   static_assert(TOTAL <= 232448, "shared memory per CTA");
   static_assert(2 * STAGES + 8 <= 32, "barrier area");
   static constexpr uint32_t TMEM_COLS = 512;     // two chunk buffers of 256 fp32 columns
@@ -681,7 +678,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                    float* __restrict__ C, int64_t M, int64_t N2, int64_t K2, int64_t PC,
                    const __grid_constant__ TileGrid grid, const uint32_t* __restrict__ mapA, const uint32_t* __restrict__ mapB, int mapA_mode,
                    int mapB_mode, const unsigned int* scaleA, const unsigned int* scaleB, unsigned int* amax_out,
-                   unsigned int* status, int vec) {
+                   unsigned int* status) {
   constexpr int BN = 256;
   using Lay = LayoutPair<STAGES>;
   constexpr int KB = Lay::KB;
@@ -831,12 +828,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   } else {
     // drain warps 0-7 of both CTAs: this CTA's 128 rows, 128 columns per warp
     constexpr int NCOL = BN / 2;
-    constexpr int NPIECE = NCOL / 16;
-    constexpr int RP = 2;
     const int q = warp & 3, half = warp >> 2;
     const int col0 = half * NCOL;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const uint32_t stage = smem_u32(smem + Lay::DATA + 256 + warp * OUT_BYTES);
     const float ua = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleA)) : 1.0f;
     const float ub = FMT == 2 ? pow2f(-fp16_scale_exp(*scaleB)) : 1.0f;
     // the leader's release barriers: acce[b] sits 8 bytes past acce[0] there
@@ -850,26 +844,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       uint32_t pg, tm, tn_;
       tile_coords(grid, t, pg, tm, tn_);
       float acc[NCOL];
-#pragma unroll
-      for (int e = 0; e < NCOL; ++e) acc[e] = 0.0f;
       for (int c = 0; c < nch; ++c) {
         const int b = (int)(cc & 1);
         const uint32_t u = cc >> 1;
         ok = mbar_wait(&accf[b], u & 1, abort_flag);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-        for (int p0 = 0; p0 < NPIECE; p0 += RP) {
-          uint32_t v[RP][16];
-#pragma unroll
-          for (int j = 0; j < RP; ++j)
-            tmem_ld16(tmem + lane_base + (uint32_t)(b * BN) + (uint32_t)(col0 + 16 * (p0 + j)), v[j]);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int j = 0; j < RP; ++j)
-#pragma unroll
-            for (int e = 0; e < 16; ++e) acc[16 * (p0 + j) + e] += __uint_as_float(v[j][e]);
-        }
+        drain_chunk(tmem + lane_base + (uint32_t)(b * BN + col0), acc, c == 0);
         asm volatile("tcgen05.fence::before_thread_sync;");
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * (uint32_t)b);
@@ -883,36 +864,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int e = 0; e < NCOL; ++e) tmax = fmaxf(tmax, fabsf(acc[e]));
       }
-      if (grid.sub_log2 >= 0) {
-#pragma unroll
-        for (int pp = 0; pp < NPIECE; ++pp) {
-          float w[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
-          if (lane < rows)
-            store_patterns(w, C, ((int64_t)tn_ << grid.br_log2) + col0 + 16 * pp, grid.sub_log2, M, row0 + lane, N2);
-        }
-        continue;
-      }
-#pragma unroll
-      for (int pp = 0; pp < NPIECE; ++pp) {
-        const int cl = col0 + 16 * pp;
-        const int f = cl >> grid.br_log2;
-        const int64_t pc = tile_pattern(grid, pg, f, PC);
-        const int64_t col = ((int64_t)tn_ << grid.br_log2) + (cl & (br - 1));
-        if (pc < 0) continue;
-        float* dst = C + (pc * M + row0) * N2 + col;
-        float w[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) w[e] = FMT == 2 ? (acc[16 * pp + e] * ua) * ub : acc[16 * pp + e];
-        if (vec && col + 16 <= N2) {
-          store_piece(stage, w, dst, N2, rows);
-        } else if (lane < rows) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (col + e < N2) dst[lane * N2 + e] = w[e];
-        }
-      }
+      store_tile<NCOL, FMT>(acc, C, grid, pg, tn_, col0, row0, rows, M, N2, PC, ua, ub);
     }
     if (amax_out) {
       if (FMT == 2) tmax = (tmax * ua) * ub;
@@ -1024,7 +976,7 @@ static cudaError_t run(const GemmParams& p, int fold, unsigned int* status, cuda
   const int64_t ctas = std::min<int64_t>(n_tiles, sm_count());
   k_gemm_tc<BN, STAGES, FMT><<<(unsigned)ctas, kThreads, Lay::TOTAL, s>>>(
       tah, tal, tbh, tbl, (float*)p.C, p.M, N2, K2, p.PC, grid, p.mapA, p.mapB, p.mapA_mode,
-      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status, (uintptr_t)p.C % 16 == 0);
+      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status);
   return cudaGetLastError();
 }
 
@@ -1074,7 +1026,7 @@ static cudaError_t run_pair(const GemmParams& p, int fold, unsigned int* status,
   const int64_t clusters = std::min<int64_t>(n_tiles, sm_count() / 2);
   k_gemm_tc_pair<kPairStages, FMT><<<(unsigned)(2 * clusters), kThreads, Lay::TOTAL, s>>>(
       tah, tal, tbh, tbl, (float*)p.C, p.M, N2, K2, p.PC, grid, p.mapA, p.mapB, p.mapA_mode,
-      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status, (uintptr_t)p.C % 16 == 0);
+      p.mapB_mode, p.scaleA, p.scaleB, p.amax, status);
   return cudaGetLastError();
 }
 
