@@ -190,6 +190,13 @@ struct ScratchLease {
         g_scratch.erase(g_scratch.begin() + (std::ptrdiff_t)at);
       }
     }
+    // allocations below must not end a stream capture that another thread has begun
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    struct Restore {
+      cudaStreamCaptureMode mode;
+      ~Restore() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    } restore{mode};
     if (!c.rep) {
       c.device = dev;
       void* h = nullptr;
@@ -215,7 +222,7 @@ struct ScratchLease {
       cudaFreeHost(c.host);
       c.host = nullptr;
       c.host_bytes = 0;
-      if (cudaHostAlloc(&c.host, host_bytes, cudaHostAllocPortable) != cudaSuccess) {
+      if (cudaHostAlloc(&c.host, host_bytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
         cudaGetLastError();
         return fail(TN_ERR_OOM, "scratch allocation failed");
       }
@@ -1488,14 +1495,19 @@ extern "C" int tn_head_norm(tn_head_t* h, double* norm, double* group_norms, voi
   tn_plan_t* p = h->plan;
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t L = (int64_t)p->P.tails_raw.size();
+  // the group norms of up to 8,192 groups come back through mapped memory, as
+  // the norm does; more by a copy (one block writes them)
+  const bool mapped = group_norms && L <= 8192;
   ScratchLease lease(st);
-  if (int rc = lease.take(0)) return rc;
+  if (int rc = lease.take(0, mapped ? (size_t)L * sizeof(double) : 0)) return rc;
   CUDA_TRY(tn::launch_group_norms(h->H, L, (int)p->P.open_qubits.size(), h->d_Z, nullptr, lease.c.part, st,
-                                  lease.c.rep, p->d_status));
-  if (group_norms) CUDA_TRY(cudaMemcpyAsync(group_norms, h->d_Z, (size_t)L * sizeof(double), cudaMemcpyDeviceToHost, st));
+                                  lease.c.rep, p->d_status, mapped ? (double*)lease.c.host : nullptr));
+  if (group_norms && !mapped)
+    CUDA_TRY(cudaMemcpyAsync(group_norms, h->d_Z, (size_t)L * sizeof(double), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   const tn::HeadReport rep = lease.done();
   if (norm) *norm = rep.sum[0];
+  if (mapped) std::memcpy(group_norms, lease.c.host, (size_t)L * sizeof(double));
   return tn::report_status(h, rep.word, st);
 }
 

@@ -65,6 +65,7 @@ DirectPlan plan_direct(const DirectShape& s, bool fold) {
   const int64_t stages = 1LL << (s.nk - tkb);
   while (d.cluster < 8 && tiles * d.cluster * 2 <= kSmCount * kResident && stages >= 8 * d.cluster) d.cluster *= 2;
   const double ctas = tiles * d.cluster;
+  if (ctas > 2147483647.0) return d;   // one grid dimension; left to the other forms
   const double padded = tiles * std::ldexp(1.0, g.tr + g.tc + s.nk);
   // fewer CTAs than the chip holds run at their share of the rate; X passes
   // through L2 once per column tile

@@ -14,7 +14,7 @@
 // Whole calls, before (a warp scan per 32 members in every kernel, status words
 // and results by copies) and now; a launch and a synchronisation take 14 us:
 //   amplitudes, 65,536 of 64 groups, pinned host in and out    54 ->  26 us
-//   norm with group norms, 64 groups of 1,024                  74 ->  41 us
+//   norm with group norms, 64 groups of 1,024                  74 ->  31 us
 //   norm, 65,536 groups of 64                                 123 ->  48 us
 //   10,000 exact draws, 64 groups of 1,024                    362 ->  37 us
 //   65,536 exact draws, 65,536 groups of 64                   198 ->  39 us
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(256) k_norm_wide(const double2* __restrict__ H
 __global__ void __launch_bounds__(1024) k_final_sums(const double* __restrict__ part, int nb, int n_sums,
                                                      const double* __restrict__ unit, int64_t L, int seg_log2,
                                                      double* __restrict__ Z, double* out, HeadReport* rep,
-                                                     const unsigned int* plan_status) {
+                                                     const unsigned int* plan_status, double* host_Z) {
   __shared__ double w[32];
   report_word(rep, plan_status);
   if (seg_log2)
@@ -183,7 +183,10 @@ __global__ void __launch_bounds__(1024) k_final_sums(const double* __restrict__ 
       double t = 0.0;
       for (int64_t s = 0; s < 1LL << seg_log2; ++s) t += unit[(g << seg_log2) + s];
       Z[g] = t;
+      if (host_Z) host_Z[g] = t;
     }
+  else if (host_Z)
+    for (int64_t g = threadIdx.x; g < L; g += blockDim.x) host_Z[g] = Z[g];
   for (int q = 0; q < n_sums; ++q) {
     double acc = 0.0;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) acc += part[(int64_t)q * nb + i];
@@ -205,7 +208,7 @@ __global__ void __launch_bounds__(1024) k_final_sums(const double* __restrict__ 
 }
 
 cudaError_t launch_group_norms(const double2* H, int64_t L, int h, double* Z, double* N, double* scratch,
-                               cudaStream_t s, HeadReport* rep, const unsigned int* plan_status) {
+                               cudaStream_t s, HeadReport* rep, const unsigned int* plan_status, double* host_Z) {
   double* part = scratch;                      // kHeadParts block totals, then kHeadParts units
   double* unit = scratch + kHeadParts;
   int nb, seg = 0;
@@ -222,7 +225,7 @@ cudaError_t launch_group_norms(const double2* H, int64_t L, int h, double* Z, do
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_final_sums<<<1, 1024, 0, s>>>(part, nb, 1, unit, L, seg, Z, N, rep, plan_status);
+  k_final_sums<<<1, 1024, 0, s>>>(part, nb, 1, unit, L, seg, Z, N, rep, plan_status, host_Z);
   return cudaGetLastError();
 }
 
@@ -276,7 +279,7 @@ cudaError_t launch_xeb(const double2* H, int h, const uint64_t* keys, const uint
                                      &rep->missing);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_final_sums<<<1, 1024, 0, s>>>(scratch, nb, 2, nullptr, 0, 0, nullptr, nullptr, rep, nullptr);
+  k_final_sums<<<1, 1024, 0, s>>>(scratch, nb, 2, nullptr, 0, 0, nullptr, nullptr, rep, nullptr, nullptr);
   return cudaGetLastError();
 }
 

@@ -183,9 +183,11 @@ cudaError_t launch_amplitudes(const double2* H, int h, const uint64_t* keys, con
                               int dtype, unsigned long long* status, cudaStream_t s, const int64_t* seg_end = nullptr,
                               int n_seg = 1, HeadReport* rep = nullptr, const unsigned int* plan_status = nullptr);
 
-// per-group squared norms Z[g] and their total (into *N and the report, where given)
+// per-group squared norms Z[g] (also into mapped host memory host_Z, if given)
+// and their total (into *N and the report, where given)
 cudaError_t launch_group_norms(const double2* H, int64_t L, int h, double* Z, double* N, double* scratch,
-                               cudaStream_t s, HeadReport* rep = nullptr, const unsigned int* plan_status = nullptr);
+                               cudaStream_t s, HeadReport* rep = nullptr, const unsigned int* plan_status = nullptr,
+                               double* host_Z = nullptr);
 
 // rep->sum = sum |a_i|^2 and sum log |a_i|^2 over the amplitudes a_i of n samples
 cudaError_t launch_xeb(const double2* H, int h, const uint64_t* keys, const uint32_t* groups, int64_t n_keys,

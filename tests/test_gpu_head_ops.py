@@ -100,7 +100,7 @@ def test_exact_draws_bit_for_bit(tn, L, h, n, kind):
     assert np.array_equal(tn.tn_sample(head, n, 0.0, seed), _reference(H, tails, oq, n, seed))
 
 
-@pytest.mark.parametrize("L,h", [(1, 0), (7, 2), (1000, 3), (333, 4), (65, 6), (3, 9), (40, 10), (2, 13), (1, 16)])
+@pytest.mark.parametrize("L,h", [(1, 0), (7, 2), (1000, 3), (333, 4), (65, 6), (3, 9), (40, 10), (2, 13), (1, 16), (9000, 1)])
 def test_norms_and_xeb(tn, L, h):
     """FP64 sums of up to 2^16 terms in any order: within 2^16 units of 2^-53 of
     the sum of magnitudes, and far closer in fact."""
@@ -146,3 +146,25 @@ def test_amplitudes_from_any_memory(tn, where):
             tn.tn_amplitudes(head, b, out=o)
         assert e.value.code == tn.TN_ERR_NOT_IN_STATE and f"bitstring {missing[0]} " in str(e.value)
         assert o.cpu().numpy()[missing[0]] == 0
+
+
+def test_open_qubits_that_are_not_consecutive(tn):
+    import torch
+    oq = [5, 2, 39, 17]
+    L, h = 9, 4
+    H = _values("plain", L, 1 << h, seed=8)
+    tails = ci.draw_tails(NQ, oq, L, seed=4)
+    c = ci.make_grid_circuit(2, 2, 1, seed=1)
+    c.n_qubits = NQ
+    plan = tn.tn_plan(c, oq, tails, host_fold_log2=-1)
+    buf = torch.zeros((L, 1 << h), dtype=torch.complex128, device="cuda")
+    head = tn.tn_head_create(plan, buf)
+    buf.copy_(torch.from_numpy(H))
+    torch.cuda.synchronize()
+    bits = np.array([int(t) | sum(((mu >> j) & 1) << q for j, q in enumerate(oq)) for t in tails
+                     for mu in range(1 << h)], dtype=np.uint64)
+    assert np.array_equal(tn.tn_amplitudes(head, bits).reshape(L, -1), H)
+    lin, _ = tn.tn_xeb(head, bits)
+    assert math.isclose(lin, 2.0 ** NQ * (np.abs(H) ** 2).mean() - 1, rel_tol=2.0 ** -40, abs_tol=2.0 ** -40)
+    tn.tn_head_set_fidelity(head, 1.0)
+    assert np.array_equal(tn.tn_sample(head, 40, 0.0, 3), _reference(H, tails, oq, 40, 3))
