@@ -165,6 +165,23 @@ def _spawn_ranks(n):
     return subprocess.call(cmd)
 
 
+def launches_of(tn, plan, slices):
+    """Kernel launches of a contraction of `slices` slices: the batched steps
+    once per chunk of passes, the others per pass, a GEMM's permute and the B
+    gather right after it in one launch, the accumulation per pass (per chunk
+    when every step is batched)."""
+    d = tn.tn_plan_describe(plan)
+    steps, most = d["steps"], d["batch"][0]
+    passes = slices << d["n_internal"]
+    batched = sum(s["batch"] for s in steps) if most > 1 else 0
+    joined = sum(x["kind"] == 1 and x["split"] >= 1 and y["kind"] == 2 and x["contraction"] == y["contraction"] and
+                 y["fork"] < 0 and not (y["alts"] and (y["variant"] == 0) == bool(y["bprep_embed0"]))
+                 for x, y in zip(steps, steps[1:]))
+    chunks = -(-passes // most)
+    own = len(steps) - batched - joined
+    return chunks * batched + passes * own + (chunks if most > 1 and batched == len(steps) else passes)
+
+
 def _dist():
     ws = int(os.environ.get("WORLD_SIZE", "1"))
     rank = int(os.environ.get("RANK", "0"))
@@ -429,7 +446,7 @@ def run_ours(args):
         "alg_bytes_per_slice": st["alg_bytes"],
         "e2e": {"value": round(e2e, 3), "unit": "TFLOP/s", "ms_per_step": round(ms_e2e, 3),
                 "h2d_bytes_per_step": int(n_amp * 8), "d2h_bytes_per_step": int(n_amp * 16 + n_samples * 8 + 8)},
-        "gpu_launches": int(args.steps * (n_slices * n_pass * n_launch + 4)),
+        "gpu_launches": int(args.steps * (launches_of(tn, plan, n_slices) + 5)),
         "roofline": roof,
         "clocks": clocks,
     }
@@ -670,7 +687,7 @@ def run_batch(args):
         heads = [tn.tn_head_create(p) for p in plans]
         ranges = [(0, 1 << st["n_sliced"]) for st in stats]
         flops = 8.0 * sum(st["tc_macs"] for st in stats)
-        launches = sum(st["n_launches"] for st in stats)
+        launches = sum(launches_of(tn, p, r[1] - r[0]) for p, r in zip(plans, ranges))
 
         def step():
             for h in heads:

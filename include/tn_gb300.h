@@ -110,8 +110,9 @@ typedef struct {
                                  host tensors (leaves or earlier folds) and whose result has at most
                                  2^this elements (and at most 2^6 slice variants) is done on the host
                                  in FP64 at plan time and becomes a leaf (0: 12; -1: off) */
-  int    gemm_pair;           /* 0: 16-bit GEMM steps with 256-wide tiles and M >= 256 run on CTA pairs
-                                 (cta_group::2, 256 x 256 tiles); -1: one-CTA 128-row tiles only.
+  int    gemm_pair;           /* 0: GEMM steps with 256-wide tiles and M >= 256 run on CTA pairs
+                                 (cta_group::2, 256 x 256 tiles; in tf32 where there are tiles for
+                                 every pair); -1: one-CTA 128-row tiles only.
                                  tn_plan_autotune times both and keeps the faster. */
   int    side_bprep;          /* 1: a large tensor-core B-preparation step (>= 64 MiB) whose operand
                                  is already written runs on a second stream beside the previous
