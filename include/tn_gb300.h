@@ -280,9 +280,10 @@ int  tn_contract_batch(tn_plan_t* const* plans, const tn_range* ranges, tn_head_
                        void* stream);
 
 /* out[i] = H[g(s_i)][mu(s_i)] for n bitstrings.  `bitstrings` and `out` may be
- * host or device pointers; dtype TN_C64 or TN_C128.  Synchronises `stream`.
- * TN_ERR_NOT_IN_STATE if a bitstring's tail is not a group (the first such
- * index is in tn_last_error()); `out` then holds 0 for those entries. */
+ * host or device pointers, at any alignment, and may overlap; dtype TN_C64 or
+ * TN_C128.  Synchronises `stream`.  TN_ERR_NOT_IN_STATE if a bitstring's tail
+ * is not a group (the first such index is in tn_last_error()); `out` then holds
+ * 0 for those entries. */
 int  tn_amplitudes(tn_head_t* head, const uint64_t* bitstrings, int64_t n,
                    void* out, int dtype, void* stream);
 

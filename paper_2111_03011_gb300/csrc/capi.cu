@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "buffers.h"
 #include "handles.h"
 #include "kernels.h"
 #include "planner.h"
@@ -1412,9 +1413,12 @@ static int ensure_stage(tn_head* h, size_t bytes) {
   return TN_OK;
 }
 
-// A pointer that kernels can use as it is: device or managed memory, or pinned
-// host memory, which GB300 reads and writes over NVLink-C2C without a copy.
-static bool kernel_ptr(const void* p) {
+// A buffer that kernels can use as it is: device or managed memory, or pinned
+// host memory, which GB300 reads and writes over NVLink-C2C without a copy, if
+// it starts on the `align` bytes that the kernel moves at a time.  Other buffers
+// go through the head's staging buffer.
+static bool kernel_ptr(const void* p, size_t align) {
+  if (!tn::kernel_aligned(p, align)) return false;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
@@ -1433,7 +1437,10 @@ extern "C" int tn_amplitudes(tn_head_t* h, const uint64_t* bitstrings, int64_t n
   tn_plan_t* p = h->plan;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t esz = dtype == TN_C128 ? 16 : 8;
-  const bool dev_in = kernel_ptr(bitstrings), dev_out = kernel_ptr(out);
+  // bitstrings that the output covers are copied before any of it is written
+  const bool dev_in =
+      kernel_ptr(bitstrings, 8) && !tn::ranges_overlap(bitstrings, (size_t)n * 8, out, (size_t)n * esz);
+  const bool dev_out = kernel_ptr(out, esz);
   size_t need = 0;
   if (!dev_in) need += (size_t)n * 8;
   size_t out_off = (need + 255) / 256 * 256;
@@ -1446,14 +1453,14 @@ extern "C" int tn_amplitudes(tn_head_t* h, const uint64_t* bitstrings, int64_t n
   if (int rc = lease.take(0)) return rc;
   const uint64_t* d_bits = bitstrings;
   if (!dev_in) {
-    CUDA_TRY(cudaMemcpyAsync(h->d_stage, bitstrings, (size_t)n * 8, cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync(h->d_stage, bitstrings, (size_t)n * 8, cudaMemcpyDefault, st));
     d_bits = (const uint64_t*)h->d_stage;
   }
   void* d_out = dev_out ? out : (void*)((char*)h->d_stage + out_off);
   CUDA_TRY(tn::launch_amplitudes(h->H, (int)p->P.open_qubits.size(), p->d_keys, p->d_key_groups, p->n_keys,
                                  p->P.tail_mask, p->d_open, d_bits, n, d_out, dtype == TN_C128 ? 1 : 0,
                                  &lease.c.rep->missing, st, nullptr, 1, lease.c.rep, p->d_status));
-  if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, d_out, (size_t)n * esz, cudaMemcpyDeviceToHost, st));
+  if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, d_out, (size_t)n * esz, cudaMemcpyDefault, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   const tn::HeadReport rep = lease.done();
   if (int rc = tn::report_status(h, rep.word, st)) return rc;
@@ -1470,9 +1477,9 @@ extern "C" int tn_xeb(tn_head_t* h, const uint64_t* samples, int64_t n, double* 
   tn_plan_t* p = h->plan;
   cudaStream_t st = (cudaStream_t)stream;
   const uint64_t* d_bits = samples;
-  if (!kernel_ptr(samples)) {
+  if (!kernel_ptr(samples, 8)) {
     if (int rc = ensure_stage(h, (size_t)n * 8)) return rc;
-    CUDA_TRY(cudaMemcpyAsync(h->d_stage, samples, (size_t)n * 8, cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync(h->d_stage, samples, (size_t)n * 8, cudaMemcpyDefault, st));
     d_bits = (const uint64_t*)h->d_stage;
   }
   ScratchLease lease(st);
@@ -1544,7 +1551,7 @@ static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t
   double mix = 0.0;
   if (target_fidelity > 0.0 && f_head > 0.0 && target_fidelity < f_head) mix = 1.0 - target_fidelity / f_head;
   cudaStream_t st = (cudaStream_t)stream;
-  const bool dev_out = kernel_ptr(out);
+  const bool dev_out = kernel_ptr(out, 8);
   uint64_t* d_out = out;
   if (!dev_out) {
     int rc = ensure_stage(h, (size_t)n * 8);
@@ -1573,7 +1580,7 @@ static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t
   sp.rep = lease.c.rep;
   sp.plan_status = p->d_status;
   CUDA_TRY(tn::launch_sample(sp, st));
-  if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, d_out, (size_t)n * 8, cudaMemcpyDeviceToHost, st));
+  if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, d_out, (size_t)n * 8, cudaMemcpyDefault, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   return tn::report_status(h, lease.done().word, st);
 }
