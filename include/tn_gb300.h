@@ -418,7 +418,8 @@ int  tn_head_norm_noalloc(const void* head_c128, int64_t n_groups, int n_open, d
 /* Standalone complex GEMM step (the contraction kernel of every GEMM step, the
  * K2 step of the contraction; Supplement complexity table, 8 flops per complex
  * multiply-add): C[p] = A[mapA(p)] B[mapB(p)] for p < PC, complex64, with
- * A [PA][M][K], B [PB][K][N] and C [PC][M][N] row-major device buffers.
+ * A [PA][M][K], B [PB][K][N] and C [PC][M][N] row-major device buffers; C may
+ * lie over A or B, which are then read before C is written.
  * M, N and K are powers of two (K >= 2 on the tensor-core engines; 16-bit
  * engines take K = 2 in tf32, as the planner does).  mapA / mapB are host
  * arrays of PC pattern indices, or NULL for the identity (P = PC) or pattern 0

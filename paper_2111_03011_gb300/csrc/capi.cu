@@ -1639,10 +1639,15 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
     }
   }
   cudaStream_t st = (cudaStream_t)stream;
+  // An operand that C covers is read before any of C is written: the tensor-core
+  // path always reads planes of both, the CUDA-core one a copy of that operand.
+  const size_t a_in = (size_t)(PA * M * K) * 8, b_in = (size_t)(PB * K * N) * 8, c_out = (size_t)(PC * M * N) * 8;
+  const bool over_a = tn::ranges_overlap(A, a_in, C, c_out), over_b = tn::ranges_overlap(B, b_in, C, c_out);
   // The direct kernel where it is modelled faster than the three launches
   // below (as the planner chooses; C is row-major, so its rows are N and X is
-  // B).  pair != 0 asks for the GEMM kernels themselves.
-  if (!simt && pair == 0 && nmk <= 31 && nk + nn <= 31) {
+  // B), and its operands, which it reads where they lie, are apart from C.
+  // pair != 0 asks for the GEMM kernels themselves.
+  if (!simt && pair == 0 && !over_a && !over_b && nmk <= 31 && nk + nn <= 31) {
     int nm = nmk - nk;
     std::vector<int> xr, xk, yk, yc;
     for (int j = 0; j < nn; ++j) xr.push_back(j);
@@ -1704,9 +1709,9 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
   const int64_t es = h16 ? 2 : 4;
   const size_t n_map = maps[0].size() + maps[1].size();
   const size_t map_off = 256, a_off = (map_off + n_map * sizeof(uint32_t) + 1023) / 1024 * 1024;
-  const size_t a_bytes = simt ? 0 : (size_t)(2 * PA * M * (2 * K) * es);
+  const size_t a_bytes = simt ? (over_a ? a_in : 0) : (size_t)(2 * PA * M * (2 * K) * es);
   const size_t b_off = a_off + (a_bytes + 1023) / 1024 * 1024;
-  const size_t b_bytes = simt ? 0 : (size_t)(2 * PB * (2 * N) * (2 * K) * es);
+  const size_t b_bytes = simt ? (over_b ? b_in : 0) : (size_t)(2 * PB * (2 * N) * (2 * K) * es);
   ScratchLease lease(st);
   if (int rc = lease.take(b_off + b_bytes, n_map * sizeof(uint32_t))) return rc;
   char* d = (char*)lease.c.buf;
@@ -1723,11 +1728,14 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
     if (e == cudaSuccess && h16 == 2) e = cudaMemsetAsync(d_scale, 0, 2 * sizeof(unsigned int), st);
     tn::GemmOperands op{(const float2*)A, (const float2*)B, d + a_off, d + b_off, PA * M * K, K, N, PB, h16, d_scale};
     if (e == cudaSuccess) e = tn::launch_gemm_operands(op, st);
+  } else {
+    if (e == cudaSuccess && over_a) e = cudaMemcpyAsync(d + a_off, A, a_in, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess && over_b) e = cudaMemcpyAsync(d + b_off, B, b_in, cudaMemcpyDeviceToDevice, st);
   }
   if (e == cudaSuccess) {
-    // the CUDA-core GEMM reads both row-major operands as they are
-    gp.A = simt ? (const float2*)A : (const float2*)(d + a_off);
-    gp.B = simt ? B : (const void*)(d + b_off);
+    // the CUDA-core GEMM reads row-major operands as they are
+    gp.A = simt && !over_a ? (const float2*)A : (const float2*)(d + a_off);
+    gp.B = simt && !over_b ? B : (const void*)(d + b_off);
     gp.C = (float2*)C;
     gp.M = M;
     gp.N = N;
