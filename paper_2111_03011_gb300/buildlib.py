@@ -21,7 +21,7 @@ INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["capi.cu", "kernels.cu", "gemm_tc.cu", "direct.cu", "head_ops.cu", "noalloc.cu", "server.cu"]
-CPP_SOURCES = ["planner.cpp", "direct_plan.cpp"]
+CPP_SOURCES = ["planner.cpp", "direct_plan.cpp", "gemm_tile.cpp"]
 
 
 def _nvcc():

@@ -1010,20 +1010,19 @@ constexpr int kNumGemmVariants = (int)(sizeof(kGemmVariants) / sizeof(kGemmVaria
 // so that a step's variant numbers never change).
 std::vector<int> gemm_variants(const tn::Step& x) {
   std::vector<int> out;
-  std::vector<tn::GemmTile> seen;
+  std::vector<tn::GemmForm> seen;
   for (int v = 0; v < kNumGemmVariants; ++v) {
-    tn::GemmParams gp;
-    gp.M = 1LL << x.nm;
-    gp.N = 1LL << x.nn;
-    gp.K = 1LL << x.nk;
-    gp.PC = x.PC;
-    gp.mapA_mode = x.mapA_mode;
-    gp.h16 = x.h16;
-    gp.pair = kGemmVariants[v].pair;
-    gp.tile_cap = kGemmVariants[v].cap;
-    const tn::GemmTile t = tn::gemm_tc_tile(gp);
+    tn::GemmShape gs;
+    gs.M = 1LL << x.nm;
+    gs.N = 1LL << x.nn;
+    gs.PC = x.PC;
+    gs.mapA_mode = x.mapA_mode;
+    gs.h16 = x.h16;
+    gs.pair = kGemmVariants[v].pair;
+    gs.tile_cap = kGemmVariants[v].cap;
+    const tn::GemmForm t = tn::gemm_form(gs, 1 << 30);
     bool dup = false;
-    for (const tn::GemmTile& q : seen) dup |= q.bn == t.bn && q.fold == t.fold && q.paired == t.paired;
+    for (const tn::GemmForm& q : seen) dup |= q.bn == t.bn && q.fold == t.fold && q.paired == t.paired;
     if (!dup) {
       seen.push_back(t);
       out.push_back(v);

@@ -55,7 +55,7 @@ namespace tn {
 
 namespace tc {
 
-constexpr int BM = 128;
+constexpr int BM = kGemmRows;
 // K per k-block (one pipeline stage), KB bytes of each operand row: 128 (the
 // 128-byte swizzle) or 64 (the 64-byte swizzle; stages half the size, twice
 // as many in flight, half the MMAs per k-block).
@@ -934,9 +934,9 @@ static cudaError_t set_attr() {
 static int sm_count() {
   static int n[64] = {0};
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  if (!n[dev] && cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n[dev] = 152;
-  return n[dev] > 0 ? n[dev] : 152;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return kGemmSMs;
+  if (!n[dev] && cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n[dev] = kGemmSMs;
+  return n[dev] > 0 ? n[dev] : kGemmSMs;
 }
 
 // fold = patterns per tile side by side along N (1: none); see the kernel
@@ -1032,81 +1032,50 @@ static cudaError_t run_pair(const GemmParams& p, int fold, unsigned int* status,
 
 }  // namespace tc
 
-// Tile width: the smallest of 16..cap (cap = p.tile_cap, a power of two in
-// 16..256; 256 by default) that covers 2N, or, when all patterns share A and
-// 2N >= 16, up to cap columns of consecutive patterns folded side by side
-// (fold = BN / 2N, as many as the pattern count rounded up to a power of two
-// allows).  256-wide 16-bit tiles with at least 256 rows run on CTA pairs
-// unless p.pair < 0.
-GemmTile gemm_tc_tile(const GemmParams& p) {
-  int cap = 16;
-  while (cap < 256 && cap < p.tile_cap) cap *= 2;
-  const int64_t N2 = 2 * p.N;
-  int64_t w = N2;
-  int fold = 1;
-  if (p.mapA_mode == 1 && p.PC > 1 && N2 >= 16 && N2 < cap) {
-    while (w < cap && fold < p.PC) {
-      w *= 2;
-      fold *= 2;
-    }
-  }
-  GemmTile t;
-  t.bn = 16;
-  while (t.bn < 256 && t.bn < std::min<int64_t>(w, cap)) t.bn *= 2;
-  t.fold = fold;
-  t.paired = p.h16 != 0 && t.bn == 256 && p.M >= 2 * tc::BM && p.pair >= 0;
-  return t;
+GemmShape gemm_shape(const GemmParams& p) {
+  GemmShape q;
+  q.M = p.M;
+  q.N = p.N;
+  q.PA = p.PA;
+  q.PB = p.PB;
+  q.PC = p.PC;
+  q.mapA_mode = p.mapA_mode;
+  q.mapB_mode = p.mapB_mode;
+  q.h16 = p.h16;
+  q.pair = p.pair;
+  q.tile_cap = p.tile_cap;
+  q.grp_fold = p.grp ? p.grp_fold : 0;
+  q.n_groups = p.n_groups;
+  return q;
 }
 
 namespace tc {
 
 template <int FMT>
 static cudaError_t dispatch(const GemmParams& q, unsigned int* status, cudaStream_t s) {
+  const GemmForm f = gemm_form(gemm_shape(q), sm_count());
   GemmParams p = q;
-  // Every pattern has its own A and all share B: one GEMM over the PC x M rows,
-  // which lie one after another in A's planes and in C.  Small M then fills the
-  // 128-row tiles, and a wave's row tiles share each B tile.
-  if (p.mapA_mode == 0 && p.mapB_mode == 1 && p.PA == p.PC && p.PC > 1 && p.PC * p.M <= 0x7fffffffLL) {
-    p.M *= p.PC;
-    p.PA = p.PC = 1;
-    p.mapA_mode = 1;
-  }
-  // All patterns share A and each has its own narrow B: the prepared B is one
-  // matrix of all their columns, so this is one GEMM over PC x N columns whose
-  // results go to their patterns.  53 patterns of one column each (2^18 x 2^6)
-  // took 2.4 ms as 53 passes over A.
-  if (p.mapA_mode == 1 && p.mapB_mode == 0 && p.PB == p.PC && p.PC > 1 && 2 * p.N < 16 &&
-      p.PC * p.N <= 0x3fffffffLL && p.tile_cap >= 256) {
-    p.sub_log2 = p.N == 1 ? 1 : p.N == 2 ? 2 : 3;
-    p.N *= p.PC;
-    p.PB = p.PC = 1;
-    p.mapB_mode = 1;
-  }
-  GemmTile t = gemm_tc_tile(p);
-  // Groups of patterns with one A pattern, where a table of them is given, for
-  // the widest tiles; other tile choices take the patterns one by one.
-  if (p.grp && p.tile_cap >= 256) {
-    t.fold = p.grp_fold;
-    t.bn = (int)std::min<int64_t>(256, 2 * p.N * p.grp_fold);
-    t.paired = FMT != 0 && t.bn == 256 && p.M >= 2 * BM && p.pair >= 0;
-  } else {
+  p.M = f.M;
+  p.N = f.N;
+  p.PA = f.PA;
+  p.PB = f.PB;
+  p.PC = f.PC;
+  p.mapA_mode = f.mapA_mode;
+  p.mapB_mode = f.mapB_mode;
+  p.sub_log2 = f.sub_log2;
+  if (!f.grouped) {
     p.grp = nullptr;
     p.grp_fold = 0;
   }
-  const int fold = t.fold;
-  if (t.bn == 16) return run<16, kb_stages(16, kb_bytes(16, FMT)), FMT>(p, fold, status, s);
-  if (t.bn == 32) return run<32, kb_stages(32, kb_bytes(32, FMT)), FMT>(p, fold, status, s);
-  if (t.bn == 64) return run<64, kb_stages(64, kb_bytes(64, FMT)), FMT>(p, fold, status, s);
-  if (t.bn == 128) return run<128, kb_stages(128, kb_bytes(128, FMT)), FMT>(p, fold, status, s);
-  // In tf32 a 128 x 256 tile on one CTA already feeds the tensor cores; pairs
-  // load a third less per tile from L2, which is what bounds short K, and pay
-  // once there are tiles for every pair: 53-qubit lattice in 3xTF32 23.3 -> 21.4 ms.
-  if (FMT == 0 && t.bn == 256 && p.M >= 2 * BM && p.pair >= 0) {
-    const int64_t groups = p.grp ? p.n_groups : (p.PC + fold - 1) / fold;
-    t.paired = groups * ((p.M + 2 * BM - 1) / (2 * BM)) * (fold > 1 ? 1 : (2 * p.N + 255) / 256) >= sm_count() / 2;
+  if (f.paired) return run_pair<FMT>(p, f.fold, status, s);
+  switch (f.bn) {
+    case 16: return run<16, kb_stages(16, kb_bytes(16, FMT)), FMT>(p, f.fold, status, s);
+    case 32: return run<32, kb_stages(32, kb_bytes(32, FMT)), FMT>(p, f.fold, status, s);
+    case 64: return run<64, kb_stages(64, kb_bytes(64, FMT)), FMT>(p, f.fold, status, s);
+    case 128: return run<128, kb_stages(128, kb_bytes(128, FMT)), FMT>(p, f.fold, status, s);
+    case 256: return run<256, kb_stages(256, kb_bytes(256, FMT)), FMT>(p, f.fold, status, s);
   }
-  if (t.paired) return run_pair<FMT>(p, fold, status, s);
-  return run<256, kb_stages(256, kb_bytes(256, FMT)), FMT>(p, fold, status, s);
+  return cudaErrorInvalidValue;
 }
 
 template <int FMT>

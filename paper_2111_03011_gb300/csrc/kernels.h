@@ -6,6 +6,7 @@
 #include <cstdint>
 
 #include "direct.h"
+#include "gemm_tile.h"
 
 namespace tn {
 
@@ -102,7 +103,7 @@ struct GemmParams {
   int h16;               // tensor-core engine: 0 tf32, 1 bf16, 2 scaled fp16 hi/lo operand planes
   const unsigned int* scaleA; const unsigned int* scaleB;   // h16 == 2: the operands' scale slots
   unsigned int* amax;    // non-null: atomicMax of the output's max |re|, |im| (fp32 bits)
-  int pair = 0;          // 0: CTA-pair 256 x 256 tiles where they apply (16-bit, M >= 256); -1: one-CTA tiles
+  int pair = 0;          // 0: CTA-pair 256 x 256 tiles where they apply (gemm_tile.h); -1: one-CTA tiles
   int tile_cap = 256;    // widest tile the dispatch may pick, real columns (16..256)
   // table of pattern groups (see gemm_tc.cu) of grp_fold patterns, or null
   const uint32_t* grp = nullptr;
@@ -112,13 +113,7 @@ struct GemmParams {
   int prepare = 0;       // 1: set the launched kernel's attributes first (no plan upload did)
 };
 
-// Tile a tensor-core GEMM launch runs with: BN real columns per tile, fold
-// patterns side by side in one tile, on CTA pairs or not.
-struct GemmTile {
-  int bn = 256, fold = 1;
-  bool paired = false;
-};
-GemmTile gemm_tc_tile(const GemmParams& p);
+GemmShape gemm_shape(const GemmParams& p);   // what the form of a launch depends on
 
 // C[p][c][r] = sum_k X[mapX(p)][r, k] Y[mapY(p)][k, c], operands where they lie
 struct DirectParams : DirectParamsBase, BatchParams {

@@ -1714,6 +1714,23 @@ int build_plan(const PlanInput& in, Plan& plan, std::string& err) {
 
 // ------------------------------------------------------------------- describe
 
+GemmShape step_gemm_shape(const Plan& plan, const Step& x) {
+  GemmShape g;
+  g.M = 1LL << x.nm;
+  g.N = 1LL << x.nn;
+  g.PA = x.PA;
+  g.PB = x.PB;
+  g.PC = x.PC;
+  g.mapA_mode = x.mapA_mode;
+  g.mapB_mode = x.mapB_mode;
+  g.h16 = x.h16;
+  g.pair = plan.gemm_pair < 0 ? -1 : x.pair;
+  g.tile_cap = x.tile_cap;
+  g.grp_fold = x.grp_fold;
+  g.n_groups = x.n_groups;
+  return g;
+}
+
 std::string describe_plan(const Plan& plan, bool with_data) {
   std::ostringstream o;
   o.precision(17);
@@ -1834,7 +1851,17 @@ std::string describe_plan(const Plan& plan, bool with_data) {
   }
   o << ",\"tc_macs\":" << plan.tc_macs << ",\"alg_bytes\":" << plan.alg_bytes << ",\"max_log2\":" << plan.max_log2
     << ",\"workspace_bytes\":" << plan.workspace_bytes << ",\"batch\":[" << plan.batch_max << "," << plan.batch_stride
-    << "]}";
+    << "],\"gemm_tiles\":[";
+  // tensor-core GEMM launches: step, rows and real columns after merging, tile width, patterns per tile, CTA pairs, groups
+  bool first = true;
+  for (size_t i = 0; i < plan.steps.size(); ++i) {
+    if (plan.steps[i].kind != ST_GEMM_TC) continue;
+    const GemmForm f = gemm_form(step_gemm_shape(plan, plan.steps[i]), kGemmSMs);
+    o << (first ? "" : ",") << "[" << i << "," << f.M << "," << 2 * f.N << "," << f.bn << "," << f.fold << ","
+      << (int)f.paired << "," << (int)f.grouped << "]";
+    first = false;
+  }
+  o << "]}";
   return o.str();
 }
 

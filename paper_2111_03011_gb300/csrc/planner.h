@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "direct.h"
+#include "gemm_tile.h"
 
 namespace tn {
 
@@ -235,6 +236,7 @@ struct PlanInput {
 // every pattern has its own B, in order).
 double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, bool b_own, double a, double b, double c,
                   bool h16);
+GemmShape step_gemm_shape(const Plan& plan, const Step& x);   // of a tensor-core GEMM step as it is set
 int build_plan(const PlanInput& in, Plan& plan, std::string& err);
 void apply_perm_schedule(Step& s, const PermSched& ps);
 std::string describe_plan(const Plan& plan, bool with_data);
