@@ -1005,22 +1005,25 @@ struct GemmVariant {
 constexpr GemmVariant kGemmVariants[] = {{256, 0}, {256, -1}, {128, 0}, {64, 0}, {32, 0}};
 constexpr int kNumGemmVariants = (int)(sizeof(kGemmVariants) / sizeof(kGemmVariants[0]));
 
-// Indices into kGemmVariants of the choices that launch differently for the
-// shape of tensor-core GEMM step x (independent of the plan-wide pair flag,
-// so that a step's variant numbers never change).
-std::vector<int> gemm_variants(const tn::Step& x) {
+// Indices into kGemmVariants of the choices that launch differently for
+// tensor-core GEMM step x (independent of the plan-wide pair flag, so that a
+// step's variant numbers never change): the launched form, merges included.  A
+// step with a table of pattern groups uses it whenever 256 columns are allowed;
+// its pattern-by-pattern variants are those narrower than a pattern's own tile.
+std::vector<int> gemm_variants(const tn::Plan& P, const tn::Step& x) {
   std::vector<int> out;
   std::vector<tn::GemmForm> seen;
   for (int v = 0; v < kNumGemmVariants; ++v) {
-    tn::GemmShape gs;
-    gs.M = 1LL << x.nm;
-    gs.N = 1LL << x.nn;
-    gs.PC = x.PC;
-    gs.mapA_mode = x.mapA_mode;
-    gs.h16 = x.h16;
+    tn::GemmShape gs = tn::step_gemm_shape(P, x);
     gs.pair = kGemmVariants[v].pair;
     gs.tile_cap = kGemmVariants[v].cap;
-    const tn::GemmForm t = tn::gemm_form(gs, 1 << 30);
+    tn::GemmForm t = tn::gemm_form(gs, tn::kGemmSMs);
+    if (t.grouped) {
+      const bool paired = t.paired;
+      gs.grp_fold = 0;
+      t = tn::gemm_form(gs, tn::kGemmSMs);
+      t.paired = paired;
+    }
     bool dup = false;
     for (const tn::GemmForm& q : seen) dup |= q.bn == t.bn && q.fold == t.fold && q.paired == t.paired;
     if (!dup) {
@@ -1031,17 +1034,28 @@ std::vector<int> gemm_variants(const tn::Step& x) {
   return out;
 }
 
-int step_variant_count(const tn::Step& x) {
-  if (x.kind == tn::ST_GEMM_TC) return (int)gemm_variants(x).size();
+// Whether a GEMM step of the plan runs on CTA pairs where they are allowed.
+bool any_paired(const tn::Plan& P) {
+  for (const tn::Step& x : P.steps) {
+    if (x.kind != tn::ST_GEMM_TC) continue;
+    tn::GemmShape gs = tn::step_gemm_shape(P, x);
+    gs.pair = x.pair;
+    if (tn::gemm_form(gs, tn::kGemmSMs).paired) return true;
+  }
+  return false;
+}
+
+int step_variant_count(const tn::Plan& P, const tn::Step& x) {
+  if (x.kind == tn::ST_GEMM_TC) return (int)gemm_variants(P, x).size();
   if (x.kind == tn::ST_PERMUTE) return std::max<int>(1, (int)x.alts.size());
   if (x.kind == tn::ST_BPREP_TC) return x.alts.empty() ? 1 : 2;
   return 1;
 }
 
-void apply_step_variant(tn::Step& x, int v) {
+void apply_step_variant(const tn::Plan& P, tn::Step& x, int v) {
   x.variant = v;
   if (x.kind == tn::ST_GEMM_TC) {
-    const GemmVariant& g = kGemmVariants[gemm_variants(x)[(size_t)v]];
+    const GemmVariant& g = kGemmVariants[gemm_variants(P, x)[(size_t)v]];
     x.tile_cap = g.cap;
     x.pair = g.pair;
   } else if (x.kind == tn::ST_PERMUTE && !x.alts.empty()) {
@@ -1063,7 +1077,7 @@ extern "C" int tn_plan_step_variants(const tn_plan_t* plan, int64_t i, int* n_va
   if (!plan) return fail(TN_ERR_INVALID, "NULL plan");
   if (i < 0 || i >= (int64_t)plan->P.steps.size()) return fail(TN_ERR_INVALID, "step index out of range");
   const tn::Step& x = plan->P.steps[(size_t)i];
-  if (n_variants) *n_variants = step_variant_count(x);
+  if (n_variants) *n_variants = step_variant_count(plan->P, x);
   if (chosen) *chosen = x.variant;
   return TN_OK;
 }
@@ -1072,9 +1086,9 @@ extern "C" int tn_plan_set_step_variant(tn_plan_t* plan, int64_t i, int variant)
   if (!plan) return fail(TN_ERR_INVALID, "NULL plan");
   if (i < 0 || i >= (int64_t)plan->P.steps.size()) return fail(TN_ERR_INVALID, "step index out of range");
   tn::Step& x = plan->P.steps[(size_t)i];
-  if (variant < 0 || variant >= step_variant_count(x)) return fail(TN_ERR_INVALID, "variant out of range");
+  if (variant < 0 || variant >= step_variant_count(plan->P, x)) return fail(TN_ERR_INVALID, "variant out of range");
   if (x.variant != variant) {
-    apply_step_variant(x, variant);
+    apply_step_variant(plan->P, x, variant);
     drop_graphs(plan);
   }
   return TN_OK;
@@ -1091,7 +1105,7 @@ extern "C" int tn_plan_tune_steps(tn_plan_t* plan, int reps, void* stream, doubl
   int max_v = 1;
   for (int64_t i = 0; i < ns; ++i) {
     start[i] = P.steps[i].variant;
-    count[i] = step_variant_count(P.steps[i]);
+    count[i] = step_variant_count(P, P.steps[i]);
     max_v = std::max(max_v, count[i]);
   }
   tn_head_t* h = nullptr;
@@ -1114,7 +1128,7 @@ extern "C" int tn_plan_tune_steps(tn_plan_t* plan, int reps, void* stream, doubl
   }
   auto set_all = [&](const std::vector<int>& v) {
     for (int64_t i = 0; i < ns; ++i)
-      if (P.steps[i].variant != v[i]) apply_step_variant(P.steps[i], v[i]);
+      if (P.steps[i].variant != v[i]) apply_step_variant(P, P.steps[i], v[i]);
   };
   // 1. per-step times of variant v of every step (v past a step's count: its default)
   std::vector<double> best_ms(ns, 1e300);
@@ -1799,9 +1813,9 @@ extern "C" int tn_plan_autotune(const tn_circuit* circuit, const tn_open_spec* o
     rc = tn_head_create(p, nullptr, &h);
     double ms = 1e300;
     if (rc == TN_OK) {
-      // with 16-bit operands, time the CTA-pair and the one-CTA GEMM tiles and
+      // where a GEMM runs on CTA pairs, time those and the one-CTA tiles and
       // keep the faster (unless the caller turned pairs off)
-      const bool both = o.gemm_pair == 0 && (o.gemm == TN_GEMM_TC_BF16X3 || o.gemm == TN_GEMM_TC_FP16X3);
+      const bool both = o.gemm_pair == 0 && any_paired(p->P);
       int best_pair = p->P.gemm_pair;
       for (int v = 0; v < (both ? 2 : 1) && rc == TN_OK; ++v) {
         if (both) p->P.gemm_pair = v == 0 ? 0 : -1;
