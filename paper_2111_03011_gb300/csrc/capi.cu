@@ -1685,7 +1685,16 @@ extern "C" int tn_gemm_c64(int engine, const void* A, const void* B, void* C, in
       const tn::DirectPlan d = tn::plan_direct(ds, fold != 0);
       if (d.seconds < best.seconds) best = d;
     }
-    if (best.seconds < tn::tc_seconds(nm, nn, nk, PC, mode[0] == 1, mode[1] == 0, (double)PA * (double)(M * K),
+    tn::GemmShape gs;
+    gs.M = M;
+    gs.N = N;
+    gs.PA = PA;
+    gs.PB = PB;
+    gs.PC = PC;
+    gs.mapA_mode = mode[0];
+    gs.mapB_mode = mode[1];
+    gs.h16 = h16;
+    if (best.seconds < tn::tc_seconds(tn::gemm_form(gs, tn::kGemmSMs), nk, (double)PA * (double)(M * K),
                                       (double)PB * (double)(K * N), (double)PC * (double)(M * N), h16 != 0)) {
       const size_t n_map = maps[0].size() + maps[1].size();
       ScratchLease lease(st);

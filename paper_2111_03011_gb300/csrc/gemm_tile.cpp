@@ -1,6 +1,7 @@
 #include "gemm_tile.h"
 
 #include <algorithm>
+#include <cmath>
 
 namespace tn {
 
@@ -41,18 +42,18 @@ GemmForm gemm_form(const GemmShape& s, int sm_count) {
   // the widest tiles allowed, a tile takes the columns of one group of it.
   const int64_t N2 = 2 * f.N;
   int64_t w = N2;
-  int64_t groups = f.PC;
+  f.groups = f.PC;
   f.grouped = s.grp_fold > 0 && f.mapA_mode == 2 && cap == 256;
   if (f.grouped) {
     f.fold = s.grp_fold;
     w = N2 * f.fold;
-    groups = s.n_groups;
+    f.groups = s.n_groups;
   } else if (f.mapA_mode == 1 && f.PC > 1 && N2 >= 16 && N2 < cap) {
     while (w < cap && f.fold < f.PC) {
       w *= 2;
       f.fold *= 2;
     }
-    groups = (f.PC + f.fold - 1) / f.fold;
+    f.groups = (f.PC + f.fold - 1) / f.fold;
   }
   while (f.bn < cap && f.bn < w) f.bn *= 2;
   // 256-wide tiles with at least 256 rows run on CTA pairs unless pair < 0.  In
@@ -62,10 +63,30 @@ GemmForm gemm_form(const GemmShape& s, int sm_count) {
   f.paired = f.bn == 256 && f.M >= 2 * kGemmRows && s.pair >= 0;
   if (f.paired && s.h16 == 0) {
     const int64_t tiles =
-        groups * ((f.M + 2 * kGemmRows - 1) / (2 * kGemmRows)) * (f.fold > 1 ? 1 : (N2 + 255) / 256);
+        f.groups * ((f.M + 2 * kGemmRows - 1) / (2 * kGemmRows)) * (f.fold > 1 ? 1 : (N2 + 255) / 256);
     f.paired = tiles >= sm_count / 2;
   }
   return f;
+}
+
+// To set against the direct form's time (plan_direct).  Measured on GB300: about
+// 4 us per launch; the passes stream at 5 TB/s and a GEMM writes C at 3.7 TB/s;
+// it runs its tiles of 128 rows x BN real columns in whole waves of 152, each SM
+// at its share of 280 (3xTF32) or 560 (16-bit) TFLOP/s for BN = 256, where an
+// MMA narrower than 128 columns takes as long as one of 128.  The tiles are those
+// of the launch: merged rows, joined columns and grouped patterns.  (Grouped ones
+// priced pattern by pattern kept 32 patterns of 2^8 x 2^4 x 2^9 on the GEMM, whose
+// 14 wide tiles take 41 us in one wave and 55 us with the preparations; the direct
+// form takes 25 us.)
+double tc_seconds(const GemmForm& f, int nk, double a, double b, double c, bool h16) {
+  const double tiles = (double)f.groups * (f.fold > 1 ? 1.0 : std::ceil(2.0 * (double)f.N / f.bn)) *
+                       std::ceil((double)f.M / kGemmRows);
+  const double peak = h16 ? 560e12 : 280e12;
+  const double tile_flops = 8.0 * kGemmRows * std::max(f.bn, 128) / 2.0 * std::ldexp(1.0, nk);
+  const double mma = std::ceil(tiles / kGemmSMs) * tile_flops * kGemmSMs / peak;
+  const double plane = h16 ? 8.0 : 16.0;
+  const double gemm = std::max(mma, plane * a / 5.0e12 + 8.0 * c / 3.7e12);
+  return gemm + (8.0 + plane) * a / 5.0e12 + (8.0 + 2.0 * plane) * b / 5.0e12 + 12e-6;
 }
 
 }  // namespace tn

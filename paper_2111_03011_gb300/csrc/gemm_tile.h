@@ -28,9 +28,15 @@ struct GemmForm {
   bool grouped = false;  // the table of pattern groups is used
   int bn = 16;           // real columns per tile: 16, 32, 64, 128 or 256
   int fold = 1;          // patterns side by side in a tile
+  int64_t groups = 1;    // sets of patterns that tiles cover
   bool paired = false;   // 256 x 256 tiles on CTA pairs
 };
 
 GemmForm gemm_form(const GemmShape& s, int sm_count);
+
+// Modelled time of a contraction that runs as f with 2^nk reductions: split
+// permute, B preparation and tensor-core GEMM (a, b, c: elements of the
+// operands and the result).
+double tc_seconds(const GemmForm& f, int nk, double a, double b, double c, bool h16);
 
 }  // namespace tn

@@ -943,33 +943,31 @@ static std::vector<uint32_t> group_patterns(const std::vector<uint32_t>& mapA, i
   return ids;
 }
 
-// Modelled time of a contraction as split permute, B preparation and
-// tensor-core GEMM, to set against the direct form's (plan_direct).  Measured
-// on GB300: about 4 us per launch; the passes stream at 5 TB/s and a
-// GEMM writes C at 3.7 TB/s; it runs
-// its tiles of 128 rows x BN real columns in whole waves of 152, each SM at
-// its share of 280 (3xTF32) or 560 (16-bit) TFLOP/s for BN >= 256, where an
-// MMA narrower than 128 columns takes as long as one of 128.
-double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, bool b_own, double a, double b, double c,
-                  bool h16) {
-  int64_t cols = 2LL << nn, groups = PC;
-  if (a_shared && b_own && cols < 16 && PC > 1) {   // one matrix of all patterns' columns
-    cols *= PC;
-    groups = 1;
-  }
-  if (a_shared && cols >= 16)
-    while (cols < 256 && groups > 1) {
-      cols *= 2;
-      groups = (groups + 1) / 2;
+// The groups for a step with 2^nn columns, up to 256 real columns side by side:
+// the width with the least MMA time (a tile of 128 columns takes 0.77 of one of
+// 256, narrower ones as long as one of 128).
+struct GroupTable {
+  int fold = 0;
+  int64_t n_groups = 0;
+  std::vector<uint32_t> tab;
+};
+
+static GroupTable best_groups(const std::vector<uint32_t>& mapA, int nn) {
+  GroupTable g;
+  double best = 1e300;
+  for (int fold = 1; fold == 1 || ((2LL << nn) >= 16 && ((2LL << nn) * fold) <= 256); fold *= 2) {
+    int64_t ng = 0;
+    std::vector<uint32_t> t = group_patterns(mapA, fold, ng);
+    const double cols = (double)(2LL << nn) * fold;
+    const double cost = (double)ng * (cols >= 256 ? cols / 256.0 : 0.77);
+    if (cost < best) {
+      best = cost;
+      g.tab.swap(t);
+      g.fold = fold;
+      g.n_groups = ng;
     }
-  const double bn = (double)std::min<int64_t>(256, std::max<int64_t>(cols, 16));
-  const double tiles = (double)groups * std::ceil((double)cols / bn) * std::ceil(std::ldexp(1.0, nm) / 128.0);
-  const double peak = h16 ? 560e12 : 280e12;
-  const double tile_flops = 8.0 * 128.0 * std::max(bn, 128.0) / 2.0 * std::ldexp(1.0, nk);
-  const double mma = std::ceil(tiles / 152.0) * tile_flops * 152.0 / peak;
-  const double plane = h16 ? 8.0 : 16.0;
-  const double gemm = std::max(mma, plane * a / 5.0e12 + 8.0 * c / 3.7e12);
-  return gemm + (8.0 + plane) * a / 5.0e12 + (8.0 + 2.0 * plane) * b / 5.0e12 + 12e-6;
+  }
+  return g;
 }
 
 static int layout_steps(Plan& plan, std::string& err) {
@@ -1064,7 +1062,23 @@ static int layout_steps(Plan& plan, std::string& err) {
         if (d.seconds < dp.seconds) dp = d;
       }
     }
-    const bool direct = dp.seconds < tc_seconds(nm, nn, nk, C.P, mapA_mode == 1, mapB_mode == 0, (double)vt_elems(big),
+    // what the GEMM would run as, its patterns grouped by the A pattern they read
+    GroupTable groups;
+    GemmShape shape;
+    shape.M = 1LL << nm;
+    shape.N = 1LL << nn;
+    shape.PA = big.P;
+    shape.PB = sml.P;
+    shape.PC = C.P;
+    shape.mapA_mode = mapA_mode;
+    shape.mapB_mode = mapB_mode;
+    shape.h16 = h16_step ? 1 : 0;
+    if (!use_small && plan.gemm_engine != TN_GEMM_SIMT_FP32 && mapA_mode == 2 && big.P < C.P && C.P < (1LL << 24)) {
+      groups = best_groups({plan.meta.begin() + mapA_off, plan.meta.begin() + mapA_off + C.P}, nn);
+      shape.grp_fold = groups.fold;
+      shape.n_groups = groups.n_groups;
+    }
+    const bool direct = dp.seconds < tc_seconds(gemm_form(shape, kGemmSMs), nk, (double)vt_elems(big),
                                                 (double)vt_elems(sml), (double)C.P * std::exp2(nm + nn), h16_step);
     if (use_small || (direct && !dp.swap)) {
       for (int l : M) cl.push_back(l);
@@ -1207,26 +1221,10 @@ static int layout_steps(Plan& plan, std::string& err) {
       g.nk = nk; g.nm = nm; g.nn = nn;
       g.mapA_mode = mapA_mode; g.mapA_off = mapA_off;
       g.mapB_mode = mapB_mode; g.mapB_off = mapB_off;
-      if (tc && mapA_mode == 2 && big.P < C.P && C.P < (1LL << 24)) {
-        // patterns with one A pattern side by side, up to 256 columns: the
-        // width with the least MMA time (a tile of 128 columns takes 0.77 of
-        // one of 256, narrower ones as long as one of 128)
-        const std::vector<uint32_t> ma(plan.meta.begin() + mapA_off, plan.meta.begin() + mapA_off + C.P);
-        double best = 1e300;
-        std::vector<uint32_t> tab;
-        for (int fold = 1; fold == 1 || ((2LL << nn) >= 16 && ((2LL << nn) * fold) <= 256); fold *= 2) {
-          int64_t ng = 0;
-          std::vector<uint32_t> t = group_patterns(ma, fold, ng);
-          const double cols = (double)(2LL << nn) * fold;
-          const double cost = (double)ng * (cols >= 256 ? cols / 256.0 : 0.77);
-          if (cost < best) {
-            best = cost;
-            tab.swap(t);
-            g.grp_fold = fold;
-            g.n_groups = ng;
-          }
-        }
-        g.grp_off = meta_push(plan, tab);
+      if (tc && groups.fold > 0) {
+        g.grp_fold = groups.fold;
+        g.n_groups = groups.n_groups;
+        g.grp_off = meta_push(plan, groups.tab);
       }
       g.macs = macs;
       g.bytes = 8.0 * (double)(vt_elems(big) + eC) + (double)bprep_bytes;

@@ -231,11 +231,6 @@ struct PlanInput {
   bool side_bprep = false;  // B-prep steps whose operand is ready run beside the previous GEMM
 };
 
-// Modelled time of a contraction as split permute, B preparation and
-// tensor-core GEMM (a, b, c: elements of the operands and the result; b_own:
-// every pattern has its own B, in order).
-double tc_seconds(int nm, int nn, int nk, int64_t PC, bool a_shared, bool b_own, double a, double b, double c,
-                  bool h16);
 GemmShape step_gemm_shape(const Plan& plan, const Step& x);   // of a tensor-core GEMM step as it is set
 int build_plan(const PlanInput& in, Plan& plan, std::string& err);
 void apply_perm_schedule(Step& s, const PermSched& ps);

@@ -1,7 +1,8 @@
 """Which tile a tensor-core GEMM runs on.  The rule is checked on the CPU, from
 its own source, over every kind of shape: a width that a kernel exists for, no
 wider than the columns need, folds that the kernels accept, merges that keep the
-work.  Plans with narrow gathered steps (a table of pattern groups, fewer than
+work; and the modelled time is that of the merged, joined or grouped launch.
+Merged rows are compared with NumPy on the GPU.  Plans with narrow gathered steps (a table of pattern groups, fewer than
 16 real columns) are contracted on the GPU and compared with the state vector."""
 import os
 import subprocess
@@ -18,6 +19,7 @@ CHECK = r"""
 #include "gemm_tile.h"
 #include <algorithm>
 #include <cstdio>
+#include <initializer_list>
 using namespace tn;
 int main() {
   long bad = 0, seen = 0;
@@ -60,6 +62,56 @@ def test_tile_rule(tmp_path):
     assert subprocess.run([str(exe)], stdout=subprocess.PIPE, check=True).stdout == b"0 1\n"
 
 
+MODEL = r"""
+#include "gemm_tile.h"
+#include <cstdio>
+#include <initializer_list>
+using namespace tn;
+static double t(const GemmShape& s) {
+  return tc_seconds(gemm_form(s, kGemmSMs), 9, 1e6, 1e5, 1e6, s.h16 != 0);
+}
+int main() {
+  int bad = 0;
+  for (int h16 = 0; h16 < 2; ++h16)
+    for (int64_t P : {2, 64, 400, 3000}) for (int64_t M : {1, 2, 16}) for (int64_t N : {1, 4, 64, 512}) {
+      GemmShape s, r;
+      s.h16 = r.h16 = h16;
+      // own A, shared B: one GEMM of P M rows
+      s.M = M; s.N = N; s.PA = s.PC = P; s.mapA_mode = 0; s.mapB_mode = 1;
+      r.M = P * M; r.N = N;
+      bad += t(s) != t(r);
+      // shared A, own narrow B: one GEMM of P N columns
+      if (2 * N < 16) {
+        s = GemmShape(); r = GemmShape();
+        s.h16 = r.h16 = h16;
+        s.M = 4096; s.N = N; s.PB = s.PC = P; s.mapB_mode = 0;
+        r.M = 4096; r.N = P * N;
+        bad += t(s) != t(r);
+      }
+      // gathered A in groups of 4: as many patterns of 4 N columns
+      if (2 * N >= 16 && 8 * N <= 256) {
+        s = GemmShape(); r = GemmShape();
+        s.h16 = r.h16 = h16;
+        s.M = 2048; s.N = N; s.PA = 7; s.PB = 9; s.PC = P; s.mapA_mode = s.mapB_mode = 2;
+        s.grp_fold = 4; s.n_groups = (P + 3) / 4 + 3;
+        r.M = 2048; r.N = 4 * N; r.PA = 7; r.PB = 9; r.PC = s.n_groups; r.mapA_mode = r.mapB_mode = 2;
+        bad += t(s) != t(r);
+      }
+    }
+  std::printf("%d\n", bad);
+  return 0;
+}
+"""
+
+
+def test_modelled_time_is_that_of_the_launch(tmp_path):
+    src, exe = tmp_path / "model.cpp", tmp_path / "model"
+    src.write_text(MODEL)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), os.path.join(CSRC, "gemm_tile.cpp"), "-o",
+                    str(exe)], check=True)
+    assert subprocess.run([str(exe)], stdout=subprocess.PIPE, check=True).stdout == b"0\n"
+
+
 CIRCUITS = [dict(r=4, c=4, m=8, L=24, seed=0), dict(r=4, c=5, m=10, L=50, seed=1), dict(r=3, c=6, m=9, L=40, seed=2)]
 IDS = [f"{c['r']}x{c['c']}" for c in CIRCUITS]
 
@@ -99,3 +151,30 @@ def test_plans_with_narrow_gathered_steps(case, gemm):
     bits = np.array([O.bitstring_index(int(t), oq, mu) for t in tails for mu in range(1 << len(oq))], np.uint64)
     H = tn.tn_amplitudes(head, bits).reshape(len(tails), -1)
     assert np.linalg.norm(H - ref) <= (1e-4 if gemm == 3 else 1e-5) * np.linalg.norm(ref)
+
+
+# (M, N, K, patterns): ragged last row tiles of one CTA and of pairs, one row a
+# pattern, columns narrower than 16 and K = 2
+ROWS = [(64, 16, 32, 3), (128, 128, 64, 3), (1, 64, 64, 217), (2, 64, 1024, 130), (256, 256, 16, 5), (8, 2, 128, 77),
+        (16, 512, 2, 50)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("gemm", [1, 3, 4])
+@pytest.mark.parametrize("pair", [1, -1])
+@pytest.mark.parametrize("shape", ROWS, ids=str)
+def test_merged_rows(gemm, pair, shape):
+    """Every pattern its own A, one B for all.  Relative L2 as for any GEMM: 1e-5
+    (3xTF32, FP16x3) or 1e-4 (BF16x3)."""
+    import torch
+    import paper_2111_03011_gb300 as tn
+    M, N, K, P = shape
+    rng = np.random.default_rng(M + N + K + P)
+    A, B = ((rng.normal(size=s) + 1j * rng.normal(size=s)).astype(np.complex64) for s in ((P, M, K), (1, K, N)))
+    ref = A.astype(np.complex128) @ B.astype(np.complex128)
+    buf = torch.full((P * M * N + 2,), float("nan"), dtype=torch.complex64, device="cuda")
+    c = buf[1:-1].view(P, M, N)
+    tn.tn_gemm_c64(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), c, engine=gemm, pair=pair)
+    assert np.linalg.norm(c.cpu().numpy() - ref) <= (1e-4 if gemm == 3 else 1e-5) * np.linalg.norm(ref)
+    rest = buf.cpu().numpy()
+    assert np.isnan(rest[0]) and np.isnan(rest[-1])
