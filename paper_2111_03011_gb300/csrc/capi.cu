@@ -106,6 +106,9 @@ extern "C" const char* tn_version(void) { return kVersion; }
 // its duration, so calls from several threads and streams share none.  Between
 // calls at most kMost are kept, with at most kKeepBytes of buffers among them;
 // all of it is given back when a device allocation of the library fails.
+// Every call that takes one synchronises its stream, which CUDA refuses while any
+// stream is captured in global mode (and which ends that capture); beside a
+// thread-local capture of another thread it may allocate and free.
 struct CallScratch {
   tn::HeadReport* rep = nullptr;
   double* part = nullptr;
@@ -191,13 +194,6 @@ struct ScratchLease {
         g_scratch.erase(g_scratch.begin() + (std::ptrdiff_t)at);
       }
     }
-    // allocations below must not end a stream capture that another thread has begun
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    struct Restore {
-      cudaStreamCaptureMode mode;
-      ~Restore() { cudaThreadExchangeStreamCaptureMode(&mode); }
-    } restore{mode};
     if (!c.rep) {
       c.device = dev;
       void* h = nullptr;
