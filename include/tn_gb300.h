@@ -429,8 +429,8 @@ int  tn_head_norm_noalloc(const void* head_c128, int64_t n_groups, int n_open, d
  * that engine) where it is modelled faster (small or narrow shapes).  pair = -1: one-CTA GEMM tiles,
  * pair > 0: the GEMM kernels with CTA pairs where they apply.  Its
  * scratch (split planes, prepared B, maps) comes from a bounded pool that the
- * library keeps between calls (at most 2 GiB, given back when an allocation
- * fails); it synchronises `stream`.  TN_ERR_TIMEOUT if a bounded device
+ * library keeps between calls (at most 2 GiB, given back when an allocation of
+ * the library fails or its server needs room); it synchronises `stream`.  TN_ERR_TIMEOUT if a bounded device
  * wait gave up. */
 int  tn_gemm_c64(int engine, const void* A, const void* B, void* C, int64_t M, int64_t N, int64_t K,
                  int64_t PA, int64_t PB, int64_t PC, const int32_t* mapA, const int32_t* mapB, int pair,

@@ -130,14 +130,17 @@ static void free_scratch(CallScratch& c) {
   c = CallScratch();
 }
 
-static void trim_scratch() {
-  std::lock_guard<std::mutex> lock(g_scratch_mu);
-  for (CallScratch& c : g_scratch) free_scratch(c);
-  g_scratch.clear();
+namespace tn {
+void trim_scratch() {
+  std::vector<CallScratch> kept;
+  {
+    std::lock_guard<std::mutex> lock(g_scratch_mu);
+    kept.swap(g_scratch);
+  }
+  for (CallScratch& c : kept) free_scratch(c);
 }
 
-// cudaMalloc that gives the kept scratch back and tries again before it fails
-static cudaError_t malloc_or_trim(void** p, size_t bytes) {
+cudaError_t device_malloc(void** p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
@@ -146,6 +149,7 @@ static cudaError_t malloc_or_trim(void** p, size_t bytes) {
   }
   return e;
 }
+}  // namespace tn
 
 struct ScratchLease {
   static constexpr size_t kMost = 32, kKeepBytes = (size_t)2 << 30;
@@ -160,8 +164,8 @@ struct ScratchLease {
     if (in_flight) cudaStreamSynchronize(stream);   // the call failed after a launch
     {
       std::lock_guard<std::mutex> lock(g_scratch_mu);
-      size_t kept = c.bytes;
-      for (const CallScratch& o : g_scratch) kept += o.bytes;
+      size_t kept = c.bytes + c.host_bytes;
+      for (const CallScratch& o : g_scratch) kept += o.bytes + o.host_bytes;
       if (g_scratch.size() < kMost && kept <= kKeepBytes) {
         g_scratch.push_back(c);
         return;
@@ -198,7 +202,7 @@ struct ScratchLease {
       c.device = dev;
       void* h = nullptr;
       if (cudaHostAlloc(&h, sizeof(tn::HeadReport), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
-          malloc_or_trim((void**)&c.part, 2 * tn::kHeadParts * sizeof(double)) != cudaSuccess) {
+          tn::device_malloc((void**)&c.part, 2 * tn::kHeadParts * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         if (h) cudaFreeHost(h);
         return fail(TN_ERR_OOM, "scratch allocation failed");
@@ -209,7 +213,7 @@ struct ScratchLease {
       cudaFree(c.buf);
       c.buf = nullptr;
       c.bytes = 0;
-      if (malloc_or_trim(&c.buf, bytes) != cudaSuccess) {
+      if (tn::device_malloc(&c.buf, bytes) != cudaSuccess) {
         cudaGetLastError();
         return fail(TN_ERR_OOM, "scratch allocation failed");
       }
@@ -268,14 +272,14 @@ static int plan_upload(tn_plan_t* p) {
   for (size_t i = 0; i < leaves.size(); ++i)
     leaves[i] = make_float2((float)P.leaf_arena[i].real(), (float)P.leaf_arena[i].imag());
   p->on_device = true;
-  CUDA_TRY(cudaMalloc(&p->d_leaves, std::max<size_t>(leaves.size(), 1) * sizeof(float2)));
+  CUDA_TRY(tn::device_malloc((void**)&p->d_leaves, std::max<size_t>(leaves.size(), 1) * sizeof(float2)));
   if (!leaves.empty())
     CUDA_TRY(cudaMemcpy(p->d_leaves, leaves.data(), leaves.size() * sizeof(float2), cudaMemcpyHostToDevice));
-  CUDA_TRY(cudaMalloc(&p->d_meta, std::max<size_t>(P.meta.size(), 1) * sizeof(uint32_t)));
+  CUDA_TRY(tn::device_malloc((void**)&p->d_meta, std::max<size_t>(P.meta.size(), 1) * sizeof(uint32_t)));
   if (!P.meta.empty())
     CUDA_TRY(cudaMemcpy(p->d_meta, P.meta.data(), P.meta.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
   if (P.workspace_bytes > 0) {
-    cudaError_t e = malloc_or_trim((void**)&p->d_arena, (size_t)P.workspace_bytes);
+    cudaError_t e = tn::device_malloc((void**)&p->d_arena, (size_t)P.workspace_bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(TN_ERR_OOM, "workspace of " + std::to_string(P.workspace_bytes) + " bytes: " + cudaGetErrorString(e));
@@ -290,20 +294,20 @@ static int plan_upload(tn_plan_t* p) {
   std::vector<uint32_t> grp(L);
   for (size_t i = 0; i < L; ++i) { keys[i] = kv[i].first; grp[i] = kv[i].second; }
   p->n_keys = (int64_t)L;
-  CUDA_TRY(cudaMalloc(&p->d_keys, L * sizeof(uint64_t)));
-  CUDA_TRY(cudaMalloc(&p->d_key_groups, L * sizeof(uint32_t)));
-  CUDA_TRY(cudaMalloc(&p->d_tails, L * sizeof(uint64_t)));
+  CUDA_TRY(tn::device_malloc((void**)&p->d_keys, L * sizeof(uint64_t)));
+  CUDA_TRY(tn::device_malloc((void**)&p->d_key_groups, L * sizeof(uint32_t)));
+  CUDA_TRY(tn::device_malloc((void**)&p->d_tails, L * sizeof(uint64_t)));
   CUDA_TRY(cudaMemcpy(p->d_keys, keys.data(), L * sizeof(uint64_t), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(p->d_key_groups, grp.data(), L * sizeof(uint32_t), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(p->d_tails, P.tails_raw.data(), L * sizeof(uint64_t), cudaMemcpyHostToDevice));
   const size_t h = P.open_qubits.size();
-  CUDA_TRY(cudaMalloc(&p->d_open, std::max<size_t>(h, 1) * sizeof(int)));
+  CUDA_TRY(tn::device_malloc((void**)&p->d_open, std::max<size_t>(h, 1) * sizeof(int)));
   if (h) CUDA_TRY(cudaMemcpy(p->d_open, P.open_qubits.data(), h * sizeof(int), cudaMemcpyHostToDevice));
-  CUDA_TRY(cudaMalloc(&p->d_status, sizeof(unsigned int)));
+  CUDA_TRY(tn::device_malloc((void**)&p->d_status, sizeof(unsigned int)));
   CUDA_TRY(cudaMemset(p->d_status, 0, sizeof(unsigned int)));
   const size_t n_static = P.scale_static.size(), n_slots = n_static + (size_t)P.n_scale_slots * P.batch_max;
   if (n_slots > 0) {
-    CUDA_TRY(cudaMalloc(&p->d_scale, n_slots * sizeof(unsigned int)));
+    CUDA_TRY(tn::device_malloc((void**)&p->d_scale, n_slots * sizeof(unsigned int)));
     CUDA_TRY(cudaMemset(p->d_scale, 0, n_slots * sizeof(unsigned int)));
     if (n_static)
       CUDA_TRY(cudaMemcpy(p->d_scale, P.scale_static.data(), n_static * sizeof(unsigned int), cudaMemcpyHostToDevice));
@@ -462,7 +466,7 @@ extern "C" int tn_head_create(tn_plan_t* plan, void* dev_c128, tn_head_t** out) 
   if (dev_c128) {
     h->H = (double2*)dev_c128;
   } else {
-    cudaError_t e = malloc_or_trim((void**)&h->H, (size_t)elems * sizeof(double2));
+    cudaError_t e = tn::device_malloc((void**)&h->H, (size_t)elems * sizeof(double2));
     if (e != cudaSuccess) {
       cudaGetLastError();
       delete h;
@@ -472,7 +476,7 @@ extern "C" int tn_head_create(tn_plan_t* plan, void* dev_c128, tn_head_t** out) 
   }
   cudaError_t e1 = cudaMemset(h->H, 0, (size_t)elems * sizeof(double2));
   if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(0);   // zeroed before any stream, blocking or not, uses it
-  cudaError_t e2 = cudaMalloc(&h->d_Z, (size_t)std::max<int64_t>(L, 1) * sizeof(double));
+  cudaError_t e2 = tn::device_malloc((void**)&h->d_Z, (size_t)std::max<int64_t>(L, 1) * sizeof(double));
   if (e1 != cudaSuccess || e2 != cudaSuccess) {
     cudaGetLastError();
     tn_head_free(h);
@@ -1413,7 +1417,7 @@ static int ensure_stage(tn_head* h, size_t bytes) {
   cudaFree(h->d_stage);
   h->d_stage = nullptr;
   h->stage_bytes = 0;
-  cudaError_t e = malloc_or_trim(&h->d_stage, bytes);
+  cudaError_t e = tn::device_malloc(&h->d_stage, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(TN_ERR_OOM, "staging buffer allocation failed");

@@ -78,6 +78,11 @@ struct tn_head {
 
 namespace tn {
 void set_last_error(const std::string& msg);
+// cudaMalloc for everything that the library keeps on the device: it gives the
+// scratch that calls have left behind (capi.cu) back and tries again before it
+// fails.  trim_scratch gives that scratch back at once.
+cudaError_t device_malloc(void** p, size_t bytes);
+void trim_scratch();
 // Enqueue the slices of `r` of `plan` into H on `stream` (no range checks).
 // On failure *done_end (if given) is the end of the leading sub-range whose
 // slices were enqueued whole, or -1 if a slice was left partly accumulated.

@@ -105,7 +105,7 @@ int ensure_slot_buffers(Slot& s, size_t dev_bytes, size_t host_bytes) {
     cudaFree(s.d_buf);
     s.d_buf = nullptr;
     s.d_cap = 0;
-    if (cudaMalloc(&s.d_buf, dev_bytes) != cudaSuccess) {
+    if (tn::device_malloc(&s.d_buf, dev_bytes) != cudaSuccess) {
       cudaGetLastError();
       return TN_ERR_OOM;
     }
@@ -278,11 +278,19 @@ constexpr int64_t kHbmReserve = (int64_t)1 << 30;
 
 // Admission by memory: a new head must fit both the byte budget and the
 // device's free memory as the driver reports it now (cudaMemGetInfo), less a
-// reserve.  Least-recently-used idle heads are freed until it does.
+// reserve.  Scratch that other calls have left with the library counts as used
+// there, so it is given back first; then least-recently-used idle heads are
+// freed until the new one fits.
 bool make_room(tn_server* sv, int64_t need) {
+  bool trimmed = false;
   while (true) {
     size_t fr = 0, tot = 0;
     const bool dev_ok = cudaMemGetInfo(&fr, &tot) != cudaSuccess || (int64_t)fr >= need + kHbmReserve;
+    if (!dev_ok && !trimmed) {
+      trimmed = true;
+      tn::trim_scratch();
+      continue;
+    }
     if (sv->head_bytes + need <= sv->opts.hbm_budget_bytes && dev_ok) return true;
     int victim = -1;
     for (size_t i = 0; i < sv->circuits.size(); ++i) {
@@ -437,6 +445,7 @@ extern "C" int tn_server_create(const tn_server_opts* opts, tn_server_t** out) {
   if (opts && opts->hbm_budget_bytes > 0) {
     sv->opts.hbm_budget_bytes = opts->hbm_budget_bytes;
   } else {   // the device's free memory now, less the reserve
+    tn::trim_scratch();
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
       cudaGetLastError();
@@ -452,7 +461,7 @@ extern "C" int tn_server_create(const tn_server_opts* opts, tn_server_t** out) {
   for (auto& s : sv->slots) {
     if (cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess ||
-        cudaMalloc(&s.d_status, sizeof(unsigned long long)) != cudaSuccess ||
+        tn::device_malloc((void**)&s.d_status, sizeof(unsigned long long)) != cudaSuccess ||
         cudaMallocHost(&s.h_status, sizeof(unsigned long long)) != cudaSuccess) {
       cudaGetLastError();
       tn_server_free(sv);

@@ -1,7 +1,10 @@
-"""Scratch that the library keeps between calls."""
+"""Scratch that the library keeps between calls: it stands in no other call's way."""
 import threading
 
+import numpy as np
 import pytest
+
+import circuit_inputs as ci
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +52,35 @@ def test_scratch_beyond_the_pool_leaves_a_capture_alone(tn):
     torch.cuda.synchronize()
     assert x.tolist() == [6.0] * 8
     assert float((c - (1 << 13)).abs().max()) <= 1e-5 * (1 << 13)
+
+
+def test_server_counts_kept_scratch_as_free(tn):
+    """700 MiB free beside 1 GiB of kept scratch: a request whose head needs the
+    server's reserve of 1 GiB is admitted (the scratch is given back), and nothing
+    else had to go."""
+    import torch
+    cfg = ci.config_small(4, 4, 8, seed=11, n_open=6, L=8, n_cut_gates=1)
+    plan = tn.tn_plan(cfg["circuit"], cfg["open_qubits"], cfg["tails"], cfg["edges"])
+    n = 1 << tn.tn_plan_get_stats(plan)["n_sliced"]
+    head = tn.tn_head_create(plan)
+    tn.tn_contract_slices(plan, 0, n, head)
+    bits = np.array([int(t) | (mu << 10) for t in cfg["tails"] for mu in range(64)], dtype=np.uint64)
+    want = tn.tn_amplitudes(head, bits)
+    sv = tn.tn_server_create(n_slots=2, hbm_budget_bytes=1 << 30)
+    cid = tn.tn_server_add_circuit(sv, plan, 0, n)
+    tn.tn_gemm_c64(*_operands(1 << 13, 16, 1 << 13), engine=1, pair=1)     # planes of 1 GiB
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (700 << 20), dtype=torch.uint8, device="cuda")
+    got = []
+    ticket = tn.tn_server_submit(sv, cid, tn.TN_REQ_AMPLITUDES, 0, bitstrings=bits)
+    t = threading.Thread(target=lambda: got.append(tn.tn_server_wait(sv, ticket)[0]))
+    t.start()
+    t.join(20)
+    waited = t.is_alive()
+    del fill
+    torch.cuda.empty_cache()                   # a request that waits for memory has it now
+    t.join(60)
+    st = tn.tn_server_get_stats(sv)
+    tn.tn_server_free(sv)
+    assert np.array_equal(got[0], want) and not waited and st["evictions"] == 0
