@@ -269,9 +269,11 @@ int  tn_contract_slices(tn_plan_t* plan, tn_range slice_range, tn_head_t* head, 
  * tn_contract_batch: items (plans[i], ranges[i], heads[i]) as parallel
  * branches of one graph (items of the same plan share a branch, since they
  * share its workspace), so many small contractions overlap on the GPU.  The
- * first time a thread submits a batch it is launched on branch streams; from
- * the second time on its captured graph is replayed (the last 8 batches'
- * graphs are kept per thread).  Both asynchronous on `stream`; both reject slices already
+ * first time a thread submits a batch whose heads are empty and in memory of the
+ * library's that tn_head_data has not handed out, it is launched on branch
+ * streams; otherwise, and from the second time on, as a captured graph (the last
+ * 8 batches' graphs are kept per thread).  A submission that fails leaves every
+ * head as it was.  Both asynchronous on `stream`; both reject slices already
  * accumulated into a head, and a batch rejects a head listed twice.  Items
  * with an empty range record nothing.  tn_contract_slices_graph keeps at most
  * 16 captured ranges per plan and drops the least recently replayed one. */

@@ -494,12 +494,19 @@ extern "C" void tn_head_free(tn_head_t* h) {
   delete h;
 }
 
-extern "C" void* tn_head_data(tn_head_t* h) { return h ? (void*)h->H : nullptr; }
+extern "C" void* tn_head_data(tn_head_t* h) {
+  if (!h) return nullptr;
+  h->exposed = true;
+  return h->H;
+}
+
+static int64_t head_elems(const tn_head_t* h) {
+  return (int64_t)h->plan->P.tails_raw.size() << h->plan->P.open_qubits.size();
+}
 
 extern "C" int tn_head_reset(tn_head_t* h, void* stream) {
   if (!h) return fail(TN_ERR_INVALID, "NULL head");
-  const int64_t elems = (int64_t)h->plan->P.tails_raw.size() << h->plan->P.open_qubits.size();
-  CUDA_TRY(cudaMemsetAsync(h->H, 0, (size_t)elems * sizeof(double2), (cudaStream_t)stream));
+  CUDA_TRY(cudaMemsetAsync(h->H, 0, (size_t)head_elems(h) * sizeof(double2), (cudaStream_t)stream));
   h->done.clear();
   h->slices_done = 0;
   h->f_override = false;
@@ -1341,9 +1348,9 @@ extern "C" int tn_contract_batch(tn_plan_t* const* plans, const tn_range* ranges
   const int n_branches = std::min<int>((int)branch_of_plan.size(), 32);
   for (int i = 0; i < n; ++i) branch[i] %= n_branches;
   // A batch is known by its handles' serials (never reused) and ranges.  The
-  // first time one is seen its launches go straight to the branch streams,
-  // which takes less host time than capturing and instantiating a graph; from
-  // the second time on a captured graph is replayed.  Per thread, the graphs
+  // first time one is seen its launches may go straight to the branch streams
+  // (below), which takes less host time than capturing and instantiating a graph;
+  // from the second time on a captured graph is replayed.  Per thread, the graphs
   // of the kBatchGraphs batches replayed last are kept, and the keys of the
   // kBatchSeen seen last.
   struct Batch {
@@ -1375,16 +1382,22 @@ extern "C" int tn_contract_batch(tn_plan_t* const* plans, const tn_range* ranges
   it->last_use = ++clock;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   CUDA_TRY(cudaStreamIsCapturing((cudaStream_t)stream, &cap));
-  // into a capture of the caller's, and with a fault armed (which must leave
-  // every head as it was), only as a graph
-  if (!seen && cap == cudaStreamCaptureStatusNone && !std::getenv("TN_FAULT_INJECT")) {
+  // Launched directly where a failure on the way can be undone: heads that are
+  // still zero and that nobody else can write.  Otherwise, and into a capture of
+  // the caller's, only as a graph, which runs whole or not at all.
+  bool undoable = cap == cudaStreamCaptureStatusNone;
+  for (int i = 0; i < n; ++i)
+    undoable = undoable && (R[i].begin == R[i].end || (Hs[i]->owns && !Hs[i]->exposed && Hs[i]->done.empty()));
+  if (!seen && undoable) {
     std::vector<cudaStream_t>* streams = nullptr;
     if (int rc = branch_streams(n_branches + 1, &streams)) return rc;
-    const int rc = fork_items(P, R, Hs, branch, n_branches, (cudaStream_t)stream, *streams);
-    if (rc) {   // a launch failed: which passes reached the heads is not recorded
+    if (const int rc = fork_items(P, R, Hs, branch, n_branches, (cudaStream_t)stream, *streams)) {
       for (int i = 0; i < n; ++i)
-        if (R[i].begin < R[i].end) Hs[i]->invalid = true;
-      g_err += "; the heads of the batch are invalid until tn_head_reset";
+        if (R[i].begin < R[i].end && cudaMemsetAsync(Hs[i]->H, 0, (size_t)head_elems(Hs[i]) * sizeof(double2),
+                                                     (cudaStream_t)stream) != cudaSuccess) {
+          cudaGetLastError();
+          Hs[i]->invalid = true;
+        }
       return rc;
     }
   } else {

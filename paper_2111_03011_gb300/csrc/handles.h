@@ -62,6 +62,7 @@ struct tn_head {
   tn_plan_t* plan = nullptr;
   double2* H = nullptr;
   bool owns = false;
+  bool exposed = false;              // tn_head_data has handed H out: others may write it
   std::map<int64_t, int64_t> done;   // begin -> end of accumulated slice ranges
   int64_t slices_done = 0;
   // set when H may hold part of a slice (a call failed between the passes of
