@@ -260,7 +260,8 @@ int  tn_head_set_fidelity(tn_head_t* head, double f_est);
  * CUDA call), "slice:S" or "slice:S:T" (the contraction fails with
  * TN_ERR_CUDA before pass T, default 0, of user slice S), "status" (every
  * successful tn_contract_slices sets the plan's device status word, as a wait
- * that gave up would). */
+ * that gave up would), "scratch:B" (scratch of more than B bytes for one call
+ * cannot be had: TN_ERR_OOM where the call cannot do with less). */
 int  tn_contract_slices(tn_plan_t* plan, tn_range slice_range, tn_head_t* head, void* stream);
 
 /* Batched form.  tn_contract_slices_graph: the same result as

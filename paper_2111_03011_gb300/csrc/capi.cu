@@ -81,6 +81,10 @@ bool fault_slice(int64_t s, int64_t t) {
   return s == S && t == T;
 }
 bool fault_status() { return fault_env() == "status"; }
+size_t fault_scratch() {
+  const std::string f = fault_env();
+  return f.rfind("scratch:", 0) == 0 ? (size_t)std::strtoull(f.c_str() + 8, nullptr, 10) : (size_t)-1;
+}
 
 // After the caller's stream is synchronised: a nonzero device status word of
 // the plan means a bounded wait of a tensor-core GEMM gave up in some
@@ -182,7 +186,7 @@ struct ScratchLease {
   int take(size_t bytes, size_t host_bytes = 0) {
     int dev = -1;
     CUDA_TRY(cudaGetDevice(&dev));
-    {
+    if (!c.rep) {   // (one that a failed attempt has taken is used again)
       // the kept one with the smallest buffer that is large enough, else the largest
       std::lock_guard<std::mutex> lock(g_scratch_mu);
       g_scratch.reserve(kMost);
@@ -209,6 +213,8 @@ struct ScratchLease {
       }
       c.rep = (tn::HeadReport*)h;   // one address on host and device (unified addressing)
     }
+    if (bytes > tn::fault_scratch())
+      return fail(TN_ERR_OOM, "scratch allocation failed (injected: TN_FAULT_INJECT=scratch)");
     if (c.bytes < bytes) {
       cudaFree(c.buf);
       c.buf = nullptr;
@@ -1585,9 +1591,13 @@ static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t
     d_out = (uint64_t*)h->d_stage;
   }
   ScratchLease lease(st);
-  if (int rc = lease.take(8 * tn::sample_scratch_doubles((int64_t)p->P.tails_raw.size(),
-                                                         (int)p->P.open_qubits.size(), n, method)))
-    return rc;
+  const int n_open = (int)p->P.open_qubits.size();
+  int64_t groups = tn::sample_groups((int64_t)p->P.tails_raw.size(), n_open, n, method);
+  // with memory short, the prefix sums of fewer groups at a time
+  while (int rc = lease.take(8 * tn::sample_scratch_doubles(n_open, groups))) {
+    if (rc != TN_ERR_OOM || groups <= 1) return rc;
+    groups = (groups + 1) / 2;
+  }
   tn::SampleParams sp;
   sp.H = h->H;
   sp.L = (int64_t)p->P.tails_raw.size();
@@ -1603,6 +1613,7 @@ static int sample_impl(tn_head_t* h, int64_t n, double target_fidelity, uint64_t
   sp.method = method;
   sp.param = param;
   sp.carry = (double*)lease.c.buf;
+  sp.carry_groups = groups;
   sp.rep = lease.c.rep;
   sp.plan_status = p->d_status;
   CUDA_TRY(tn::launch_sample(sp, st));

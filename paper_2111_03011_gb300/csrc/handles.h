@@ -92,10 +92,12 @@ int enqueue_slices(tn_plan_t* plan, tn_range r, double2* H, cudaStream_t stream,
 // the named fault is armed.  "alloc": device allocations of plans and heads
 // fail; "slice:S[:T]": the contraction fails before pass T (default 0) of
 // user slice S; "status": each plain contraction call sets the plan's device
-// status word, as a bounded wait that gave up would.
+// status word, as a bounded wait that gave up would; "scratch:B": scratch of more
+// than B bytes for one call cannot be had.
 bool fault_alloc();
 bool fault_slice(int64_t s, int64_t t);
 bool fault_status();
+size_t fault_scratch();   // B, or the largest number
 // Range checks and bookkeeping of tn_contract_slices.
 int check_slice_range(tn_plan_t* plan, tn_range r, tn_head_t* head);
 void mark_slices_done(tn_head_t* head, tn_range r);

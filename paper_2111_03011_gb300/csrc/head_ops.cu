@@ -322,6 +322,7 @@ __device__ __forceinline__ double warp_inclusive_scan(double v) {
 // tree over adjacent pairs, which a butterfly adds in the same pairs; eight
 // chunks go through one butterfly at a time (after its first three steps
 // a lane holds one chunk), 9 additions instead of 40, with the same bits.
+// H: from the first of the n_groups groups on.
 __global__ void __launch_bounds__(256) k_group_prefix(const double2* __restrict__ H, int h, int64_t n_groups,
                                                       double* __restrict__ carry) {
   constexpr int kPiece = 1024;                 // chunks per pass through shared memory
@@ -410,6 +411,18 @@ __device__ __forceinline__ uint64_t bitstring_of(const SampleParams& p, int64_t 
   return (p.tails[g] & ~p.open_mask) | ((uint64_t)hi << 32) | lo;
 }
 
+// Sample j of the launch and its group: sample i is drawn from group i mod L; with
+// a window of groups the launch takes those samples whose group is in it.
+__device__ __forceinline__ int64_t sample_of(const SampleParams& p, int64_t j, int64_t& g) {
+  if (p.win == 0) {
+    g = j % p.L;
+    return j;
+  }
+  const int64_t round = j / p.win;
+  g = p.g0 + (j - round * p.win);
+  return round * p.L + g;
+}
+
 __device__ __forceinline__ uint64_t uniform_string(const SampleParams& p, int64_t i, uint2 key) {
   const uint64_t full = p.n_qubits >= 64 ? ~0ULL : ((1ULL << p.n_qubits) - 1);
   const uint4 q = philox4x32_10(make_uint4((uint32_t)i, (uint32_t)((uint64_t)i >> 32), 1u, 0u), key);
@@ -427,15 +440,16 @@ __global__ void __launch_bounds__(256) k_sample_prefix(SampleParams p) {
   const int lane = threadIdx.x & 31;
   const int64_t l = 1LL << p.h, nch = (l + 31) >> 5;
   const uint2 key = make_uint2((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
-  for (int64_t i = warp; i < p.n; i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t g = i % p.L;
+  for (int64_t j = warp; j < p.m; j += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    int64_t g;
+    const int64_t i = sample_of(p, j, g);
     const uint4 r = philox4x32_10(make_uint4((uint32_t)i, (uint32_t)((uint64_t)i >> 32), 0u, 0u), key);
     if (p.mix > 0.0 && u53(r.x, r.y) < p.mix) {
       if (lane == 0) p.out[i] = uniform_string(p, i, key);
       continue;
     }
     const double u_pick = u53(r.z, r.w);
-    const double* __restrict__ cr = p.carry + g * (nch + 1);
+    const double* __restrict__ cr = p.carry + (g - p.g0) * (nch + 1);
     const double Z = cr[nch];
     int64_t mu;
     if (Z > 0.0) {
@@ -563,8 +577,9 @@ __global__ void __launch_bounds__(128) k_sample_chain(SampleParams p) {
   report_word(p.rep, p.plan_status);
   const int64_t l = 1LL << p.h, nch = (l + 31) >> 5;
   const uint2 key = make_uint2((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t g = i % p.L;
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p.m; j += (int64_t)gridDim.x * blockDim.x) {
+    int64_t g;
+    const int64_t i = sample_of(p, j, g);
     const uint32_t ilo = (uint32_t)i, ihi = (uint32_t)((uint64_t)i >> 32);
     if (p.mix > 0.0) {
       const uint4 r = philox4x32_10(make_uint4(ilo, ihi, 0u, 0u), key);
@@ -585,7 +600,7 @@ __global__ void __launch_bounds__(128) k_sample_chain(SampleParams p) {
         if (__dmul_rn(u, wc) < wp) { mu = prop; wc = wp; }
       }
     } else {
-      const double Z = p.carry[g * (nch + 1) + nch];
+      const double Z = p.carry[(g - p.g0) * (nch + 1) + nch];
       const double bound = __dmul_rn((double)p.param, Z);
       for (int64_t t = 0; t < 64 * p.param; ++t) {
         const uint4 q = philox4x32_10(make_uint4(ilo, ihi, 3u, (uint32_t)t), key);
@@ -604,26 +619,50 @@ __global__ void __launch_bounds__(128) k_sample_chain(SampleParams p) {
 // a group, or from 256 members up, its prefix sums are worked out first.
 static bool exact_by_prefix(int64_t L, int h, int64_t n) { return h >= 8 || (h >= 6 && n > 4 * L); }
 
-size_t sample_scratch_doubles(int64_t L, int h, int64_t n, int method) {
+size_t sample_scratch_doubles(int h, int64_t groups) { return (size_t)(groups * ((((1LL << h) + 31) >> 5) + 1)); }
+
+int64_t sample_groups(int64_t L, int h, int64_t n, int method, size_t max_bytes) {
   if (method == 1 || (method == 0 && !exact_by_prefix(L, h, n))) return 0;
-  const int64_t nch = ((1LL << h) + 31) >> 5;
-  return (size_t)(std::min(L, n) * (nch + 1));
+  const int64_t fit = (int64_t)std::min<size_t>(max_bytes / 8 / sample_scratch_doubles(h, 1), (size_t)1 << 62);
+  return std::max<int64_t>(1, std::min(std::min(L, n), fit));
 }
 
-cudaError_t launch_sample(const SampleParams& p, cudaStream_t s) {
-  if (p.n <= 0) return cudaSuccess;
-  if (sample_scratch_doubles(p.L, p.h, p.n, p.method) > 0) {
-    if (!p.carry) return cudaErrorInvalidValue;
-    const int64_t ng = std::min(p.L, p.n);
-    k_group_prefix<<<(unsigned)std::min<int64_t>(ng, (int64_t)kSMs * 8), 256, 0, s>>>(p.H, p.h, ng, p.carry);
-    const cudaError_t e = cudaGetLastError();
+static cudaError_t launch_sample_window(const SampleParams& p, cudaStream_t s);
+
+// Samples from wide groups need the prefix sums of their groups, 1/64 of the
+// head's size for groups from 32 members up.  Where the caller has scratch for
+// fewer groups, they are taken in windows, one after another in the same scratch.
+cudaError_t launch_sample(const SampleParams& q, cudaStream_t s) {
+  if (q.n <= 0) return cudaSuccess;
+  SampleParams p = q;
+  p.g0 = p.win = 0;
+  p.m = p.n;
+  const int64_t ng = sample_groups(p.L, p.h, p.n, p.method);   // groups drawn from, or 0: no scratch
+  if (ng == 0) return launch_sample_window(p, s);
+  if (!p.carry || p.carry_groups < 1) return cudaErrorInvalidValue;
+  for (int64_t g0 = 0; g0 < ng; g0 += p.carry_groups) {
+    const int64_t w = std::min(p.carry_groups, ng - g0);
+    const double2* first = p.H + (g0 << p.h);
+    k_group_prefix<<<(unsigned)std::min<int64_t>(w, (int64_t)kSMs * 8), 256, 0, s>>>(first, p.h, w, p.carry);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (w < ng) {
+      p.g0 = g0;
+      p.win = w;
+      p.m = p.n / p.L * w + std::max<int64_t>(0, std::min(p.n % p.L - g0, w));
+    }
+    e = launch_sample_window(p, s);
     if (e != cudaSuccess) return e;
   }
+  return cudaSuccess;
+}
+
+static cudaError_t launch_sample_window(const SampleParams& p, cudaStream_t s) {
   if (p.method != 0) {
-    const int64_t grid = std::min<int64_t>((p.n + 127) / 128, (int64_t)kSMs * 16);
+    const int64_t grid = std::min<int64_t>((p.m + 127) / 128, (int64_t)kSMs * 16);
     k_sample_chain<<<(unsigned)grid, 128, 0, s>>>(p);
   } else if (exact_by_prefix(p.L, p.h, p.n)) {
-    const int64_t grid = std::min<int64_t>((p.n * 32 + 255) / 256, (int64_t)kSMs * 16);
+    const int64_t grid = std::min<int64_t>((p.m * 32 + 255) / 256, (int64_t)kSMs * 16);
     k_sample_prefix<<<(unsigned)grid, 256, 0, s>>>(p);
   } else {
     // consecutive samples per warp once there are more samples than warps

@@ -199,11 +199,18 @@ struct SampleParams {
   uint64_t* out;
   int method;                 // 0 exact inverse CDF, 1 Metropolis chain, 2 frugal rejection
   int64_t param;              // chain length (1) or the bound M (2)
-  double* carry = nullptr;    // scratch of sample_scratch_doubles() doubles (prefix sums)
+  double* carry = nullptr;    // scratch (prefix sums) of carry_groups groups, sample_scratch_doubles() long
+  int64_t carry_groups = 0;
   HeadReport* rep = nullptr;  // may be null, as may plan_status
   const unsigned int* plan_status = nullptr;
+  // set by launch_sample: the samples of groups g0 .. g0 + win - 1, m of them (win 0: all n)
+  int64_t g0 = 0, win = 0, m = 0;
 };
-size_t sample_scratch_doubles(int64_t L, int h, int64_t n, int method);
+// Groups whose prefix sums a draw keeps at once: all that it draws from if their
+// scratch fits in max_bytes, fewer otherwise (taken in turn), at least one; 0 if
+// it needs none.
+int64_t sample_groups(int64_t L, int h, int64_t n, int method, size_t max_bytes = (size_t)-1);
+size_t sample_scratch_doubles(int h, int64_t groups);
 cudaError_t launch_sample(const SampleParams& p, cudaStream_t s);
 
 }  // namespace tn

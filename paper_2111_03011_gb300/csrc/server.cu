@@ -186,6 +186,10 @@ int enqueue_amplitudes(Slot& s, Circuit& c) {
   return TN_OK;
 }
 
+// Prefix sums of a sampling request in its slot's buffer: those of 8 GiB of head
+// at a time.  Eight slots keep them within the reserve that admission leaves free.
+constexpr size_t kSampleScratch = (size_t)128 << 20;
+
 // Enqueue one request's device work on its slot (the head is, or will be,
 // ready): an amplitude batch, or one sampling request.
 int enqueue_op(Slot& s, Request* q, Circuit& c) {
@@ -194,7 +198,10 @@ int enqueue_op(Slot& s, Request* q, Circuit& c) {
   tn_plan_t* p = c.plan;
   const int h = (int)p->P.open_qubits.size();
   const size_t n = (size_t)r.n;
-  const size_t scratch = 8 * tn::sample_scratch_doubles((int64_t)p->P.tails_raw.size(), h, r.n, r.method);
+  const int64_t L = (int64_t)p->P.tails_raw.size();
+  const int64_t groups =
+      tn::sample_groups(L, h, r.n, r.method, std::min<size_t>(kSampleScratch, tn::fault_scratch()));
+  const size_t scratch = 8 * tn::sample_scratch_doubles(h, groups);
   if (ensure_slot_buffers(s, std::max<size_t>(n * 8 + scratch, 256), std::max<size_t>(n * 8, 256)))
     return fail(TN_ERR_OOM, "server: slot staging allocation failed");
   cudaStream_t st = s.stream;
@@ -206,7 +213,7 @@ int enqueue_op(Slot& s, Request* q, Circuit& c) {
   if (r.target_fidelity > 0.0 && f_head > 0.0 && r.target_fidelity < f_head) mix = 1.0 - r.target_fidelity / f_head;
   tn::SampleParams sp;
   sp.H = c.head->H;
-  sp.L = (int64_t)p->P.tails_raw.size();
+  sp.L = L;
   sp.h = h;
   sp.tails = p->d_tails;
   sp.open_mask = p->P.open_mask;
@@ -220,6 +227,7 @@ int enqueue_op(Slot& s, Request* q, Circuit& c) {
   sp.param = r.param != 0 ? r.param
                           : (r.method == TN_SAMPLE_METROPOLIS ? ((int64_t)1 << h) : (r.method == TN_SAMPLE_FRUGAL ? 10 : 0));
   sp.carry = scratch ? (double*)d + n : nullptr;
+  sp.carry_groups = groups;
   cudaError_t e = tn::launch_sample(sp, st);
   if (e != cudaSuccess) return fail(TN_ERR_CUDA, std::string("server: sample: ") + cudaGetErrorString(e));
   if (cudaMemcpyAsync(s.h_buf, d, n * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
