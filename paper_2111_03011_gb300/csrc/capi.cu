@@ -286,6 +286,13 @@ static int plan_upload(tn_plan_t* p) {
     CUDA_TRY(cudaMemcpy(p->d_meta, P.meta.data(), P.meta.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
   if (P.workspace_bytes > 0) {
     cudaError_t e = tn::device_malloc((void**)&p->d_arena, (size_t)P.workspace_bytes);
+    if (e == cudaErrorMemoryAllocation && P.batch_max > 1) {
+      // without the copies of the batched steps (up to 64 MB): every pass runs its whole launch list
+      cudaGetLastError();
+      P.workspace_bytes -= (P.batch_max - 1) * P.batch_stride;
+      P.batch_max = 1;
+      e = tn::device_malloc((void**)&p->d_arena, (size_t)P.workspace_bytes);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(TN_ERR_OOM, "workspace of " + std::to_string(P.workspace_bytes) + " bytes: " + cudaGetErrorString(e));
