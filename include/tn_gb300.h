@@ -426,15 +426,16 @@ int  tn_head_norm_noalloc(const void* head_c128, int64_t n_groups, int n_open, d
  * M, N and K are powers of two (K >= 2 on the tensor-core engines; 16-bit
  * engines take K = 2 in tf32, as the planner does).  mapA / mapB are host
  * arrays of PC pattern indices, or NULL for the identity (P = PC) or pattern 0
- * (P = 1).  The operands pass through the same kernels as a plan's steps
- * (engine TN_GEMM_*): split permute, B preparation and GEMM, or, with pair = 0
- * and a tensor-core engine, the direct kernel (FP32 products; BF16x3 ones for
- * that engine) where it is modelled faster (small or narrow shapes).  pair = -1: one-CTA GEMM tiles,
- * pair > 0: the GEMM kernels with CTA pairs where they apply.  Its
- * scratch (split planes, prepared B, maps) comes from a bounded pool that the
- * library keeps between calls (at most 2 GiB, given back when an allocation of
- * the library fails or its server needs room); it synchronises `stream`.  TN_ERR_TIMEOUT if a bounded device
- * wait gave up. */
+ * (P = 1).  On the tensor-core engines (TN_GEMM_*) the operands are split and
+ * embedded by a preparation launch of their own and multiplied by the GEMM of a
+ * plan's steps, or, with pair = 0, the product is the direct kernel's (FP32
+ * products; BF16x3 ones for that engine) where it is modelled faster (small or
+ * narrow shapes) and C lies apart from A and B.  pair = -1: one-CTA GEMM tiles,
+ * pair > 0: the GEMM kernels with CTA pairs where they apply.  Its scratch
+ * (split planes, prepared B, maps) comes from a bounded pool that the library
+ * keeps between calls (at most 2 GiB, given back when an allocation of the
+ * library fails or its server needs room); it synchronises `stream`.
+ * TN_ERR_TIMEOUT if a bounded device wait gave up. */
 int  tn_gemm_c64(int engine, const void* A, const void* B, void* C, int64_t M, int64_t N, int64_t K,
                  int64_t PA, int64_t PB, int64_t PC, const int32_t* mapA, const int32_t* mapB, int pair,
                  void* stream);
